@@ -14,11 +14,44 @@
 
 namespace sabr {
 
-constexpr int kClqBlock = 128;
+constexpr int kClqBlock = 64;
+
+// Sum over the block, the same in every run: butterflies within the warps,
+// then the warps' sums in order by thread 0 (which returns the total).
+__device__ __forceinline__ double clq_block_sum(double v, double* row) {
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  if ((threadIdx.x & 31) == 0) row[threadIdx.x >> 5] = v;
+  __syncthreads();
+  double t = 0.0;
+  if (threadIdx.x == 0)
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += row[w];
+  return t;
+}
+
+// Paths per thread.
+template <class R> constexpr int kClqPaths = sizeof(R) == 4 ? 4 : kMcPathsPerThread;
+
+// What one path pays: the returns between resets, clipped and added.
+template <class R> struct ClqPath {
+  R prev, sum;
+  // F at reset `reset`: R_i = F(d_i)/F(d_{i-1}) - 1; a path absorbed before
+  // d_{i-1} adds R_i = 0 (0 to 0)
+  __device__ __forceinline__ void land(int reset, R F, R fl, R cl) {
+    if (reset >= 1) {
+      const R ret = prev > (R)0 ? F / prev - (R)1 : (R)0;
+      const R c = ret < cl ? ret : cl;
+      sum += c > fl ? c : fl;
+    }
+    prev = F;
+  }
+};
 
 // Grid-stride over paths: thread t of the grid prices paths t, t + stride,
 // ... and keeps FP64 sums of the payoff and its square; each block adds its
-// threads' sums in thread order into partial[2 b], partial[2 b + 1].
+// threads' sums in a fixed order into partial[2 b], partial[2 b + 1].  FP32
+// paths advance in two pairs a thread with the packed FP32x2 instructions
+// (run_path_pairs), FP64 paths kMcPathsPerThread at a time.
 template <class R>
 __global__ void __launch_bounds__(kClqBlock) cliquet_kernel(McDev P, const double* __restrict__ params,
                                                            double floor_l, double cap_l, double floor_g,
@@ -26,66 +59,63 @@ __global__ void __launch_bounds__(kClqBlock) cliquet_kernel(McDev P, const doubl
   extern __shared__ __align__(16) unsigned char smem[];
   StepCoef<R>* tab = (StepCoef<R>*)smem;
   int* land = (int*)(tab + P.n_steps);  // land[r] = the step ending at reset r
-  __shared__ double red[2][kClqBlock];
+  __shared__ double red[2][kClqBlock / 32];
   double p[kMaxD];
 #pragma unroll
   for (int i = 0; i < kMaxD; ++i) p[i] = params[i];
-  build_steps<R>(P, p, tab, land);
+  build_steps<R>(P, p, 0, tab, land);
   __syncthreads();
   const R beta_m1 = (R)(p[1] - 1.0);
   const R lnf = (R)PathUnits<R>::logu(P.fwd), lna = (R)PathUnits<R>::logu(p[0]);
   const R log_abs = (R)(P.log_absorb * PathUnits<R>::kLogUnit);
   const R fl = (R)floor_l, cl = (R)cap_l;
   double s1 = 0.0, s2 = 0.0;
-  // kMcPathsPerThread paths per thread (path, path + stride, ...) advance
-  // together
-  constexpr int NPT = kMcPathsPerThread;
+  constexpr int NPT = kClqPaths<R>;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t p0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p0 < P.n_paths; p0 += NPT * stride) {
-    int64_t path[NPT];
-    PathState<R> st[NPT];
-    R prev[NPT], sum[NPT];
+    ClqPath<R> pay[NPT];
 #pragma unroll
-    for (int k = 0; k < NPT; ++k) {
-      path[k] = p0 + k * stride;
-      st[k] = PathState<R>{lnf, lna, false};
-      prev[k] = (R)0;
-      sum[k] = (R)0;
-    }
-    int reset = 0, i_land = land[0];
-    auto at_reset = [&]() {
+    for (int k = 0; k < NPT; ++k) pay[k] = ClqPath<R>{(R)0, (R)0};
+    int reset = 0;
+    if constexpr (sizeof(R) == 4) {
+      PathPairs<2> st;
+      st.start(P, lnf, lna, p0, stride);
+      run_path_pairs<2, kOrderCliquet>(P, tab, beta_m1, st, land[0], [&]() {
 #pragma unroll
-      for (int k = 0; k < NPT; ++k) {
-        const R F = st[k].absorbed ? (R)0 : PathUnits<R>::expu(st[k].lnF);
-        if (reset >= 1) {
-          // R_i = F(d_i)/F(d_{i-1}) - 1; a path absorbed before d_{i-1}
-          // adds R_i = 0 (0 to 0)
-          const R ret = prev[k] > (R)0 ? F / prev[k] - (R)1 : (R)0;
-          const R c = ret < cl ? ret : cl;
-          sum[k] += c > fl ? c : fl;
+        for (int k = 0; k < 4; ++k) pay[k].land(reset, st.forward(k, log_abs), fl, cl);
+        ++reset;
+        return reset < P.n_mats ? land[reset] : -1;
+      });
+    } else {
+      PathState<R> st[NPT];
+#pragma unroll
+      for (int k = 0; k < NPT; ++k) st[k] = PathState<R>{lnf, lna, false};
+      int i_land = land[0];
+      auto at_reset = [&]() {
+#pragma unroll
+        for (int k = 0; k < NPT; ++k)
+          pay[k].land(reset, st[k].absorbed ? (R)0 : PathUnits<R>::expu(st[k].lnF), fl, cl);
+        ++reset;
+        i_land = reset < P.n_mats ? land[reset] : -1;
+      };
+      for (int i = 0; i < P.n_steps; i += 2) {
+        uint4 w[NPT];
+#pragma unroll
+        for (int k = 0; k < NPT; ++k) w[k] = path_words(P, p0 + k * stride, i);
+#pragma unroll
+        for (int k = 0; k < NPT; ++k) path_step<R>(tab[i], w[k].x, w[k].y, beta_m1, log_abs, st[k]);
+        if (i == i_land) at_reset();
+        if (i + 1 < P.n_steps) {
+#pragma unroll
+          for (int k = 0; k < NPT; ++k) path_step<R>(tab[i + 1], w[k].z, w[k].w, beta_m1, log_abs, st[k]);
+          if (i + 1 == i_land) at_reset();
         }
-        prev[k] = F;
-      }
-      ++reset;
-      i_land = reset < P.n_mats ? land[reset] : -1;
-    };
-    for (int i = 0; i < P.n_steps; i += 2) {
-      uint4 w[NPT];
-#pragma unroll
-      for (int k = 0; k < NPT; ++k) w[k] = path_words<R>(P, path[k], i);
-#pragma unroll
-      for (int k = 0; k < NPT; ++k) path_step<R>(tab[i], w[k].x, w[k].y, beta_m1, log_abs, st[k]);
-      if (i == i_land) at_reset();
-      if (i + 1 < P.n_steps) {
-#pragma unroll
-        for (int k = 0; k < NPT; ++k) path_step<R>(tab[i + 1], w[k].z, w[k].w, beta_m1, log_abs, st[k]);
-        if (i + 1 == i_land) at_reset();
       }
     }
 #pragma unroll
     for (int k = 0; k < NPT; ++k) {
-      if (path[k] < P.n_paths) {
-        double g = (double)sum[k];
+      if (p0 + k * stride < P.n_paths) {
+        double g = (double)pay[k].sum;
         g = g < cap_g ? g : cap_g;
         g = g > floor_g ? g : floor_g;
         s1 += g;
@@ -93,29 +123,27 @@ __global__ void __launch_bounds__(kClqBlock) cliquet_kernel(McDev P, const doubl
       }
     }
   }
-  red[0][threadIdx.x] = s1;
-  red[1][threadIdx.x] = s2;
-  __syncthreads();
+  const double a = clq_block_sum(s1, red[0]), b = clq_block_sum(s2, red[1]);
   if (threadIdx.x == 0) {
-    double a = 0.0, b = 0.0;
-    for (int t = 0; t < (int)blockDim.x; ++t) {
-      a += red[0][t];
-      b += red[1][t];
-    }
     partial[2 * blockIdx.x] = a;
     partial[2 * blockIdx.x + 1] = b;
   }
 }
 
-// Block sums in block order -> discounted mean and its standard error.
-__global__ void cliquet_reduce_kernel(const double* __restrict__ partial, int blocks, int64_t n_paths, double disc,
-                                      double* __restrict__ price, double* __restrict__ se) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double s = 0.0, s2 = 0.0;
-  for (int b = 0; b < blocks; ++b) {
-    s += partial[2 * b];
-    s2 += partial[2 * b + 1];
+// Block sums, by one block in a fixed order -> discounted mean and its
+// standard error.
+__global__ void __launch_bounds__(kClqBlock) cliquet_reduce_kernel(const double* __restrict__ partial, int blocks,
+                                                                  int64_t n_paths, double disc,
+                                                                  double* __restrict__ price,
+                                                                  double* __restrict__ se) {
+  __shared__ double red[2][kClqBlock / 32];
+  double v = 0.0, v2 = 0.0;
+  for (int b = threadIdx.x; b < blocks; b += blockDim.x) {
+    v += partial[2 * b];
+    v2 += partial[2 * b + 1];
   }
+  const double s = clq_block_sum(v, red[0]), s2 = clq_block_sum(v2, red[1]);
+  if (threadIdx.x != 0) return;
   const double N = (double)n_paths, mean = s / N;
   double var = (s2 - s * mean) / (N - 1.0);
   if (var < 0.0) var = 0.0;
@@ -149,8 +177,11 @@ extern "C" sabr_status sabr_mc_cliquet(sabr_model model, const double* params, d
   const size_t smem = (size_t)h.n_steps * (prec == SABR_FP64 ? sizeof(StepCoef<double>) : sizeof(StepCoef<float>)) +
                       (size_t)n_resets * sizeof(int);
   if (smem > 200 * 1024) return fail(SABR_EINVAL, "too many time steps for one launch");
-  // resident blocks of the GPU (grid-stride; no partly filled second wave),
-  // and no more than the paths need at kMcPathsPerThread paths per thread
+  // The grid: as many rounds of resident threads as the paths need, then
+  // only the blocks that fill these rounds evenly -- 2^20 paths are 2.2
+  // rounds of the 152 x 768 threads that fit, and three rounds of 576 threads
+  // an SM end together where the third of 768 would leave most SMs idle.
+  // Small blocks keep the SMs' shares equal.
   int per_sm = 8;
   if (prec == SABR_FP64) {
     cudaFuncSetAttribute(cliquet_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -159,13 +190,17 @@ extern "C" sabr_status sabr_mc_cliquet(sabr_model model, const double* params, d
     cudaFuncSetAttribute(cliquet_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cliquet_kernel<float>, kClqBlock, smem);
   }
-  per_sm = std::min(std::max(per_sm, 1), 8);
-  const int64_t per_block = (int64_t)kClqBlock * kMcPathsPerThread;
-  const int blocks = (int)std::min<int64_t>(device_sms() * (int64_t)per_sm, (n_paths + per_block - 1) / per_block);
+  per_sm = std::max(per_sm, 1);
+  const int64_t per_block = (int64_t)kClqBlock * mc_paths_per_thread(prec);
+  const int64_t units = (n_paths + per_block - 1) / per_block, resident = device_sms() * (int64_t)per_sm;
+  const int64_t rounds = (units + resident - 1) / resident;
+  const int blocks = (int)((units + rounds - 1) / rounds);
   const size_t img = mc_image_bytes(h);
   const size_t params_off = (img + 255) & ~(size_t)255;
   const size_t part_off = params_off + 256;
-  const size_t bytes = part_off + sizeof(double) * 2 * blocks;
+  const size_t tab_off = (part_off + sizeof(double) * 2 * blocks + 255) & ~(size_t)255;
+  const size_t tab_bytes = mc_step_table_bytes(h, 1);
+  const size_t bytes = tab_off + tab_bytes;
   cudaStream_t s = (cudaStream_t)stream;
   unsigned char* dev = nullptr;
   SABR_CUDA(cudaMallocAsync((void**)&dev, bytes, s));
@@ -174,6 +209,7 @@ extern "C" sabr_status sabr_mc_cliquet(sabr_model model, const double* params, d
   int *q_value, *q_out;
   double* disc;
   mc_fill_image(h, host.data(), dev, d, &q_value, &q_out, &disc);
+  if (tab_bytes) d.tab = dev + tab_off;
   double p10[kMaxD];
   for (int i = 0; i < kMaxD; ++i) p10[i] = i < n_params(model) ? params[i] : 0.0;
   std::memcpy(host.data() + params_off, p10, sizeof(p10));
@@ -185,6 +221,7 @@ extern "C" sabr_status sabr_mc_cliquet(sabr_model model, const double* params, d
   }
   double* part = (double*)(dev + part_off);
   const double* dp = (const double*)(dev + params_off);
+  if (tab_bytes) mc_launch_steps(h, d, dp, nullptr, 1, s);
   if (prec == SABR_FP64) {
     e = cudaFuncSetAttribute(cliquet_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess)
@@ -197,7 +234,7 @@ extern "C" sabr_status sabr_mc_cliquet(sabr_model model, const double* params, d
                                                            cap_global, part);
   }
   if (e == cudaSuccess) {
-    cliquet_reduce_kernel<<<1, 32, 0, s>>>(part, blocks, n_paths, discount, price_out, stderr_out);
+    cliquet_reduce_kernel<<<1, kClqBlock, 0, s>>>(part, blocks, n_paths, discount, price_out, stderr_out);
     e = cudaGetLastError();
   }
   cudaFreeAsync(dev, s);

@@ -16,11 +16,16 @@ namespace sabr {
 // Kernels
 // ---------------------------------------------------------------------------
 struct McSmem {
-  size_t tab, land, q0, nq, slot, K, call, wacc, total;
+  size_t tab, land, q0, nq, slot, K, call, wacc, fx, total;
 };
 
+// FP32 log-Euler options are stored as McOption (8 bytes, no call flag);
+// split: the block of 2 kMcBlock threads also needs the exchange buffer of
+// simulate_paths_f32<1>.
 template <class R>
-__host__ __device__ inline McSmem mc_smem_layout(int n_steps, int n_quotes, int n_mats, int n_slots) {
+__host__ __device__ inline McSmem mc_smem_layout(int n_steps, int n_quotes, int n_mats, int n_slots, bool split) {
+  // (the conditional-Bessel form leaves its step table in global memory and
+  // passes n_steps = 0)
   McSmem L;
   size_t o = 0;
   auto take = [&](size_t bytes) {
@@ -30,14 +35,24 @@ __host__ __device__ inline McSmem mc_smem_layout(int n_steps, int n_quotes, int 
   };
   L.wacc = take(sizeof(double) * kMcWarps * n_slots * 32);
   L.tab = take(sizeof(StepCoef<R>) * n_steps);
-  L.K = take(sizeof(R) * n_quotes);
+  L.K = take(8 * n_quotes);
   L.land = take(sizeof(int) * n_mats);
   L.q0 = take(sizeof(int) * n_mats);
   L.nq = take(sizeof(int) * n_mats);
   L.slot = take(sizeof(int) * n_mats);
   L.call = take(n_quotes);
+  L.fx = take(split ? sizeof(float) * 2 * 4 * kMcBlock : 0);
   L.total = (o + 15) & ~(size_t)15;
   return L;
+}
+// Bytes of a block's tables and accumulators by which problems are refused
+// and grids are sized: strikes at the working precision, as the scalar paths
+// keep them (within 6 KB of what any form of the kernel takes).
+static size_t mc_table_bytes(int prec, int n_steps, int n_quotes, int n_mats, int n_slots) {
+  auto up = [](size_t x) { return (x + 15) & ~(size_t)15; };
+  const size_t rs = prec == SABR_FP64 ? 8 : 4;
+  return up(sizeof(double) * kMcWarps * n_slots * 32) + up(4 * rs * n_steps) + up(rs * n_quotes) +
+         4 * up(sizeof(int) * n_mats) + up(n_quotes);
 }
 
 // grid = (blocks_per_set, n_sets).  Set s prices with set_params[s][0..9];
@@ -49,19 +64,28 @@ __host__ __device__ inline McSmem mc_smem_layout(int n_steps, int n_quotes, int 
 // the paths it would take in that grid -- and writes their partials at
 // positions 0 .. gridDim.x - 1; grid_total = 0 means the launch is the
 // whole grid.  SCHEME: SABR_MC_LOG_EULER (eq. (dis_SABRd)) or
-// SABR_MC_BESSEL (the conditional-Bessel step of mc_bessel.cuh).
-template <class R, int SCHEME>
-__global__ void __launch_bounds__(kMcBlock) mc_paths_kernel(McDev P, const double* __restrict__ set_params,
-                                                           const int* __restrict__ set_valid,
-                                                           double* __restrict__ partial, int block0,
-                                                           int grid_total) {
+// SABR_MC_BESSEL (the conditional-Bessel step of mc_bessel.cuh).  SPLIT
+// (FP32 log-Euler): blocks of 2 kMcBlock threads, a pair of paths each.
+// Resident blocks of kMcBlock threads per SM that the grids count on (and the
+// kernels' register budgets are set for).
+__host__ __device__ constexpr int mc_resident_blocks(int prec, int scheme) {
+  return prec == SABR_FP64 ? 3 : (scheme == SABR_MC_BESSEL ? 5 : 4);
+}
+template <class R, int SCHEME, bool SPLIT>
+__global__ void __launch_bounds__((SPLIT ? 2 * kMcBlock : kMcBlock),
+                                  (SPLIT ? 1 : mc_resident_blocks(sizeof(R) == 8 ? SABR_FP64 : SABR_FP32, SCHEME)))
+    mc_paths_kernel(McDev P, const double* __restrict__ set_params, const int* __restrict__ set_valid,
+                    double* __restrict__ partial, int block0, int grid_total) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int set = blockIdx.y;
   if (set_valid && !set_valid[set]) return;
-  const McSmem L = mc_smem_layout<R>(P.n_steps, P.n_quotes, P.n_mats, P.n_slots);
+  constexpr bool kPairs = sizeof(R) == 4 && SCHEME == SABR_MC_LOG_EULER;
+  const McSmem L =
+      mc_smem_layout<R>(SCHEME == SABR_MC_BESSEL ? 0 : P.n_steps, P.n_quotes, P.n_mats, P.n_slots, SPLIT);
   double* wacc = (double*)(smem + L.wacc);
   StepCoef<R>* tab = (StepCoef<R>*)(smem + L.tab);
   R* sK = (R*)(smem + L.K);
+  McOption* sopt = (McOption*)(smem + L.K);
   int* land = (int*)(smem + L.land);
   int* s_q0 = (int*)(smem + L.q0);
   int* s_nq = (int*)(smem + L.nq);
@@ -73,13 +97,21 @@ __global__ void __launch_bounds__(kMcBlock) mc_paths_kernel(McDev P, const doubl
   const int nv = P.n_slots * 32;
   for (int i = threadIdx.x; i < kMcWarps * nv; i += blockDim.x) wacc[i] = 0.0;
   if constexpr (SCHEME == SABR_MC_BESSEL) {
-    build_steps_bessel<R>(P, p, (StepCoefB<R>*)tab, land);
+    for (int i = threadIdx.x; i < P.n_steps; i += blockDim.x) {
+      const int m = P.step_mat[i];
+      if (m >= 0) land[m] = i;
+    }
   } else {
-    build_steps<R>(P, p, tab, land);
+    build_steps<R>(P, p, set, tab, land);
   }
   for (int q = threadIdx.x; q < P.n_quotes; q += blockDim.x) {
-    sK[q] = (R)P.K[q];
-    scall[q] = P.is_call[q];
+    if constexpr (kPairs) {
+      const float K = (float)P.K[q];
+      sopt[q] = P.is_call[q] != 0 ? McOption{1.0f, -K} : McOption{-1.0f, K};
+    } else {
+      sK[q] = (R)P.K[q];
+      scall[q] = P.is_call[q];
+    }
   }
   for (int m = threadIdx.x; m < P.n_mats; m += blockDim.x) {
     s_q0[m] = P.mat_q0[m];
@@ -87,21 +119,22 @@ __global__ void __launch_bounds__(kMcBlock) mc_paths_kernel(McDev P, const doubl
     s_slot[m] = P.mat_slot[m];
   }
   __syncthreads();
-  const int warp = threadIdx.x >> 5;
+  const int vt = threadIdx.x & (kMcBlock - 1);  // virtual thread of the block
   const int64_t gblocks = grid_total > 0 ? grid_total : gridDim.x;
-  const int64_t path0 = (int64_t)(block0 + blockIdx.x) * blockDim.x + threadIdx.x;
-  double* my_acc = wacc + (size_t)warp * nv;
+  const int64_t path0 = (int64_t)(block0 + blockIdx.x) * kMcBlock + vt, pstride = gblocks * kMcBlock;
+  double* my_acc = wacc + (size_t)(vt >> 5) * nv;
   if constexpr (SCHEME == SABR_MC_BESSEL) {
-    const StepCoefB<R>* tb = (const StepCoefB<R>*)tab;
+    const BesselStep<R>* tb = (const BesselStep<R>*)P.tab;
     if (p[1] == 1.0) {
-      simulate_paths_bessel<R, true>(P, p, tb, land, s_q0, s_nq, s_slot, sK, scall, path0, gblocks * blockDim.x,
-                                     my_acc);
+      simulate_paths_bessel<R, true>(P, p, tb, land, s_q0, s_nq, s_slot, sK, scall, path0, pstride, my_acc);
     } else {
-      simulate_paths_bessel<R, false>(P, p, tb, land, s_q0, s_nq, s_slot, sK, scall, path0, gblocks * blockDim.x,
-                                      my_acc);
+      simulate_paths_bessel<R, false>(P, p, tb, land, s_q0, s_nq, s_slot, sK, scall, path0, pstride, my_acc);
     }
+  } else if constexpr (kPairs) {
+    simulate_paths_f32<SPLIT ? 1 : 2>(P, p, tab, land, s_q0, s_nq, s_slot, sopt, path0, pstride, my_acc,
+                                      (float*)(smem + L.fx));
   } else {
-    simulate_paths<R>(P, p, tab, land, s_q0, s_nq, s_slot, sK, scall, path0, gblocks * blockDim.x, my_acc);
+    simulate_paths_scalar<R>(P, p, tab, land, s_q0, s_nq, s_slot, sK, scall, path0, pstride, my_acc);
   }
   __syncthreads();
   double* out = partial + ((size_t)set * gridDim.x + blockIdx.x) * nv;
@@ -113,23 +146,53 @@ __global__ void __launch_bounds__(kMcBlock) mc_paths_kernel(McDev P, const doubl
   }
 }
 
-// One thread per (set, option): fixed-order sum over blocks, eq. (payoff).
-__global__ void mc_reduce_kernel(McDev P, int n_sets, int blocks_per_set, const double* __restrict__ partial,
+// The step tables of n_sets parameter sets (blockIdx.y), one thread per step:
+// StepCoef entries of a dynamic model, or BesselStep entries.
+template <class R, int SCHEME>
+__global__ void __launch_bounds__(64) mc_steps_kernel(McDev P, const double* __restrict__ set_params,
+                                                     const int* __restrict__ set_valid, void* __restrict__ out) {
+  const int set = blockIdx.y, i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= P.n_steps || (set_valid && !set_valid[set])) return;
+  double p[kMaxD];
+#pragma unroll
+  for (int k = 0; k < kMaxD; ++k) p[k] = set_params[(size_t)set * kMaxD + k];
+  const size_t at = (size_t)set * P.n_steps + i;
+  if constexpr (SCHEME == SABR_MC_BESSEL) {
+    ((BesselStep<R>*)out)[at] = bessel_step_entry<R>(P, p, i);
+  } else {
+    ((StepCoef<R>*)out)[at] = dynamic_step_coef<R>(P, p, i);
+  }
+}
+
+// L lanes per (set, option), L a power of two: lane l sums blocks l, l + L,
+// ... and a fixed butterfly sums the lanes, eq. (payoff).  One lane over the
+// 608 blocks of a whole-GPU launch is a chain of 608 dependent loads and FP64
+// additions, which took longer than the paths of a small pricing.
+__global__ void mc_reduce_kernel(McDev P, int n_sets, int blocks_per_set, int L, const double* __restrict__ partial,
                                  const int* __restrict__ q_value, const int* __restrict__ q_out,
                                  const double* __restrict__ disc, const int* __restrict__ set_valid,
                                  double* __restrict__ price, double* __restrict__ se, int out_stride) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n_sets * P.n_quotes) return;
-  const int set = idx / P.n_quotes, q = idx % P.n_quotes;
+  const int64_t idx = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / L;
+  const int lane = threadIdx.x & (L - 1);
+  // (blockDim is a multiple of L: the lanes of an option leave together)
+  if (idx >= (int64_t)n_sets * P.n_quotes) return;
+  const int set = (int)(idx / P.n_quotes), q = (int)(idx % P.n_quotes);
   if (set_valid && !set_valid[set]) return;
   const int nv = P.n_slots * 32;
   const int v = q_value[q];
   double s = 0.0, s2 = 0.0;
-  for (int b = 0; b < blocks_per_set; ++b) {
-    const double* part = partial + ((size_t)set * blocks_per_set + b) * nv;
-    s += part[v];
-    s2 += part[v + 1];
+#pragma unroll 4
+  for (int b = lane; b < blocks_per_set; b += L) {
+    const double* part = partial + ((size_t)set * blocks_per_set + b) * nv + v;
+    s += part[0];
+    s2 += part[1];
   }
+  const unsigned mask = L == 32 ? 0xffffffffu : (((1u << L) - 1u) << ((threadIdx.x & 31) & ~(L - 1)));
+  for (int off = L >> 1; off > 0; off >>= 1) {
+    s += __shfl_xor_sync(mask, s, off);
+    s2 += __shfl_xor_sync(mask, s2, off);
+  }
+  if (lane != 0) return;
   const double N = (double)P.n_paths;
   const double mean = s / N;
   double var = (s2 - s * mean) / (N - 1.0);
@@ -137,6 +200,21 @@ __global__ void mc_reduce_kernel(McDev P, int n_sets, int blocks_per_set, const 
   const double D = disc[q];
   price[(size_t)set * out_stride + q_out[q]] = D * mean;
   if (se) se[(size_t)set * out_stride + q_out[q]] = D * sqrt(var / N);
+}
+// Lanes per option: about eight blocks a lane (a function of the grid alone,
+// so a path-sharded reduction runs in the order of the unsharded one).
+static int mc_reduce_lanes(int blocks_per_set) {
+  int L = 1;
+  while (L < 32 && 8 * L < blocks_per_set) L <<= 1;
+  return L;
+}
+static void launch_reduce(const McDev& d, int n_sets, int blocks_per_set, const double* partial, const int* q_value,
+                          const int* q_out, const double* disc, const int* set_valid, double* price, double* se,
+                          int out_stride, cudaStream_t s) {
+  const int L = mc_reduce_lanes(blocks_per_set);
+  const int64_t threads = (int64_t)n_sets * d.n_quotes * L;
+  mc_reduce_kernel<<<(unsigned)((threads + 127) / 128), 128, 0, s>>>(d, n_sets, blocks_per_set, L, partial, q_value,
+                                                                     q_out, disc, set_valid, price, se, out_stride);
 }
 
 // ---------------------------------------------------------------------------
@@ -222,9 +300,7 @@ sabr_status mc_prepare(int model, double fwd, const double* T, const double* K, 
   h.n_steps = (int)h.step_t.size();
   if (h.n_steps > kMaxMcSteps) return fail(SABR_EINVAL, "more than 8192 time steps");
   h.Tmax = h.mats.back();
-  const size_t smem = prec == SABR_FP64
-                          ? mc_smem_layout<double>(h.n_steps, h.n_quotes, (int)h.mats.size(), h.n_slots).total
-                          : mc_smem_layout<float>(h.n_steps, h.n_quotes, (int)h.mats.size(), h.n_slots).total;
+  const size_t smem = mc_table_bytes(prec, h.n_steps, h.n_quotes, (int)h.mats.size(), h.n_slots);
   if (smem > 220 * 1024) return fail(SABR_EINVAL, "too many time steps and options for one launch");
   h.smem = smem;
   return SABR_OK;
@@ -260,7 +336,14 @@ void mc_fill_image(const McHost& h, unsigned char* host_img, unsigned char* dev_
     d.rk.k0[r] = d.key0 + (uint32_t)r * 0x9E3779B9u;
     d.rk.k1[r] = d.key1 + (uint32_t)r * 0xBB67AE85u;
   }
-  d.step_t = (const double*)put(h.step_t.data(), 8 * h.step_t.size());
+  d.tab = nullptr;
+  if (h.model == SABR_DYN_I || h.model == SABR_DYN_II) {
+    d.step_t = (const double*)put(h.step_t.data(), 8 * h.step_t.size());
+  } else {
+    std::vector<double> sh(h.step_h.size());
+    for (size_t i = 0; i < sh.size(); ++i) sh[i] = std::sqrt(h.step_h[i]);
+    d.step_t = (const double*)put(sh.data(), 8 * sh.size());
+  }
   d.step_h = (const double*)put(h.step_h.data(), 8 * h.step_h.size());
   d.step_mat = (const int*)put(h.step_mat.data(), 4 * h.step_mat.size());
   d.mat_q0 = (const int*)put(h.mat_q0.data(), 4 * h.mat_q0.size());
@@ -273,24 +356,51 @@ void mc_fill_image(const McHost& h, unsigned char* host_img, unsigned char* dev_
   *disc = (double*)put(h.disc.data(), 8 * h.disc.size());
 }
 
+// Bytes of the step tables of n_sets sets: 0 where the blocks build their own
+// (static log-Euler models, whose entries cost less than a launch).
+size_t mc_step_table_bytes(const McHost& h, int n_sets) {
+  const size_t rs = h.prec == SABR_FP64 ? 8 : 4;
+  if (h.scheme == SABR_MC_BESSEL) return 12 * rs * (size_t)h.n_steps * n_sets;
+  if (h.model != SABR_DYN_I && h.model != SABR_DYN_II) return 0;
+  return 4 * rs * (size_t)h.n_steps * n_sets;
+}
+static_assert(sizeof(BesselStep<float>) == 48 && sizeof(BesselStep<double>) == 96, "step table entry");
+
 using McPathsFn = void (*)(McDev, const double*, const int*, double*, int, int);
 
-// The path kernel of a problem's precision and scheme, with its dynamic
-// shared memory allowance raised to what the problem needs.
-static McPathsFn mc_paths_fn(const McHost& h) {
+// The path kernel of a problem's precision and scheme (split: the FP32
+// log-Euler form with a pair of paths a thread), with its dynamic shared
+// memory allowance raised to what the problem needs.
+static McPathsFn mc_paths_fn(const McHost& h, bool split, size_t* smem) {
   McPathsFn fn;
+  const int M = (int)h.mats.size(), S = h.scheme == SABR_MC_BESSEL ? 0 : h.n_steps;
   if (h.prec == SABR_FP64) {
-    fn = h.scheme == SABR_MC_BESSEL ? mc_paths_kernel<double, SABR_MC_BESSEL> : mc_paths_kernel<double, SABR_MC_LOG_EULER>;
+    fn = h.scheme == SABR_MC_BESSEL ? mc_paths_kernel<double, SABR_MC_BESSEL, false>
+                                    : mc_paths_kernel<double, SABR_MC_LOG_EULER, false>;
+    *smem = mc_smem_layout<double>(S, h.n_quotes, M, h.n_slots, false).total;
   } else {
-    fn = h.scheme == SABR_MC_BESSEL ? mc_paths_kernel<float, SABR_MC_BESSEL> : mc_paths_kernel<float, SABR_MC_LOG_EULER>;
+    fn = h.scheme == SABR_MC_BESSEL ? mc_paths_kernel<float, SABR_MC_BESSEL, false>
+                                    : (split ? mc_paths_kernel<float, SABR_MC_LOG_EULER, true>
+                                             : mc_paths_kernel<float, SABR_MC_LOG_EULER, false>);
+    *smem = mc_smem_layout<float>(S, h.n_quotes, M, h.n_slots, split).total;
   }
-  cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h.smem);
+  cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem);
   return fn;
 }
 
 // Paths one thread takes at a time.
 static int mc_thread_paths(const McHost& h) {
   return h.scheme == SABR_MC_BESSEL ? kBesselPathsPerThread : mc_paths_per_thread(h.prec);
+}
+
+// Blocks per SM that the grid of a pricing counts on.  The grid decides which
+// paths share a thread and a warp, hence the order of the FP32 payoff sums,
+// so it is a rule on the precision, the scheme and the table bytes and not
+// what a build's register count happens to allow.
+static int mc_grid_blocks_per_sm(const McHost& h) {
+  const int cap = mc_resident_blocks(h.prec, h.scheme);
+  const size_t per_block = ((h.smem + 127) & ~(size_t)127) + 1024;
+  return (int)std::min<size_t>(cap, std::max<size_t>(1, (228 * 1024) / per_block));
 }
 
 // Blocks per parameter set.  Every block of a launch does the same work
@@ -302,10 +412,7 @@ static int mc_thread_paths(const McHost& h) {
 // 760 resident blocks: p = 8 (3 rounds, 0.375) instead of p = 2 (one round
 // with a third of the GPU idle, 0.5).
 int mc_blocks_per_set(const McHost& h, int n_sets) {
-  int per_sm = 8;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mc_paths_fn(h), kMcBlock, h.smem);
-  per_sm = std::min(std::max(per_sm, 1), 8);
-  const int64_t resident = device_sms() * (int64_t)per_sm;
+  const int64_t resident = device_sms() * (int64_t)mc_grid_blocks_per_sm(h);
   const int64_t sets = std::max(1, n_sets);
   const int64_t per_block = (int64_t)kMcBlock * mc_thread_paths(h);
   const int64_t by_paths = (h.n_paths + per_block - 1) / per_block;
@@ -322,18 +429,46 @@ int mc_blocks_per_set(const McHost& h, int n_sets) {
   return (int)best;
 }
 
+// A launch of at most one block of kMcBlock threads per SM runs the FP32
+// log-Euler form with a pair of paths a thread: two warps a scheduler instead
+// of one (2^15 paths x 504 steps: 158 us a call against 168; from two blocks
+// an SM on, 2^17 paths, two pairs a thread are the faster form, 217 us
+// against 231).
+static bool mc_split(const McHost& h, int64_t blocks) {
+  return h.prec == SABR_FP32 && h.scheme == SABR_MC_LOG_EULER && blocks <= (int64_t)device_sms();
+}
+
+// Fills d.tab for n_sets sets.
+void mc_launch_steps(const McHost& h, const McDev& d, const double* set_params, const int* set_valid, int n_sets,
+                     cudaStream_t s) {
+  const dim3 grid((h.n_steps + 63) / 64, n_sets);
+  void* tab = const_cast<void*>(d.tab);
+  if (h.scheme == SABR_MC_BESSEL) {
+    if (h.prec == SABR_FP64)
+      mc_steps_kernel<double, SABR_MC_BESSEL><<<grid, 64, 0, s>>>(d, set_params, set_valid, tab);
+    else
+      mc_steps_kernel<float, SABR_MC_BESSEL><<<grid, 64, 0, s>>>(d, set_params, set_valid, tab);
+  } else if (h.prec == SABR_FP64) {
+    mc_steps_kernel<double, SABR_MC_LOG_EULER><<<grid, 64, 0, s>>>(d, set_params, set_valid, tab);
+  } else {
+    mc_steps_kernel<float, SABR_MC_LOG_EULER><<<grid, 64, 0, s>>>(d, set_params, set_valid, tab);
+  }
+}
+
 static void launch_paths(const McHost& h, const McDev& d, const double* set_params, const int* set_valid,
                          dim3 grid, double* partial, int block0, int grid_total, cudaStream_t s) {
-  mc_paths_fn(h)<<<grid, kMcBlock, h.smem, s>>>(d, set_params, set_valid, partial, block0, grid_total);
+  if (d.tab != nullptr) mc_launch_steps(h, d, set_params, set_valid, (int)grid.y, s);
+  const bool split = mc_split(h, (int64_t)grid.x * grid.y);
+  size_t smem = 0;
+  const McPathsFn fn = mc_paths_fn(h, split, &smem);
+  fn<<<grid, split ? 2 * kMcBlock : kMcBlock, smem, s>>>(d, set_params, set_valid, partial, block0, grid_total);
 }
 
 sabr_status mc_launch(const McHost& h, const McDev& d, const double* set_params, const int* set_valid, int n_sets,
                       int blocks_per_set, double* partial, const int* q_value, const int* q_out,
                       const double* disc, double* price, double* se, int out_stride, cudaStream_t s) {
   launch_paths(h, d, set_params, set_valid, dim3(blocks_per_set, n_sets), partial, 0, 0, s);
-  const int total = n_sets * h.n_quotes;
-  mc_reduce_kernel<<<(total + 127) / 128, 128, 0, s>>>(d, n_sets, blocks_per_set, partial, q_value, q_out, disc,
-                                                       set_valid, price, se, out_stride);
+  launch_reduce(d, n_sets, blocks_per_set, partial, q_value, q_out, disc, set_valid, price, se, out_stride, s);
   SABR_CUDA(cudaGetLastError());
   return SABR_OK;
 }
@@ -391,7 +526,9 @@ static sabr_status mc_price(sabr_model model, const double* params, double fwd, 
   const size_t img = mc_image_bytes(h);
   const size_t params_off = (img + 255) & ~(size_t)255;
   const size_t part_off = params_off + 256;
-  const size_t dev_bytes = part_off + sizeof(double) * (size_t)bps * h.n_slots * 32;
+  const size_t tab_off = part_off + sizeof(double) * (size_t)bps * h.n_slots * 32;
+  const size_t tab_bytes = mc_step_table_bytes(h, 1);
+  const size_t dev_bytes = tab_off + tab_bytes;
   std::lock_guard<std::mutex> lock(g_mc_mutex);
   int dev = 0;
   SABR_CUDA(cudaGetDevice(&dev));
@@ -404,6 +541,7 @@ static sabr_status mc_price(sabr_model model, const double* params, double fwd, 
   double* disc;
   unsigned char* base = (unsigned char*)w.dev;
   mc_fill_image(h, w.host, base, d, &q_value, &q_out, &disc);
+  if (tab_bytes) d.tab = base + tab_off;
   double p10[kMaxD];
   for (int i = 0; i < kMaxD; ++i) p10[i] = i < n_params(model) ? params[i] : 0.0;
   std::memcpy(w.host + params_off, p10, sizeof(p10));
@@ -472,9 +610,11 @@ static sabr_status mc_shard_upload(const McShardCall& c, const double* params, c
   SABR_CUDA(cudaGetDevice(&dev));
   if ((int)g_mc_ws.size() <= dev) g_mc_ws.resize(dev + 1);
   McWorkspace& w = g_mc_ws[dev];
-  SABR_TRY(ensure_ws(w, part_off, part_off));
+  const size_t tab_bytes = mc_step_table_bytes(c.h, 1);
+  SABR_TRY(ensure_ws(w, part_off + tab_bytes, part_off));
   unsigned char* base = (unsigned char*)w.dev;
   mc_fill_image(c.h, w.host, base, d, q_value, q_out, disc);
+  if (tab_bytes) d.tab = base + part_off;
   double p10[kMaxD];
   for (int i = 0; i < kMaxD; ++i) p10[i] = i < n_params(c.h.model) ? params[i] : 0.0;
   std::memcpy(w.host + params_off, p10, sizeof(p10));
@@ -546,8 +686,7 @@ extern "C" sabr_status sabr_mc_shard_reduce(sabr_model model, const double* para
   const double* dp;
   McWorkspace* w;
   SABR_TRY(mc_shard_upload(c, params, s, d, &q_value, &q_out, &disc, &dp, &w));
-  mc_reduce_kernel<<<(c.h.n_quotes + 127) / 128, 128, 0, s>>>(d, 1, total_blocks, partials, q_value, q_out, disc,
-                                                               nullptr, price_out, stderr_out, (int)n);
+  launch_reduce(d, 1, total_blocks, partials, q_value, q_out, disc, nullptr, price_out, stderr_out, (int)n, s);
   SABR_CUDA(cudaGetLastError());
   SABR_CUDA(cudaEventRecord(w->done, s));
   return SABR_OK;

@@ -46,43 +46,13 @@ constexpr int kBesselTrials = 8;
 // dependency chains; the Gamma trials branch per path).
 constexpr int kBesselPathsPerThread = 2;
 
-// Per-step coefficients (same size as StepCoef, so the pricer's shared
-// memory layout serves both schemes).
+// Per-step coefficients.
 template <class R> struct __align__(16) StepCoefB {
   R kap;  // nu sqrt(h)
   R rsh;  // rho sqrt(h)
   R hh;   // h / 2
   R omr;  // 1 - rho^2
 };
-static_assert(sizeof(StepCoefB<float>) == sizeof(StepCoef<float>), "step table layout");
-static_assert(sizeof(StepCoefB<double>) == sizeof(StepCoef<double>), "step table layout");
-
-template <class R>
-__device__ __forceinline__ void build_steps_bessel(const McDev& P, const double* p, StepCoefB<R>* tab, int* land) {
-  for (int i = threadIdx.x; i < P.n_steps; i += blockDim.x) {
-    const double h = P.step_h[i], t = P.step_t[i];
-    double nu, rho;
-    if (P.model == SABR_DYN_I) {
-      rho = p[2] * exp(-p[4] * t);
-      nu = p[3] * exp(-p[5] * t);
-    } else if (P.model == SABR_DYN_II) {
-      rho = (p[2] + p[8] * t) * exp(-p[4] * t) + p[6];
-      nu = (p[3] + p[9] * t) * exp(-p[5] * t) + p[7];
-    } else {
-      rho = p[2];
-      nu = p[3];
-    }
-    const double sh = sqrt(h);
-    StepCoefB<R> s;
-    s.kap = (R)(nu * sh);
-    s.rsh = (R)(rho * sh);
-    s.hh = (R)(0.5 * h);
-    s.omr = (R)fmax(0.0, (1.0 - rho) * (1.0 + rho));
-    tab[i] = s;
-    const int m = P.step_mat[i];
-    if (m >= 0) land[m] = i;
-  }
-}
 
 // The elementary functions of the step in each precision: FP32 takes the
 // SFU forms where their error is far below the Monte Carlo noise (ln and the
@@ -115,11 +85,14 @@ __device__ __forceinline__ uint4 bessel_words(const McDev& P, int64_t path, int 
   }
 }
 
-// Per-step constants shared by every path of the step.
-template <class R> struct BesselStep {
+// Everything a step shares between its paths: formed once per step by
+// mc_steps_kernel (a division, a square root and two reciprocals, which every
+// thread used to repeat in every step) and read by all paths through L1.
+template <class R> struct __align__(16) BesselStep {
   StepCoefB<R> s;
   R inv_kap;        // 1 / kap, or 0 at nu = 0
   R a, d, c, inva;  // Gamma shape, Marsaglia-Tsang d and c, 1/a for a < 1 (else 0)
+  R unused[3];
 };
 
 template <class R>
@@ -137,6 +110,25 @@ __device__ __forceinline__ BesselStep<R> bessel_step_setup(const StepCoefB<R>& s
     k.inva = k.a < (R)1 ? (R)1 / k.a : (R)0;
   }
   return k;
+}
+
+template <class R>
+__device__ __forceinline__ BesselStep<R> bessel_step_entry(const McDev& P, const double* p, int i) {
+  const double h = P.step_h[i];
+  double nu = p[3], rho = p[2];
+  double sh;
+  if (P.model == SABR_DYN_I || P.model == SABR_DYN_II) {
+    dynamic_nu_rho(P.model, p, P.step_t[i], nu, rho);
+    sh = sqrt(h);
+  } else {
+    sh = P.step_t[i];
+  }
+  StepCoefB<R> s;
+  s.kap = (R)(nu * sh);
+  s.rsh = (R)(rho * sh);
+  s.hh = (R)(0.5 * h);
+  s.omr = (R)fmax(0.0, (1.0 - rho) * (1.0 + rho));
+  return bessel_step_setup<R>(s, p[1] == 1.0 ? (R)0 : (R)(p[1] / (1.0 - p[1])));
 }
 
 template <class R>
@@ -221,7 +213,7 @@ __device__ __forceinline__ void bessel_step(const McDev& P, const BesselStep<R>&
 // landing steps and payoff accumulation of simulate_paths_scalar, one step
 // at a time.
 template <class R, bool LOGNORMAL>
-__device__ __forceinline__ void simulate_paths_bessel(const McDev& P, const double* p, const StepCoefB<R>* tab,
+__device__ __forceinline__ void simulate_paths_bessel(const McDev& P, const double* p, const BesselStep<R>* tab,
                                                       const int* land, const int* s_q0, const int* s_nq,
                                                       const int* s_slot, const R* sK, const int8_t* scall,
                                                       int64_t path0, int64_t pstride, double* wacc) {
@@ -281,7 +273,7 @@ __device__ __forceinline__ void simulate_paths_bessel(const McDev& P, const doub
       i_land = m < P.n_mats ? land[m] : -1;
     };
     for (int i = 0; i < n_steps; ++i) {
-      const BesselStep<R> k = bessel_step_setup<R>(tab[i], bb);
+      const BesselStep<R> k = tab[i];
 #pragma unroll
       for (int j = 0; j < NPT; ++j) bessel_step<R, LOGNORMAL>(P, k, bb, path[j], i, st[j]);
       if (i == i_land) pay_out();

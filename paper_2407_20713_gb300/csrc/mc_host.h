@@ -31,6 +31,13 @@ size_t mc_image_bytes(const McHost& h);
 void mc_fill_image(const McHost& h, unsigned char* host_img, unsigned char* dev_base, McDev& d, int** q_value,
                    int** q_out, double** disc);
 int mc_blocks_per_set(const McHost& h, int n_sets);
+// Device bytes of the step tables of n_sets parameter sets (McDev::tab), 0
+// where none is used.  A caller without room for them leaves McDev::tab null
+// (log-Euler only): the blocks then build their tables themselves.
+size_t mc_step_table_bytes(const McHost& h, int n_sets);
+// Fills McDev::tab of n_sets parameter sets.
+void mc_launch_steps(const McHost& h, const McDev& d, const double* set_params, const int* set_valid, int n_sets,
+                     cudaStream_t s);
 // Enqueues the path kernel (grid blocks_per_set x n_sets) and the reduction.
 sabr_status mc_launch(const McHost& h, const McDev& d, const double* set_params, const int* set_valid, int n_sets,
                       int blocks_per_set, double* partial, const int* q_value, const int* q_out,

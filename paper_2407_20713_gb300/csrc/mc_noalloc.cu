@@ -89,6 +89,9 @@ extern "C" sabr_status sabr_mc_price_noalloc(sabr_model model, const double* par
   int* q_out;
   double* disc;
   mc_fill_image(h, g_noalloc_host, base, d, &q_value, &q_out, &disc);
+  // the step table where the scratch has room for it beside the partial sums
+  const size_t tab_bytes = mc_step_table_bytes(h, 1);
+  if (tab_bytes && need + tab_bytes <= kNoAllocScratchBytes) d.tab = base + need;
   double p10[kMaxD];
   for (int i = 0; i < kMaxD; ++i) p10[i] = i < n_params(model) ? params[i] : 0.0;
   std::memcpy(g_noalloc_host + params_off, p10, sizeof(p10));

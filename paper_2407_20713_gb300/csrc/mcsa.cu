@@ -1,4 +1,5 @@
 // mcsa.cu -- kernels and host enqueue of Technique II (see mcsa.cuh).
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 
@@ -223,6 +224,10 @@ __global__ void mcsa_rescore_kernel(McSaDev P) {
 // ---------------------------------------------------------------------------
 // Host
 // ---------------------------------------------------------------------------
+// Step tables beyond this (chains x steps x 16 bytes) are built by the path
+// blocks instead.
+constexpr size_t kMaxStepTables = 64u << 20;
+
 size_t mcsa_arena_bytes(const McSaHost& m) {
   // dry run of mcsa_layout from offset 0 (no image, no device base)
   McSaHost t = m;
@@ -286,6 +291,13 @@ void mcsa_layout(McSaHost& m, unsigned char* img, unsigned char* base, size_t of
   d.one_prices = (double*)(base + take(8 * Q));
   m.partial = (double*)(base + take(8 * C * (size_t)m.bps * nv));
   m.partial1 = (double*)(base + take(8 * (size_t)m.bps1 * nv));
+  // step tables, shared by the waves, the single evaluations and the re-score
+  // (they follow one another on a stream)
+  const size_t tab_bytes = std::max(mc_step_table_bytes(m.mc, m.n_chains), mc_step_table_bytes(m.mc64, 1));
+  if (m.step_tables && tab_bytes > 0 && tab_bytes <= kMaxStepTables) {
+    const size_t o_tab = take(tab_bytes);
+    if (write) m.dmc.tab = m.dmc64.tab = base + o_tab;
+  }
   d.result = dres;
   m.end = o;
 }

@@ -22,6 +22,7 @@ struct McSaHost {
   int *q_value = nullptr, *q_out = nullptr, *q_value64 = nullptr, *q_out64 = nullptr;
   double *disc = nullptr, *disc64 = nullptr;
   double *partial = nullptr, *partial1 = nullptr;
+  bool step_tables = true;  // dynamic models: keep room for every chain's step table
   size_t end = 0;
 };
 

@@ -118,9 +118,6 @@ constexpr int kSpecDepth = 2;
 // 20 quotes: ten pairs, measured against five on the 21-strike smiles
 // (3.08e10 against 2.96e10 cost-evals/s).
 constexpr int kBigChunk = 10;
-template <int N> struct IntTag {
-  static constexpr int value = N;
-};
 
 template <int MODEL> struct Dim {
   static constexpr int value = MODEL == SABR_DYN_II ? 10 : (MODEL == SABR_DYN_I ? 6 : 4);

@@ -14,6 +14,11 @@
 
 namespace sabr {
 
+// A compile-time number as an argument.
+template <int N> struct IntTag {
+  static constexpr int value = N;
+};
+
 // ---------------------------------------------------------------------------
 // Precision traits
 // ---------------------------------------------------------------------------

@@ -480,6 +480,10 @@ static sabr_status submit(sabr_server* s, const sabr_problem* pr, const sabr_bou
     r->is_mc = true;
     SABR_TRY(mcsa_prepare(*pr, *b, *c, seed, r->mh));
     r->bytes = mcsa_arena_bytes(r->mh);
+    if (r->bytes > (size_t)s->cfg.device_bytes) {  // the step tables are optional
+      r->mh.step_tables = false;
+      r->bytes = mcsa_arena_bytes(r->mh);
+    }
   } else {
     SABR_TRY(formula_prepare(*pr, *b, *c, seed, r->hp));
     if (r->hp.n_quotes > s->cfg.max_quotes) return fail(SABR_EINVAL, "request has more quotes than max_quotes");

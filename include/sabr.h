@@ -374,8 +374,11 @@ sabr_status sabr_plan_results(sabr_plan* plan, sabr_result* out);
  * more units per level than the GPU holds resident blocks, or one problem
  * two of whose levels fit in them; problems then move from level to level
  * independently, and SABR_ETIMEOUT in a result means a wait of that launch
- * gave up and its levels did not all run.  Other groups launch one kernel
- * per level.  The launch shape never changes the results. */
+ * gave up and its levels did not all run.  A group of one static problem with
+ * few chains (up to eight per SM in FP32, four in FP64) runs all levels in one
+ * cooperative launch whose blocks meet at the level ends, with the same bound
+ * on their waits.  Other groups launch one kernel per level.  The launch shape
+ * never changes the results. */
 sabr_status sabr_plan_stats(sabr_plan* plan, int64_t* launches_per_run,
                             double* level_kernel_ms);
 void sabr_plan_destroy(sabr_plan* plan);

@@ -55,7 +55,7 @@ struct ProblemDev {
   double* part_f;      // [n_blocks] block argmin of the final states
   int* part_c;
   double* part_x;      // [n_blocks][10]
-  unsigned int* arrive;
+  unsigned int* arrive;  // [2] arrivals at a level end; a wait that gave up (sa_small_kernel)
   sabr_result* result;
   // FP32 Case II term-structure rule (device copies of HostProblem's)
   const float4* c2_node;

@@ -26,6 +26,7 @@ struct HostProblem {
   std::vector<float> c2_node, c2_sub;
   std::vector<int> c2_panel;
   int c2_nsub = 0;
+  int part_rows = 0;  // block minima to keep room for beyond the level kernels' (sa_small_kernel)
 };
 
 sabr_status formula_prepare(const sabr_problem& pr, const sabr_bounds& b, const sabr_cooling& c, uint64_t seed,

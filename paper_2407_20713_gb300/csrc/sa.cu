@@ -30,80 +30,10 @@
 #include "engine.cuh"
 #include "engine_host.h"
 #include "mcsa_host.h"
+#include "sa_device.cuh"
+#include "sa_small.cuh"
 
 namespace sabr {
-
-// ---------------------------------------------------------------------------
-// Shared-memory staging of a problem's quotes.
-// ---------------------------------------------------------------------------
-template <class R>
-__device__ __forceinline__ SmemQuotes<R> stage_quotes(const ProblemDev& P, unsigned char* base,
-                                                      int nthreads, int tid, unsigned char** end) {
-  const int Q = P.n_quotes, M = P.n_mats;
-  // Q + 1 quote slots: the pair layout of an odd count needs one more
-  QuotePack<R>* pack = (QuotePack<R>*)base;  // base is 16-byte aligned
-  R* l2k = (R*)(pack + Q + 1);
-  R* mT = l2k + Q;
-  const bool dyn = P.model == SABR_DYN_I || P.model == SABR_DYN_II;
-  if (sizeof(R) == 4 && P.model == SABR_HAGAN) {
-    float4* pr = (float4*)base;
-    const float* lfk = (const float*)P.q_lfk;
-    const float* l2kf = (const float*)P.q_l2kf;
-    const float* T = (const float*)P.q_T;
-    const float* w = (const float*)P.q_w;
-    for (int j = tid; j < (Q + 1) / 2; j += nthreads) {
-      const int i0 = 2 * j, i1 = 2 * j + 1;
-      const bool two = i1 < Q;
-      pr[2 * j] = make_float4(lfk[i0], two ? lfk[i1] : 0.0f, l2kf[i0], two ? l2kf[i1] : 0.0f);
-      pr[2 * j + 1] = make_float4(T[i0], two ? T[i1] : 0.0f, -w[i0], two ? -w[i1] : 0.0f);
-    }
-  } else {
-    for (int i = tid; i < Q; i += nthreads) {
-      QuotePack<R> qp;
-      qp.lfk = ((const R*)P.q_lfk)[i];
-      qp.l2kf = dyn ? mat_in_slot(P.q_mat[i], R{}) : ((const R*)P.q_l2kf)[i];
-      qp.T = ((const R*)P.q_T)[i];
-      qp.w = ((const R*)P.q_w)[i];
-      pack[i] = qp;
-      l2k[i] = ((const R*)P.q_l2k)[i];
-    }
-  }
-  for (int j = tid; j < M; j += nthreads) mT[j] = ((const R*)P.m_T)[j];
-  unsigned char* e = (unsigned char*)(((uintptr_t)(mT + M) + 15) & ~(uintptr_t)15);
-  SmemQuotes<R> sq{pack, (const float4*)base, l2k, mT, nullptr, nullptr, nullptr};
-  if (sizeof(R) == 4 && P.model == SABR_DYN_II) {
-    // the Case II term-structure rule: nodes, sub-panels, maturity panels
-    float4* nd = (float4*)e;
-    float4* sb = nd + kC2Nodes * P.c2_nsub;
-    int2* pn = (int2*)(sb + P.c2_nsub);
-    for (int i = tid; i < kC2Nodes * P.c2_nsub; i += nthreads) nd[i] = P.c2_node[i];
-    for (int i = tid; i < P.c2_nsub; i += nthreads) sb[i] = P.c2_sub[i];
-    for (int i = tid; i < M; i += nthreads) pn[i] = P.c2_panel[i];
-    sq.c2_node = nd;
-    sq.c2_sub = sb;
-    sq.c2_panel = pn;
-    e = (unsigned char*)(((uintptr_t)(pn + M) + 15) & ~(uintptr_t)15);
-  }
-  *end = e;
-  return sq;
-}
-
-// Lexicographic minimum of (f, i): the smaller f, then the smaller index, so
-// the result does not depend on the order of merging.
-__device__ __forceinline__ void argmin_merge(double& f, int& i, double f2, int i2) {
-  if (f2 < f || (f2 == f && i2 < i)) {
-    f = f2;
-    i = i2;
-  }
-}
-__device__ __forceinline__ void warp_argmin(double& f, int& i) {
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    const double f2 = __shfl_xor_sync(0xffffffffu, f, off);
-    const int i2 = __shfl_xor_sync(0xffffffffu, i, off);
-    argmin_merge(f, i, f2, i2);
-  }
-}
 
 // Quote pairs per point the speculative Hagan loop keeps in flight (several
 // points are evaluated at once, so fewer than QueuePairs), and the steps it
@@ -118,41 +48,6 @@ constexpr int kSpecDepth = 2;
 // 20 quotes: ten pairs, measured against five on the 21-strike smiles
 // (3.08e10 against 2.96e10 cost-evals/s).
 constexpr int kBigChunk = 10;
-
-template <int MODEL> struct Dim {
-  static constexpr int value = MODEL == SABR_DYN_II ? 10 : (MODEL == SABR_DYN_I ? 6 : 4);
-};
-
-__device__ __forceinline__ unsigned group_mask(int G) {
-  if (G >= 32) return 0xffffffffu;
-  const int lane32 = threadIdx.x & 31;
-  return ((1u << G) - 1u) << (lane32 & ~(G - 1));
-}
-
-__device__ __forceinline__ void load_problem(const ProblemDev* probs, int pid, ProblemDev* P) {
-  const int words = (int)(sizeof(ProblemDev) / 4);
-  for (int i = threadIdx.x; i < words; i += blockDim.x)
-    ((int*)P)[i] = ((const int*)(probs + pid))[i];
-  __syncthreads();
-}
-
-// Proposal step: x' = x + step (2u - 1).  The FP64 form rounds each
-// operation exactly as written (no contraction into an FMA).
-__device__ __forceinline__ float propose(float x, float step, float u) {
-  return x + step * (2.0f * u - 1.0f);
-}
-__device__ __forceinline__ double propose(double x, double step, double u) {
-  return __dadd_rn(x, __dmul_rn(step, __dsub_rn(__dmul_rn(2.0, u), 1.0)));
-}
-// Metropolis acceptance of an uphill move (delta > 0) at temperature Tk.
-// FP32 form: u < 2^(-delta log2(e)/Tk) by the SFU, with log2(e)/Tk formed
-// once per level.
-__device__ __forceinline__ bool metropolis(float u, float delta, float inv_Tk, double) {
-  return u < ex2_approx(-delta * inv_Tk);
-}
-__device__ __forceinline__ bool metropolis(double u, double delta, float, double Tk) {
-  return u < exp(-delta / Tk);
-}
 
 // Ready queue of a plan's launch group.  entry[u] names unit u as
 // (problem, level, block) with the top bit set, or is 0 until the unit is
@@ -171,12 +66,6 @@ __host__ __device__ constexpr unsigned long long queue_entry(int p, int lv, int 
   return (1ull << 63) | ((unsigned long long)p << 43) | ((unsigned long long)lv << 23) | (unsigned long long)blk;
 }
 constexpr int kQueueMaxProblems = 1 << 20, kQueueMaxLevels = 1 << 20, kQueueMaxBlocks = 1 << 23;
-
-__device__ __forceinline__ unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
 
 // Waits (one thread) until entry u has been appended; 0 when the queue's
 // error flag is set or the wait runs past q.wait_ns (which then sets it).
@@ -225,6 +114,7 @@ __global__ void sa_init_kernel(const ProblemDev* __restrict__ probs, const int* 
     P.state[kMaxD] = f0;
     P.state[kMaxD + 1] = P.T0_given > 0.0 ? P.T0_given : (f0 > 0.0 ? f0 : 1.0);
     P.result->status = isfinite(f0) ? SABR_OK : SABR_EINVAL;
+    P.arrive[0] = P.arrive[1] = 0u;
   }
 }
 
@@ -250,8 +140,7 @@ __device__ __forceinline__ void sa_level_block(const ProblemDev& P, int pid, int
   const int coef_m = (MODEL == SABR_DYN_I || MODEL == SABR_DYN_II) ? P.n_mats : 0;
   constexpr int CS = CoefStride<R, MODEL>::value;
   R* coef = (R*)rest + (size_t)g * CS * coef_m;
-  double* red_f = (double*)((R*)rest + (size_t)cpb * CS * coef_m + 16);
-  red_f = (double*)(((uintptr_t)red_f + 15) & ~(uintptr_t)15);
+  double* red_f = (double*)(rest + ((((size_t)cpb * CS * coef_m + 16) * sizeof(R) + 15) & ~(size_t)15));
   R* red_x = (R*)(red_f + cpb);
   __syncthreads();
 
@@ -602,6 +491,7 @@ __device__ __forceinline__ void sa_level_block(const ProblemDev& P, int pid, int
     int best = 0x7fffffff;
     for (int c = threadIdx.x; c < cpb; c += 32) argmin_merge(fb, best, red_f[c], c);
     warp_argmin(fb, best);
+    if (best >= cpb) best = 0;  // no cost compares (all NaN)
     if (threadIdx.x == 0) {
       P.part_f[blk] = fb;
       P.part_c[blk] = blk * cpb + best;
@@ -629,6 +519,7 @@ __device__ __forceinline__ void sa_level_block(const ProblemDev& P, int pid, int
     __syncthreads();
     if (threadIdx.x == 0) {
       for (int w = 1; w < (int)(blockDim.x >> 5); ++w) argmin_merge(f, bb, s_wf[w], s_wb[w]);
+      if (bb >= P.n_blocks) bb = 0;
       for (int i = 0; i < kMaxD; ++i) P.state[i] = __ldcg(&P.part_x[(size_t)bb * kMaxD + i]);
       P.state[kMaxD] = f;
       P.state[kStateArgChain] = (double)(P.chain0 + __ldcg(&P.part_c[bb]));
@@ -698,11 +589,7 @@ template <class R, int MODEL> struct QueuePairs {
   static constexpr int value = 5;
 };
 
-// SEL: the speculative Hagan loop takes its decisions as selects (the
-// launches of single problems, whose chains have several lanes; in the
-// kernel that also runs the one-lane step loop of large batches they
-// measured 1.6% slower there, from its register allocation).
-template <class R, int MODEL, bool SEL = false>
+template <class R, int MODEL>
 __global__ void __launch_bounds__(kLevelBlock, (QueueBlocks<R, MODEL>::value))
     sa_queue_kernel(const ProblemDev* __restrict__ probs, LevelQueue q) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -724,7 +611,7 @@ __global__ void __launch_bounds__(kLevelBlock, (QueueBlocks<R, MODEL>::value))
     const int lv = (int)((e >> 23) & (kQueueMaxLevels - 1));
     const int blk = (int)(e & (kQueueMaxBlocks - 1));
     load_problem(probs, pid, &P);
-    sa_level_block<R, MODEL, QueuePairs<R, MODEL>::value, SEL>(P, pid, blk, lv, smem, &q);
+    sa_level_block<R, MODEL, QueuePairs<R, MODEL>::value>(P, pid, blk, lv, smem, &q);
     __syncthreads();
   }
 }
@@ -808,7 +695,7 @@ __global__ void __launch_bounds__(kSaBlock) sa_finalize_kernel(const ProblemDev*
     }
     r->misfit = f;
     r->restart_misfit = P.state[kMaxD];
-    if (queue_err != nullptr && *queue_err != 0u) r->status = SABR_ETIMEOUT;
+    if ((queue_err != nullptr && *queue_err != 0u) || P.arrive[1] != 0u) r->status = SABR_ETIMEOUT;
     r->n_evals = (int64_t)te;
     r->n_accepts = (int64_t)ta;
   }
@@ -1078,14 +965,14 @@ size_t formula_layout(const HostProblem& h, int G, unsigned char* img, unsigned 
   d.key0 = (uint32_t)h.seed;
   d.key1 = (uint32_t)(h.seed >> 32);
   const size_t rs = h.prec == SABR_FP64 ? 8 : 4;
-  const size_t Q = h.n_quotes, M = h.n_mats, C = h.n_chains, B = d.n_blocks;
+  const size_t Q = h.n_quotes, M = h.n_mats, C = h.n_chains, B = std::max(d.n_blocks, h.part_rows);
   const size_t o_lfk = take(Q * rs), o_l2kf = take(Q * rs), o_l2k = take(Q * rs), o_T = take(Q * rs),
                o_w = take(Q * rs), o_mat = take(Q * 4), o_mT = take(M * rs);
   const size_t o64_lfk = take(Q * 8), o64_l2kf = take(Q * 8), o64_l2k = take(Q * 8), o64_T = take(Q * 8),
                o64_mkt = take(Q * 8), o64_mT = take(M * 8);
   const size_t o_ck = take(h.ck.size() * 8), o_x0 = take(kMaxD * 8), o_state = take(kStateLen * 8);
   const size_t o_bf = take(C * 8), o_bx = take(C * kMaxD * rs), o_ev = take(C * 8), o_ac = take(C * 8);
-  const size_t o_pf = take(B * 8), o_pc = take(B * 4), o_px = take(B * kMaxD * 8), o_arr = take(4);
+  const size_t o_pf = take(B * 8), o_pc = take(B * 4), o_px = take(B * kMaxD * 8), o_arr = take(8);
   const size_t o_c2n = take(4 * h.c2_node.size()), o_c2s = take(4 * h.c2_sub.size()),
                o_c2p = take(4 * h.c2_panel.size());
   if (write) {
@@ -1121,7 +1008,7 @@ size_t formula_layout(const HostProblem& h, int G, unsigned char* img, unsigned 
     put(o64_mT, h.mT.data(), M * 8);
     put(o_ck, h.ck.data(), h.ck.size() * 8);
     put(o_x0, h.x0, kMaxD * 8);
-    std::memset(img + o_arr, 0, 4);
+    std::memset(img + o_arr, 0, 8);
     put(o_c2n, h.c2_node.data(), 4 * h.c2_node.size());
     put(o_c2s, h.c2_sub.data(), 4 * h.c2_sub.size());
     put(o_c2p, h.c2_panel.data(), 4 * h.c2_panel.size());
@@ -1216,26 +1103,13 @@ void launch_finalize(int prec, int model, const ProblemDev* probs, const int* pl
   SABR_DISPATCH(prec, model, (sa_finalize_kernel<R, M><<<n, kSaBlock, 0, s>>>(probs, plist, queue_err)));
 }
 
-// single: the group is one problem (FP32 Hagan then takes the SEL kernel)
-static bool queue_sel(int prec, int model, bool single) { return single && prec == SABR_FP32 && model == SABR_HAGAN; }
-
 static void launch_queue(int prec, int model, const ProblemDev* probs, const LevelQueue& q, int grid, size_t smem,
-                         bool single, cudaStream_t s) {
-  if (queue_sel(prec, model, single)) {
-    sa_queue_kernel<float, SABR_HAGAN, true><<<grid, kLevelBlock, smem, s>>>(probs, q);
-    return;
-  }
+                         cudaStream_t s) {
   SABR_DISPATCH(prec, model, (sa_queue_kernel<R, M><<<grid, kLevelBlock, smem, s>>>(probs, q)));
 }
 
-static int queue_blocks_per_sm(int prec, int model, size_t smem, bool single) {
+static int queue_blocks_per_sm(int prec, int model, size_t smem) {
   int nb = 1;
-  if (queue_sel(prec, model, single)) {
-    cudaFuncSetAttribute(sa_queue_kernel<float, SABR_HAGAN, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sa_queue_kernel<float, SABR_HAGAN, true>, kLevelBlock, smem);
-    return nb < 1 ? 1 : nb;
-  }
   SABR_DISPATCH(prec, model, (cudaFuncSetAttribute(sa_queue_kernel<R, M>,
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
                               cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sa_queue_kernel<R, M>, kLevelBlock,
@@ -1265,6 +1139,12 @@ struct LaunchGroup {
   unsigned long long* d_level0 = nullptr;
   unsigned long long n0 = 0;
   int queue_grid = 0;
+  // few chains: one cooperative launch of sa_small_kernel (small_blocks > 0)
+  SmallShape small;
+  int small_blocks = 0;
+  size_t small_smem = 0;
+  unsigned long long small_wait_ns = 0;
+  int4* d_small = nullptr;
 };
 
 // Resident 64-thread blocks per SM that a plan's persistent level launch
@@ -1327,16 +1207,23 @@ static sabr_status enqueue_plan(sabr_plan* p, cudaStream_t s, bool capturing) {
   else
     SABR_CUDA(cudaEventRecord(p->ev_lv0, s));
   for (auto& g : p->groups) {
+    if (g.small_blocks == 0 || g.max_levels == 0) continue;
+    SABR_CUDA(launch_small(g.prec, g.model, g.small, p->d_probs, g.d_small, g.small_blocks, g.small_smem,
+                           g.small_wait_ns, s));
+    ++launches;
+    ++level_launches;
+  }
+  for (auto& g : p->groups) {
     if (!g.use_queue || g.q.total == 0) continue;
     queue_reset_kernel<<<(int)std::min<unsigned long long>(1024, (g.q.total + 255) / 256), 256, 0, s>>>(
         g.q, g.d_level0, g.n0);
-    launch_queue(g.prec, g.model, p->d_probs, g.q, g.queue_grid, g.smem_level, g.problems.size() == 1, s);
+    launch_queue(g.prec, g.model, p->d_probs, g.q, g.queue_grid, g.smem_level, s);
     launches += 2;
     ++level_launches;
   }
   for (int lv = 0; lv < p->max_levels; ++lv)
     for (auto& g : p->groups) {
-      if (g.use_queue || lv >= g.max_levels) continue;
+      if (g.use_queue || g.small_blocks > 0 || lv >= g.max_levels) continue;
       launch_level(g.prec, g.model, p->d_probs, g.d_bmap, g.total_blocks, lv, g.smem_level, s);
       ++launches;
       ++level_launches;
@@ -1372,6 +1259,33 @@ static void free_plan(sabr_plan* p) {
   if (p->arena) cudaFree(p->arena);
   if (p->h_results) cudaFreeHost(p->h_results);
   delete p;
+}
+
+// Per (precision, model): the launch of sa_small_kernel where the batch holds
+// one problem of that kind, of few chains and several lanes a chain (one lane
+// per chain sums in an order of its own, hagan_cost_g1); blocks = 0 elsewhere.
+struct SmallChoice {
+  SmallShape shape;
+  int blocks = 0;
+  size_t smem = 0;
+};
+static std::vector<SmallChoice> choose_small(const std::vector<HostProblem>& hp, const std::vector<int>& lanes) {
+  std::vector<SmallChoice> out(10);
+  std::vector<int> count(10, 0);
+  for (const HostProblem& h : hp) ++count[h.prec * 5 + h.model];
+  for (size_t i = 0; i < hp.size(); ++i) {
+    const HostProblem& h = hp[i];
+    const int kind = h.prec * 5 + h.model;
+    if (count[kind] != 1 || lanes[i] < 2 || !small_supported(h.prec, h.model) ||
+        h.n_chains > small_most_chains(h.prec))
+      continue;
+    SmallChoice c;
+    c.shape = small_shape(h.prec, h.n_quotes, h.n_chains);
+    c.smem = small_smem_bytes(h.prec, h.model, h.n_quotes, h.n_mats);
+    c.blocks = small_blocks(c.shape, h.n_chains);
+    if (c.blocks <= small_capacity(h.prec, h.model, c.shape, c.smem)) out[kind] = c;
+  }
+  return out;
 }
 
 static sabr_status build_plan(int32_t n, const sabr_problem* problems, const sabr_bounds* bounds,
@@ -1416,8 +1330,12 @@ static sabr_status build_plan(int32_t n, const sabr_problem* problems, const sab
   const size_t probs_off = take(sizeof(ProblemDev) * std::max(nf, 1));
   const size_t results_off = take(sizeof(sabr_result) * n);
   std::vector<size_t> f_off(nf), mc_off(p->mc.size());
-  for (int i = 0; i < nf; ++i) {
+  for (int i = 0; i < nf; ++i)
     lanes[i] = choose_lanes(hp[i].n_quotes, hp[i].n_mats, hp[i].model, hp[i].prec, batch_chains);
+  std::vector<SmallChoice> small = choose_small(hp, lanes);
+  for (int i = 0; i < nf; ++i) {
+    const SmallChoice& sc = small[hp[i].prec * 5 + hp[i].model];
+    if (sc.blocks > 0) hp[i].part_rows = 2 * small_blocks(sc.shape, hp[i].n_chains);
     if (level_smem_bytes(hp[i].prec, hp[i].model, hp[i].n_quotes, hp[i].n_mats, kLevelBlock / lanes[i],
                          hp[i].c2_nsub) > kMaxLevelSmem) {
       free_plan(p);
@@ -1446,12 +1364,15 @@ static sabr_status build_plan(int32_t n, const sabr_problem* problems, const sab
     p->max_levels = std::max(p->max_levels, hp[i].n_levels);
   }
   std::vector<size_t> bmap_off(p->groups.size()), plist_off(p->groups.size());
+  std::vector<size_t> small_off(p->groups.size());
   std::vector<size_t> qent_off(p->groups.size()), qctl_off(p->groups.size()), ql0_off(p->groups.size());
   std::vector<std::vector<unsigned long long>> level0(p->groups.size());
   const int sms = device_sms();
   for (size_t gi = 0; gi < p->groups.size(); ++gi) {
     LaunchGroup& g = p->groups[gi];
     bmap_off[gi] = take(sizeof(int4) * g.total_blocks);
+    const SmallChoice& sc = small[g.prec * 5 + g.model];
+    if (sc.blocks > 0) small_off[gi] = take(sizeof(int4) * sc.blocks);
     plist_off[gi] = take(sizeof(int) * g.problems.size());
     // ready queue: one entry per (problem, level, block) of the run
     unsigned long long total = 0;
@@ -1471,14 +1392,20 @@ static sabr_status build_plan(int32_t n, const sabr_problem* problems, const sab
     // instead of after a kernel launch (a level's fixed cost on one smile of
     // 64 chains: 13.7 us with a launch per level); larger single problems
     // run level by level.
-    const int per_sm = std::min(workers_per_sm(g.prec, g.model),
-                                queue_blocks_per_sm(g.prec, g.model, g.smem_level, g.problems.size() == 1));
+    const int per_sm = std::min(workers_per_sm(g.prec, g.model), queue_blocks_per_sm(g.prec, g.model, g.smem_level));
     int grid = std::max(1, std::min(g.total_blocks, sms * per_sm));
     const bool single_small = g.problems.size() == 1 && 2 * g.total_blocks <= sms * per_sm && p->max_levels > 1;
     if (single_small) grid = 2 * g.total_blocks;
     g.use_queue = queue_enabled() && ((g.problems.size() > 1 && g.total_blocks > grid) || single_small) &&
                   nf <= kQueueMaxProblems && p->max_levels < kQueueMaxLevels && total * 8 <= kMaxQueueBytes;
     for (int pi : g.problems) g.use_queue = g.use_queue && pd[pi].n_blocks <= kQueueMaxBlocks;
+    if (sc.blocks > 0) {
+      g.use_queue = false;
+      g.small = sc.shape;
+      g.small_blocks = sc.blocks;
+      g.small_smem = sc.smem;
+      g.small_wait_ns = (unsigned long long)std::min(6.0e11, 5.0e9 + 100.0 * unit_ns);
+    }
     if (g.use_queue) {
       g.q.total = total;
       g.q.wait_ns = (unsigned long long)std::min(6.0e11, 5.0e9 + 100.0 * unit_ns);
@@ -1512,6 +1439,13 @@ static sabr_status build_plan(int32_t n, const sabr_problem* problems, const sab
     std::memcpy(img.data() + plist_off[gi], g.problems.data(), sizeof(int) * g.problems.size());
     g.d_bmap = (int4*)(base + bmap_off[gi]);
     g.d_plist = (int*)(base + plist_off[gi]);
+    if (g.small_blocks > 0) {
+      std::vector<int4> sm;
+      for (int pi : g.problems)
+        for (int b = 0; b < small_blocks(g.small, hp[pi].n_chains); ++b) sm.push_back(make_int4(pi, b, 0, 0));
+      std::memcpy(img.data() + small_off[gi], sm.data(), sizeof(int4) * sm.size());
+      g.d_small = (int4*)(base + small_off[gi]);
+    }
     if (g.use_queue) {
       g.q.entry = (unsigned long long*)(base + qent_off[gi]);
       g.q.head = (unsigned long long*)(base + qctl_off[gi]);

@@ -1,0 +1,548 @@
+// sa_small.cu -- SA of problems with few chains (one smile of 64 chains is
+// the paper's case): the whole calibration in one launch, one to four warps
+// per chain.
+//
+// Such a problem cannot fill the GPU, and its time is the latency of its
+// dependent Metropolis steps plus that of its level ends.  Both are cut here:
+//
+//  * Speculation K steps deep.  Acceptance is the common outcome (94-97% of
+//    the evaluated proposals), so a chain forms the proposals of its next K
+//    steps as if every one inside the box were accepted (one outside is
+//    rejected for certain) and evaluates them side by side: NW warps, KW =
+//    K / NW groups of P = 32 / KW lanes each, a group a point.  The steps are
+//    then decided together -- step k's Metropolis test needs the cost of the
+//    step before it, which is another group's -- and the chain advances past
+//    the first rejection.  Its trajectory, counters and best point are those
+//    of the one-step loop bit for bit.
+//  * Every warp of a chain forms all K points and takes all K decisions
+//    itself, so the warps exchange nothing but the K costs (one barrier an
+//    iteration).
+//  * Proposal words are drawn 32 steps at a time, a Philox block a lane.
+//  * The blocks of a problem stay resident (a cooperative launch) and meet at
+//    each level end on one counter: every block writes its minimum, arrives,
+//    and takes the argmin over the minima itself.
+//
+// A chain's misfit is summed in the order that G lanes (ProblemDev::G) give
+// it: virtual lane v sums units v, v + G, ... and the virtual lanes are added
+// by a butterfly.  A lane here plays the virtual lanes v = p, p + P, ..., so
+// the first levels of the butterfly are additions within the lane.
+//
+// FP64: a scheduler issues one FP64 warp instruction in about 76 cycles, so
+// FP64 counts what FP64 instructions cost: box tests compare the numbers'
+// bits, the words are kept as FP32 (2u - 1 is exact there), and a chain's
+// warps sit on different schedulers.
+#include <algorithm>
+#include <cmath>
+
+#include "sa_device.cuh"
+#include "sa_small.cuh"
+
+namespace sabr {
+
+constexpr int kRing = 64;        // steps whose proposal words a warp holds
+constexpr int kLevelCache = 32;  // levels whose temperatures a block holds
+constexpr int kSmallBlock = 128;
+
+__device__ __forceinline__ double cost_xor(double v, int off) { return __shfl_xor_sync(0xffffffffu, v, off); }
+__device__ __forceinline__ DF cost_xor(DF v, int off) {
+  return DF{__shfl_xor_sync(0xffffffffu, v.hi, off), __shfl_xor_sync(0xffffffffu, v.lo, off)};
+}
+__device__ __forceinline__ double cost_add(double a, double b) { return a + b; }
+__device__ __forceinline__ DF cost_add(DF a, DF b) { return df_add(a, b); }
+// the first level of a sum: df_add of (a, 0) and (b, 0) is the exact sum
+__device__ __forceinline__ double cost_add_first(double a, double b) { return a + b; }
+__device__ __forceinline__ DF cost_add_first(float a, float b) { return df_two_sum(a, b); }
+__device__ __forceinline__ double lane_cost(double v) { return v; }
+__device__ __forceinline__ DF lane_cost(float v) { return DF{v, 0.0f}; }
+
+// Box tests.  FP64 bounds and numbers are compared as integers that order
+// like the (finite) numbers: 32-bit ALU instructions instead of FP64 compares.
+template <class R> struct BoxKey;
+template <> struct BoxKey<float> {
+  using T = float;
+  static __device__ __forceinline__ T of(float x) { return x; }
+};
+template <> struct BoxKey<double> {
+  using T = long long;
+  static __device__ __forceinline__ T of(double x) {
+    const long long b = __double_as_longlong(x);
+    return b >= 0 ? b : (long long)(0x8000000000000000ull - (unsigned long long)b);  // -0 is 0
+  }
+};
+
+// A proposal word 2u - 1, kept as the float it exactly is (an odd multiple of
+// 2^-23 in (-1, 1)), in the working precision; to FP64 by moving its bits.
+__device__ __forceinline__ float word_to(float w, float) { return w; }
+__device__ __forceinline__ double word_to(float w, double) {
+  const uint32_t b = __float_as_uint(w);
+  const uint32_t hi = (b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + ((1023u - 127u) << 20));
+  return __hiloint2double((int)hi, (int)(b << 29));
+}
+
+// One static formula at one point: constants, and the unit residuals.  A unit
+// is a quote, or for FP32 Hagan a pair of quotes (float2).
+template <class R, int MODEL> struct StaticPoint {
+  static constexpr bool kPair = MODEL == SABR_HAGAN && sizeof(R) == 4;
+  StaticConst<R> sc;
+  PolyCoef<R> c0;
+  R bw;
+  __device__ __forceinline__ StaticPoint(const R* x, R l2f) {
+    if constexpr (MODEL == SABR_EXPANDED) {
+      c0 = expanded_coef<R>(x, l2f, (R)0);
+      bw = expanded_coef<R>(x, l2f, (R)1).c0 - c0.c0;
+    } else {
+      sc = static_setup<R>(x);
+    }
+  }
+  __device__ __forceinline__ R resid_of(int q, const SmemQuotes<R>& sq) const {
+    const QuotePack<R> qp = sq.pack[q];
+    R vol;
+    if constexpr (MODEL == SABR_HAGAN) {
+      vol = vol_hagan<R>(sc, qp.lfk, qp.l2kf, qp.T);
+    } else if constexpr (MODEL == SABR_OBLOJ) {
+      vol = vol_obloj<R>(sc, qp.lfk, qp.l2kf, sq.l2k[q], qp.T);
+    } else {
+      PolyCoef<R> c = c0;
+      c.c0 = c0.c0 + bw * qp.T;
+      vol = vol_poly<R>(c, qp.lfk);
+    }
+    return resid(vol, qp.w);
+  }
+  __device__ __forceinline__ float2 resid_pair_of(int j, int n_quotes, const SmemQuotes<R>& sq) const {
+    const float4 a = sq.pair[2 * j], b = sq.pair[2 * j + 1];
+    return hagan_resid_pair(sc, make_float2(a.x, a.y), make_float2(a.z, a.w), make_float2(b.x, b.y),
+                            make_float2(b.z, b.w), make_float2(1.0f, 2 * j + 1 < n_quotes ? 1.0f : 0.0f));
+  }
+  // sums of N virtual lanes v[0..N-1], the lanes' units side by side.  A unit
+  // past the end is evaluated as unit 0 and counts 0 (adding 0 changes no sum).
+  template <int N>
+  __device__ __forceinline__ void partials(const int (&v)[N], int units, int G, int n_quotes,
+                                           const SmemQuotes<R>& sq, R (&out)[N]) const {
+    if constexpr (kPair) {
+      float2 acc[N];
+#pragma unroll
+      for (int k = 0; k < N; ++k) acc[k] = make_float2(0.0f, 0.0f);
+      for (int j0 = 0; j0 < units; j0 += G) {
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+          const bool on = j0 + v[k] < units;
+          float2 r = resid_pair_of(on ? j0 + v[k] : 0, n_quotes, sq);
+          r.x = on ? r.x : 0.0f;
+          r.y = on ? r.y : 0.0f;
+          acc[k] = fma2(r, r, acc[k]);
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < N; ++k) out[k] = acc[k].x + acc[k].y;
+    } else {
+#pragma unroll
+      for (int k = 0; k < N; ++k) out[k] = (R)0;
+      for (int j0 = 0; j0 < units; j0 += G) {
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+          const bool on = j0 + v[k] < units;
+          R r = resid_of(on ? j0 + v[k] : 0, sq);
+          r = on ? r : (R)0;
+          out[k] += r * r;
+        }
+      }
+    }
+  }
+};
+
+// How P lanes play G virtual lanes: pe of them differ (a lane beyond G repeats
+// another's work), V virtual lanes each.
+struct LaneSplit {
+  int pe, V, shift;  // shift = 32 - log2 V
+};
+__device__ __forceinline__ LaneSplit lane_split(int G, int P) {
+  LaneSplit s;
+  s.pe = G < P ? G : P;
+  s.V = G / s.pe;
+  s.shift = 32 - (31 - __clz(s.V));
+  return s;
+}
+
+// The misfit of a point by P lanes of a warp (every lane gets it).
+template <class R, int MODEL>
+__device__ __forceinline__ typename CostOf<R>::T point_cost(const R* x, int n_quotes, int units, R l2f,
+                                                            const SmemQuotes<R>& sq, int G, const LaneSplit& ls) {
+  using C = typename CostOf<R>::T;
+  const StaticPoint<R, MODEL> pt(x, l2f);
+  const int p = threadIdx.x & (ls.pe - 1);
+  C s;
+  int off = ls.pe >> 1;
+  if (ls.V == 1) {
+    const int v[1] = {p};
+    R a[1];
+    pt.template partials<1>(v, units, G, n_quotes, sq, a);
+    if (off > 0) {
+      s = cost_add_first(a[0], __shfl_xor_sync(0xffffffffu, a[0], off));
+      off >>= 1;
+    } else {
+      s = lane_cost(a[0]);
+    }
+  } else {
+    // the virtual lanes' butterfly starts with the farthest pairs: lanes are
+    // added in the order of their bit-reversed index, a binary counter holding
+    // the finished subtrees
+    C stack[5];
+#pragma unroll
+    for (int l = 0; l < 5; ++l) stack[l] = s = lane_cost((R)0);
+    for (int t = 0; t < ls.V; t += 2) {
+      const int i = (int)(__brev((unsigned)t) >> ls.shift);  // bit 0 of t is the farthest pair
+      const int v[2] = {p + ls.pe * i, p + ls.pe * (i + (ls.V >> 1))};
+      R a[2];
+      pt.template partials<2>(v, units, G, n_quotes, sq, a);
+      s = cost_add_first(a[0], a[1]);
+      bool carry = true;
+#pragma unroll
+      for (int l = 1; l < 5; ++l) {
+        if (carry) {
+          carry = ((t >> l) & 1) != 0;
+          if (carry) {
+            s = cost_add(stack[l], s);
+          } else {
+            stack[l] = s;
+          }
+        }
+      }
+    }
+  }
+  for (; off > 0; off >>= 1) s = cost_add(s, cost_xor(s, off));
+  return s;
+}
+
+// Barrier of a chain's NW warps (they are neighbours in the block).
+template <int NW> __device__ __forceinline__ void chain_sync(int chain_in_block) {
+  if constexpr (NW == 1) {
+    __syncwarp();
+  } else if constexpr (NW == kSmallBlock / 32) {
+    __syncthreads();
+  } else {
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + chain_in_block), "r"(32 * NW) : "memory");
+  }
+}
+
+// Block minima alternate between two buffers by the level's parity: a block
+// writes the minima of level k + 2 only after every block has read those of
+// level k (it arrives at k + 1 after reading them).  The costs of an iteration
+// alternate likewise.
+template <class R, int MODEL, int NW, int KW>
+__global__ void __launch_bounds__(kSmallBlock) sa_small_kernel(const ProblemDev* __restrict__ probs,
+                                                              const int4* __restrict__ work,
+                                                              unsigned long long wait_ns) {
+  using C = typename CostOf<R>::T;
+  using Key = typename BoxKey<R>::T;
+  constexpr int D = 4, P = 32 / KW, K = NW * KW, CPB = kSmallBlock / 32 / NW;
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ ProblemDev Pr;
+  __shared__ R s_step[kLevelCache][D];
+  __shared__ double s_Tk[kLevelCache];
+  __shared__ float s_invTk[kLevelCache];
+  __shared__ float s_w[kSmallBlock / 32][D][kRing];  // proposal words 2u - 1 of each warp
+  __shared__ float s_u[kSmallBlock / 32][kRing];     // acceptance uniforms
+  __shared__ __align__(16) R s_x[kSmallBlock / 32][K][D];  // points of the window
+  __shared__ C s_f[CPB][2][K];                       // their costs
+  __shared__ double s_mf[CPB], s_mx[CPB][D], s_new[D + 1];
+  __shared__ int s_stop;
+  const int4 it = work[blockIdx.x];
+  load_problem(probs, it.x, &Pr);
+  const int blk = it.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int cb = warp / NW, wc = warp % NW;  // chain in the block, warp in the chain
+  const int nb = (Pr.n_chains + CPB - 1) / CPB;
+  unsigned char* rest;
+  const SmemQuotes<R> sq = stage_quotes<R>(Pr, smem, blockDim.x, threadIdx.x, &rest);
+  if (threadIdx.x == 0) s_stop = 0;
+  const int chain = blk * CPB + cb;
+  const bool active = chain < Pr.n_chains;
+  const uint32_t gchain = (uint32_t)(Pr.chain0 + chain);
+  const int k_own = wc * KW + lane / P;  // the step (of K) this lane evaluates
+  constexpr unsigned kAll = K == 32 ? 0xffffffffu : (1u << K) - 1u;
+  const R l2f = (R)Pr.l2f;
+  const int n_quotes = Pr.n_quotes, G = Pr.G, len = Pr.chain_len, n_levels = Pr.n_levels;
+  const int units = StaticPoint<R, MODEL>::kPair ? (n_quotes + 1) >> 1 : n_quotes;
+  const LaneSplit ls = lane_split(G, P);
+  const uint32_t key0 = Pr.key0, key1 = Pr.key1;
+  // lane i & 3 forms coordinate i of the window's points
+  const int ci = lane & (D - 1);
+  Key lo[D], hi[D];
+  R x[D], bx[D];
+#pragma unroll
+  for (int i = 0; i < D; ++i) {
+    lo[i] = BoxKey<R>::of((R)Pr.lo[i]);
+    hi[i] = BoxKey<R>::of((R)Pr.hi[i]);
+    x[i] = (R)__ldcg(&Pr.state[i]);
+    bx[i] = x[i];
+  }
+  const double T0 = __ldcg(&Pr.state[kMaxD + 1]);
+  C fcur = cost_from(__ldcg(&Pr.state[kMaxD]), C{});
+  C bf = fcur;
+  unsigned long long ev_all = 0, ac_all = 0;
+  unsigned target = 0;
+  int parity = 0;
+  __syncthreads();
+
+  for (int level = 0; level < n_levels; ++level) {
+    // temperatures and step widths of the next kLevelCache levels, a level a
+    // lane of warp 0 (FP64 square roots and divisions, off the levels' path)
+    if ((level & (kLevelCache - 1)) == 0) {
+      if (warp == 0 && level + lane < n_levels) {
+        const double Tk0 = __dmul_rn(T0, Pr.ck[level + lane]);
+        double sk = __dmul_rn(Pr.step0, __dsqrt_rn(__ddiv_rn(Tk0, T0)));
+        if (sk < Pr.step_min) sk = Pr.step_min;
+        for (int i = 0; i < D; ++i) s_step[lane][i] = (R)__dmul_rn(sk, __dsub_rn(Pr.hi[i], Pr.lo[i]));
+        s_Tk[lane] = Tk0;
+        s_invTk[lane] = (float)(1.4426950408889634 / Tk0);
+      }
+      __syncthreads();
+    }
+    if (active) {
+      const R step = s_step[level & (kLevelCache - 1)][ci];
+      const float inv_Tk = s_invTk[level & (kLevelCache - 1)];
+      const double Tk = s_Tk[level & (kLevelCache - 1)];
+      unsigned ev = 0, ac = 0;
+      int filled = 0;  // steps whose words are in the ring
+      int st = 0;
+      while (st < len) {
+        if (filled < len && filled < st + K) {
+          const int s = filled + lane;
+          const uint4 w = philox4x32_10(make_uint4(gchain, (uint32_t)level, (uint32_t)s, kTagSA), key0, key1);
+          __syncwarp();  // every lane has read the entries that are replaced
+          s_w[warp][0][s & (kRing - 1)] = 2.0f * u01<float>(w.x) - 1.0f;
+          s_w[warp][1][s & (kRing - 1)] = 2.0f * u01<float>(w.y) - 1.0f;
+          s_w[warp][2][s & (kRing - 1)] = 2.0f * u01<float>(w.z) - 1.0f;
+          s_w[warp][3][s & (kRing - 1)] = 2.0f * u01<float>(w.w) - 1.0f;
+          s_u[warp][s & (kRing - 1)] = u01<float>(sa_accept_word(w.x, w.y, w.z));
+          filled += 32;
+          __syncwarp();
+        }
+        const int nv = len - st < K ? len - st : K;  // steps of this window
+        const unsigned window = nv == K ? kAll : (1u << nv) - 1u;
+        // the window's points if every proposal inside the box is accepted;
+        // one found outside (skip) is rejected for certain, and the points
+        // after it start from the one before it
+        unsigned skip = 0, out;
+        R xi0 = x[0];
+#pragma unroll
+        for (int i = 1; i < D; ++i) xi0 = ci == i ? x[i] : xi0;
+        R w[K];
+#pragma unroll
+        for (int j = 0; j < K; ++j) w[j] = word_to(s_w[warp][ci][(st + j) & (kRing - 1)], R{});
+        do {
+          R cur = xi0;
+#pragma unroll
+          for (int j = 0; j < K; ++j) {
+            const R y = move_by(cur, step, w[j]);
+            if (lane < D) s_x[warp][j][ci] = y;
+            cur = (skip >> j) & 1u ? cur : y;
+          }
+          __syncwarp();
+          const R* y = s_x[warp][K == 32 ? lane : (lane & (K - 1))];
+          bool in = true;
+#pragma unroll
+          for (int i = 0; i < D; ++i) {
+            const Key v = BoxKey<R>::of(y[i]);
+            in = in && !(v < lo[i] || v > hi[i]);
+          }
+          out = ~__ballot_sync(0xffffffffu, in) & window & ~skip;
+          skip |= out & (0u - out);
+        } while (out);
+        const unsigned in_mask = window & ~skip;
+        unsigned rej = 0;
+        if (in_mask) {
+          R xs[D];
+#pragma unroll
+          for (int i = 0; i < D; ++i) xs[i] = s_x[warp][k_own][i];
+          const C fo = point_cost<R, MODEL>(xs, n_quotes, units, l2f, sq, G, ls);
+          C* fb = s_f[cb][parity];
+          parity ^= 1;
+          if ((lane & (P - 1)) == 0) fb[k_own] = fo;
+          chain_sync<NW>(cb);
+          // lane k decides step k
+          const int k = lane & (K - 1);
+          const C f = fb[k];
+          const unsigned before = in_mask & ((1u << k) - 1u);  // the nearest earlier step inside the box
+          const C fe = fb[before ? 31 - __clz(before) : 0];
+          const C fp = before ? fe : fcur;
+          const auto delta = cost_delta(f, fp);
+          const R u = word_to(s_u[warp][(st + k) & (kRing - 1)], R{});
+          const bool acc = delta <= 0 || metropolis(u, delta, inv_Tk, Tk);
+          rej = __ballot_sync(0xffffffffu, !acc) & in_mask;
+          const int first = __ffs(rej) - 1;  // the first rejected step
+          const unsigned eval = rej ? in_mask & ((2u << first) - 1u) : in_mask;
+          const unsigned taken = rej ? eval & ~(1u << first) : eval;
+          ev += __popc(eval);
+          ac += __popc(taken);
+          unsigned better = __ballot_sync(0xffffffffu, cost_less(f, bf)) & eval;
+          if (better) {
+            int at = 0;
+            while (better) {
+              const int l = __ffs(better) - 1;
+              better &= better - 1u;
+              if (cost_less(fb[l], bf)) {
+                bf = fb[l];
+                at = l;
+              }
+            }
+#pragma unroll
+            for (int i = 0; i < D; ++i) bx[i] = s_x[warp][at][i];
+          }
+          if (taken) {
+            const int last = 31 - __clz(taken);
+            fcur = fb[last];
+#pragma unroll
+            for (int i = 0; i < D; ++i) x[i] = s_x[warp][last][i];
+          }
+          st += rej ? first + 1 : nv;
+        } else {
+          st += nv;
+        }
+        __syncwarp();  // the points are read before the next window's are written
+      }
+      ev_all += ev;
+      ac_all += ac;
+    }
+    // ---- level end: argmin over the chains of the problem ----------------
+    if (wc == 0 && lane == 0) {
+      s_mf[cb] = active ? cost_to_double(fcur) : INFINITY;
+#pragma unroll
+      for (int i = 0; i < D; ++i) s_mx[cb][i] = (double)x[i];
+    }
+    __syncthreads();
+    target += (unsigned)nb;
+    if (warp == 0) {
+      double* mf = Pr.part_f + (size_t)(level & 1) * nb;
+      int* mc = Pr.part_c + (size_t)(level & 1) * nb;
+      double* mx = Pr.part_x + (size_t)(level & 1) * nb * kMaxD;
+      double f = INFINITY;
+      int w = 0x7fffffff;
+      for (int i = 0; i < CPB; ++i) argmin_merge(f, w, s_mf[i], i);
+      if (w >= CPB) w = 0;  // no cost compares
+      if (lane < D) __stcg(&mx[(size_t)blk * kMaxD + lane], s_mx[w][lane]);
+      if (lane == D) __stcg(&mf[blk], f);
+      if (lane == D + 1) __stcg(&mc[blk], blk * CPB + w);
+      __threadfence();
+      __syncwarp();
+      if (lane == 0) {
+        atomicAdd(Pr.arrive, 1u);
+        volatile unsigned int* ctr = Pr.arrive;
+        volatile unsigned int* err = Pr.arrive + 1;
+        bool ok = *ctr >= target;
+        if (!ok) {
+          const unsigned long long t0 = global_ns();
+          while (!(ok = *ctr >= target)) {
+            if (*err) break;
+            if (global_ns() - t0 > wait_ns) {
+              atomicExch(Pr.arrive + 1, 1u);
+              break;
+            }
+          }
+        }
+        s_stop = !ok;
+        __threadfence();
+      }
+      __syncwarp();
+      if (!s_stop) {
+        double g = INFINITY;
+        int b = 0x7fffffff;
+        for (int i = lane; i < nb; i += 32) argmin_merge(g, b, __ldcg(&mf[i]), i);
+        warp_argmin(g, b);
+        if (b >= nb) b = 0;
+        if (lane < D) s_new[lane] = __ldcg(&mx[(size_t)b * kMaxD + lane]);
+        if (lane == D) s_new[D] = g;
+        if (blk == 0 && level + 1 == n_levels) {
+          if (lane < kMaxD) Pr.state[lane] = lane < D ? __ldcg(&mx[(size_t)b * kMaxD + lane]) : 0.0;
+          if (lane == 0) {
+            Pr.state[kMaxD] = g;
+            Pr.state[kStateArgChain] = (double)(Pr.chain0 + __ldcg(&mc[b]));
+          }
+        }
+      }
+    }
+    __syncthreads();
+    if (s_stop) return;
+#pragma unroll
+    for (int i = 0; i < D; ++i) x[i] = (R)s_new[i];
+    fcur = cost_from(s_new[D], C{});
+  }
+  if (n_levels > 0 && active && wc == 0 && lane == 0) {
+    Pr.chain_bf[chain] = cost_to_double(bf);
+    Pr.chain_ev[chain] = ev_all;
+    Pr.chain_ac[chain] = ac_all;
+    R* row = (R*)Pr.chain_bx + (size_t)chain * kMaxD;
+#pragma unroll
+    for (int i = 0; i < kMaxD; ++i) row[i] = i < D ? bx[i < D ? i : 0] : (R)0;
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Host side
+// ---------------------------------------------------------------------------
+bool small_supported(int prec, int model) {
+  return model == SABR_HAGAN || model == SABR_OBLOJ || (model == SABR_EXPANDED && prec == SABR_FP64);
+}
+
+// FP32, ms per calibration on 152 SMs (level kernels and queue | shape chosen):
+//   64 chains, 15 quotes, 200 x 100: 15.6 | 4 warps x 4 points 3.95 (4 x 2 4.11, 2 x 4 4.16, 1 x 4 5.65)
+//   503 chains, 350 quotes, 28 x 97: 6.45 | 4 x 2 3.51 (4 x 4 4.98, 2 x 2 4.05, 1 x 2 5.85)
+//   1000 chains, 11 quotes, 50 x 50: 2.65 | 1 x 4 1.18 (1 x 2 1.52, 2 x 4 1.23)
+//   1024 chains, 200 quotes, 40 x 50: 3.21 | 1 x 4 2.16 (1 x 2 2.17, 2 x 4 2.38)
+// A point too deep costs evaluations that are dropped, so few quotes take the
+// deeper window.  FP64, whose time is FP64 instructions a scheduler: two
+// points a warp, as many warps a chain as give every scheduler one (64 chains,
+// 15 quotes, 200 x 100: 173.9 | 4 x 2 33.5; 4 x 4 40.1, 2 x 2 48.7, 1 x 2 80.2).
+SmallShape small_shape(int prec, int n_quotes, long long chains) {
+  const long long sms = device_sms();
+  if (prec == SABR_FP64) return SmallShape{chains <= sms ? 4 : (chains <= 2 * sms ? 2 : 1), 2};
+  if (chains <= sms && n_quotes <= 64) return SmallShape{4, 4};
+  if (chains <= 4 * sms) return SmallShape{4, 2};
+  return SmallShape{1, 4};
+}
+long long small_most_chains(int prec) { return (prec == SABR_FP64 ? 4 : 8) * (long long)device_sms(); }
+
+int small_blocks(const SmallShape& s, int n_chains) {
+  const int cpb = kSmallBlock / 32 / s.nw;
+  return (n_chains + cpb - 1) / cpb;
+}
+
+size_t small_smem_bytes(int prec, int model, int Q, int M) { return level_smem_bytes(prec, model, Q, M, 1); }
+
+using SmallFn = void (*)(const ProblemDev*, const int4*, unsigned long long);
+template <int MODEL> static SmallFn small_fn_fp32(const SmallShape& s) {
+  if (s.nw == 1) return sa_small_kernel<float, MODEL, 1, 4>;
+  return s.kw == 4 ? sa_small_kernel<float, MODEL, 4, 4> : sa_small_kernel<float, MODEL, 4, 2>;
+}
+template <int MODEL> static SmallFn small_fn_fp64(const SmallShape& s) {
+  if (s.nw == 1) return sa_small_kernel<double, MODEL, 1, 2>;
+  return s.nw == 2 ? sa_small_kernel<double, MODEL, 2, 2> : sa_small_kernel<double, MODEL, 4, 2>;
+}
+static SmallFn small_fn(int prec, int model, const SmallShape& s) {
+  if (prec == SABR_FP32) return model == SABR_HAGAN ? small_fn_fp32<SABR_HAGAN>(s) : small_fn_fp32<SABR_OBLOJ>(s);
+  switch (model) {
+    case SABR_HAGAN: return small_fn_fp64<SABR_HAGAN>(s);
+    case SABR_OBLOJ: return small_fn_fp64<SABR_OBLOJ>(s);
+    default: return small_fn_fp64<SABR_EXPANDED>(s);
+  }
+}
+
+int small_capacity(int prec, int model, const SmallShape& s, size_t smem) {
+  const SmallFn fn = small_fn(prec, model, s);
+  cudaFuncAttributes at;
+  if (cudaFuncGetAttributes(&at, (const void*)fn) != cudaSuccess) return 0;
+  if (smem + at.sharedSizeBytes > 227 * 1024 ||
+      cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    return 0;
+  int nb = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, (const void*)fn, kSmallBlock, smem) != cudaSuccess) return 0;
+  return nb * device_sms();
+}
+
+cudaError_t launch_small(int prec, int model, const SmallShape& shape, const ProblemDev* probs, const int4* work,
+                         int blocks, size_t smem, unsigned long long wait_ns, cudaStream_t s) {
+  void* args[] = {&probs, &work, &wait_ns};
+  return cudaLaunchCooperativeKernel((const void*)small_fn(prec, model, shape), dim3(blocks), dim3(kSmallBlock), args,
+                                     smem, s);
+}
+
+}  // namespace sabr

@@ -27,7 +27,10 @@ constexpr int kStateArgChain = 12, kStateBestChain = 13;
 struct ProblemDev {
   int model, prec, cost, d;
   int n_quotes, n_mats, n_chains, n_levels;
-  int chain_len, G, cpb, n_blocks;
+  int chain_len;
+  int G;               // lanes by whose order a misfit is summed
+  int L;               // lanes that run a chain (L <= G, or L = G)
+  int cpb, n_blocks;   // chains per level block, level blocks
   double fwd, l2f, Tmax;
   double lo[10], hi[10];
   double T0_given, step0, step_min;
@@ -169,8 +172,7 @@ __device__ __forceinline__ DF lanes_sum(float v, int G, unsigned gmask) {
 // Shared-memory slots per maturity in a chain group's coefficient slice: the
 // polynomial (c0, c1, c2), and a fourth slot (for Case II it holds eta2^2
 // until the polynomial is formed) that aligns each polynomial to 16 bytes.
-// The FP32 Case II form also keeps, per maturity, the panel integrals its
-// term-structure rule sums (slots 4 .. 12 of a 16-slot stride).
+// The FP32 Case II form keeps a record of 16 floats (case2_group_coef_rule).
 template <class R, int MODEL> struct CoefStride {
   static constexpr int value = (MODEL == SABR_DYN_II && sizeof(R) == 4) ? 16 : 4;
 };
@@ -403,6 +405,257 @@ __device__ __forceinline__ void group_costn_hagan(const R (&xs)[SD][4], int n_qu
   for (int k = 0; k < SD; ++k) fs[k] = lanes_sum(acc[k], G, gmask);
 }
 
+// ---------------------------------------------------------------------------
+// A misfit is summed in the order that G lanes give it: virtual lane v adds
+// units (quotes, or pairs of quotes) v, v + G, ..., and a butterfly adds the
+// virtual lanes.  Any pe <= G lanes (a power of two) can play them: lane p
+// those of index p, p + pe, ..., so that the butterfly's first levels are
+// additions within the lane, and the sum is the same bit for bit whatever pe.
+// ---------------------------------------------------------------------------
+struct LaneSplit {
+  int pe, V, shift;  // lanes that differ, virtual lanes of each, 32 - log2 V
+};
+__device__ __forceinline__ LaneSplit lane_split(int G, int P) {
+  LaneSplit s;
+  s.pe = G < P ? G : P;
+  s.V = G / s.pe;
+  s.shift = 32 - (31 - __clz(s.V));
+  return s;
+}
+__device__ __forceinline__ double cost_xor(double v, int off, unsigned mask) { return __shfl_xor_sync(mask, v, off); }
+__device__ __forceinline__ DF cost_xor(DF v, int off, unsigned mask) {
+  return DF{__shfl_xor_sync(mask, v.hi, off), __shfl_xor_sync(mask, v.lo, off)};
+}
+__device__ __forceinline__ double cost_add(double a, double b) { return a + b; }
+__device__ __forceinline__ DF cost_add(DF a, DF b) { return df_add(a, b); }
+// the first level of a sum: df_add of (a, 0) and (b, 0) is the exact sum
+__device__ __forceinline__ double cost_add_first(double a, double b) { return a + b; }
+__device__ __forceinline__ DF cost_add_first(float a, float b) { return df_two_sum(a, b); }
+__device__ __forceinline__ double lane_cost(double v) { return v; }
+__device__ __forceinline__ DF lane_cost(float v) { return DF{v, 0.0f}; }
+
+// pt.partials<N>(v, units, G, sq, out): the sums of N virtual lanes v.
+template <class R, class Point>
+__device__ __forceinline__ typename CostOf<R>::T virtual_lanes_sum(const Point& pt, int units, int G,
+                                                                   const LaneSplit& ls, const SmemQuotes<R>& sq,
+                                                                   unsigned mask) {
+  using C = typename CostOf<R>::T;
+  const int p = threadIdx.x & (ls.pe - 1);
+  C s;
+  int off = ls.pe >> 1;
+  if (ls.V == 1) {
+    const int v[1] = {p};
+    R a[1];
+    pt.template partials<1>(v, units, G, sq, a);
+    if (off > 0) {
+      s = cost_add_first(a[0], __shfl_xor_sync(mask, a[0], off));
+      off >>= 1;
+    } else {
+      s = lane_cost(a[0]);
+    }
+  } else {
+    // the butterfly starts with the farthest pairs: lanes are added in the
+    // order of their bit-reversed index, a binary counter holding the
+    // finished subtrees
+    C stack[5];
+#pragma unroll
+    for (int l = 0; l < 5; ++l) stack[l] = s = lane_cost((R)0);
+    for (int t = 0; t < ls.V; t += 2) {
+      const int i = (int)(__brev((unsigned)t) >> ls.shift);  // bit 0 of t is the farthest pair
+      const int v[2] = {p + ls.pe * i, p + ls.pe * (i + (ls.V >> 1))};
+      R a[2];
+      pt.template partials<2>(v, units, G, sq, a);
+      s = cost_add_first(a[0], a[1]);
+      bool carry = true;
+#pragma unroll
+      for (int l = 1; l < 5; ++l) {
+        if (carry) {
+          carry = ((t >> l) & 1) != 0;
+          if (carry) {
+            s = cost_add(stack[l], s);
+          } else {
+            stack[l] = s;
+          }
+        }
+      }
+    }
+  }
+  for (; off > 0; off >>= 1) s = cost_add(s, cost_xor(s, off, mask));
+  return s;
+}
+
+// One static formula at one point: constants, and the unit residuals.  A unit
+// is a quote, or for FP32 Hagan a pair of quotes (float2).
+template <class R, int MODEL> struct StaticPoint {
+  static constexpr bool kPair = MODEL == SABR_HAGAN && sizeof(R) == 4;
+  StaticConst<R> sc;
+  PolyCoef<R> c0;
+  R bw;
+  int n_quotes;
+  __device__ __forceinline__ StaticPoint(const R* x, R l2f, int nq) : n_quotes(nq) {
+    if constexpr (MODEL == SABR_EXPANDED) {
+      c0 = expanded_coef<R>(x, l2f, (R)0);
+      bw = expanded_coef<R>(x, l2f, (R)1).c0 - c0.c0;
+    } else {
+      sc = static_setup<R>(x);
+    }
+  }
+  __device__ __forceinline__ R resid_of(int q, const SmemQuotes<R>& sq) const {
+    const QuotePack<R> qp = sq.pack[q];
+    R vol;
+    if constexpr (MODEL == SABR_HAGAN) {
+      vol = vol_hagan<R>(sc, qp.lfk, qp.l2kf, qp.T);
+    } else if constexpr (MODEL == SABR_OBLOJ) {
+      vol = vol_obloj<R>(sc, qp.lfk, qp.l2kf, sq.l2k[q], qp.T);
+    } else {
+      PolyCoef<R> c = c0;
+      c.c0 = c0.c0 + bw * qp.T;
+      vol = vol_poly<R>(c, qp.lfk);
+    }
+    return resid(vol, qp.w);
+  }
+  __device__ __forceinline__ float2 resid_pair_of(int j, const SmemQuotes<R>& sq) const {
+    const float4 a = sq.pair[2 * j], b = sq.pair[2 * j + 1];
+    return hagan_resid_pair(sc, make_float2(a.x, a.y), make_float2(a.z, a.w), make_float2(b.x, b.y),
+                            make_float2(b.z, b.w), make_float2(1.0f, 2 * j + 1 < n_quotes ? 1.0f : 0.0f));
+  }
+  // sums of N virtual lanes v[0..N-1], the lanes' units side by side.  A unit
+  // past the end is evaluated as unit 0 and counts 0 (adding 0 changes no sum).
+  template <int N>
+  __device__ __forceinline__ void partials(const int (&v)[N], int units, int G, const SmemQuotes<R>& sq,
+                                           R (&out)[N]) const {
+    if constexpr (kPair) {
+      float2 acc[N];
+#pragma unroll
+      for (int k = 0; k < N; ++k) acc[k] = make_float2(0.0f, 0.0f);
+      for (int j0 = 0; j0 < units; j0 += G) {
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+          const bool on = j0 + v[k] < units;
+          float2 r = resid_pair_of(on ? j0 + v[k] : 0, sq);
+          r.x = on ? r.x : 0.0f;
+          r.y = on ? r.y : 0.0f;
+          acc[k] = fma2(r, r, acc[k]);
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < N; ++k) out[k] = acc[k].x + acc[k].y;
+    } else {
+#pragma unroll
+      for (int k = 0; k < N; ++k) out[k] = (R)0;
+      for (int j0 = 0; j0 < units; j0 += G) {
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+          const bool on = j0 + v[k] < units;
+          R r = resid_of(on ? j0 + v[k] : 0, sq);
+          r = on ? r : (R)0;
+          out[k] += r * r;
+        }
+      }
+    }
+  }
+};
+
+// A dynamic model's point in FP32: the polynomials of its maturities, records
+// of CS floats in the chain's slice of shared memory.
+template <int CS> struct DynPoint {
+  const float* coef;
+  __device__ __forceinline__ float resid_of(int q, const SmemQuotes<float>& sq) const {
+    const QuotePack<float> qp = sq.pack[q];
+    const float4 c = *reinterpret_cast<const float4*>(coef + CS * mat_of_slot(qp.l2kf));
+    return resid(vol_poly<float>(PolyCoef<float>{c.x, c.y, c.z}, qp.lfk), qp.w);
+  }
+  // Rounds in chunks, so that the loads of several quotes are in flight (a
+  // quote's polynomial is addressed by its pack: two dependent shared-memory
+  // loads, a few FMAs); a chunk's residuals join the sums in order.
+  template <int N>
+  __device__ __forceinline__ void partials(const int (&v)[N], int n_quotes, int G, const SmemQuotes<float>& sq,
+                                           float (&out)[N]) const {
+    constexpr int U = 8 / N;
+#pragma unroll
+    for (int k = 0; k < N; ++k) out[k] = 0.0f;
+    int q0 = 0;
+    for (; q0 + U * G <= n_quotes; q0 += U * G) {
+      float r[U][N];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int k = 0; k < N; ++k) r[u][k] = resid_of(q0 + u * G + v[k], sq);
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int k = 0; k < N; ++k) out[k] += r[u][k] * r[u][k];
+    }
+    for (; q0 < n_quotes; q0 += G) {
+#pragma unroll
+      for (int k = 0; k < N; ++k) {
+        const bool on = q0 + v[k] < n_quotes;
+        float r = resid_of(on ? q0 + v[k] : 0, sq);
+        r = on ? r : 0.0f;
+        out[k] += r * r;
+      }
+    }
+  }
+};
+
+// Elements from one chain's slice to the next: an odd number of records of
+// four, so that the slices of a warp's chains start in different banks and the
+// chains' loads of a record do not collide.
+__host__ __device__ constexpr int coef_slice(int prec, int model, int n_mats) {
+  const int n = coef_stride(prec, model) * n_mats;
+  return (model == SABR_DYN_I || model == SABR_DYN_II) ? n + ((n / 4) % 2 == 0 ? 4 : 0) : 0;
+}
+
+// Exclusive scan of the panels' int nu rho (slot 10 of their records) in
+// rounds of VL = E L panels, Hillis-Steele within a round as VL lanes would run
+// it: lane l holds the round's elements l, l + L, ... (E of them).  Leaves the
+// integrals of G^2 in slots 11 and 12.
+template <int E>
+__device__ __forceinline__ void case2_panel_starts(int n_mats, float* rec, int lane, int L, unsigned mask) {
+  constexpr int CS = 16;
+  const int VL = E * L;
+  float carry = 0.0f;  // G at the start of the round's first panel
+  for (int r0 = 0; r0 < n_mats; r0 += VL) {
+    float n[E], in[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const int j = r0 + lane + L * e;
+      n[e] = j < n_mats ? rec[CS * j + 10] : 0.0f;
+      in[e] = n[e];
+    }
+    for (int off = 1; off < L; off <<= 1) {
+      // element l - off: the same element of lane - off, or the one before of
+      // the lane it wraps to
+      float prev = 0.0f, y[E];
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const float v = __shfl_sync(mask, in[e], (lane - off) & (L - 1), L);
+        y[e] = lane >= off ? v : prev;
+        prev = v;
+      }
+#pragma unroll
+      for (int e = 0; e < E; ++e) in[e] = lane >= off || e > 0 ? in[e] + y[e] : in[e];
+    }
+#pragma unroll
+    for (int d = 1; d < E; d <<= 1) {
+#pragma unroll
+      for (int e = E - 1; e >= d; --e) in[e] += in[e - d];
+    }
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const int j = r0 + lane + L * e;
+      if (j < n_mats) {
+        const float Gs = carry + (in[e] - n[e]);
+        float* r = rec + CS * j;
+        const float4 q = *reinterpret_cast<const float4*>(r);
+        r[12] = fmaf(Gs, fmaf(Gs, r[13], 2.0f * q.x), q.y);  // int G^2 over the panel
+        r[11] = fmaf(Gs, fmaf(Gs, r[14], 2.0f * q.z), q.w);  // int (T_j - t) G^2
+      }
+    }
+    carry += __shfl_sync(mask, in[E - 1], L - 1, L);
+  }
+}
+
 // FP32 Case II: the four functions of eq. (integrales_SABRd) of every
 // maturity from one composite rule over [0, Tmax] whose panels end at the
 // maturities (sub-panels and nodes prepared per problem, case2_rule_build).
@@ -414,120 +667,156 @@ __device__ __forceinline__ void group_costn_hagan(const R (&xs)[SD][4], int n_qu
 // its own integrals with weights in T_j - t; across panels the totals obey
 // positive recurrences in Delta = T_j - T_{j-1} (e.g. A_j = A_{j-1} +
 // Delta (2 B_{j-1} + Delta C_{j-1}) + a_j with B = int (T-t) nu^2,
-// C = int nu^2), so no difference of large terms is formed.  Lanes take
-// whole panels (maturity j on lane j mod G); at a node only nu and rho are
-// evaluated (two 2^x), G inside a sub-panel comes from the Gauss-Legendre
-// integration matrix, and G at a panel's start from a scan over the lanes.
-// With G = G_start + g(t), the panel's integrals of G^2 are kept as
-// coefficients of a quadratic in G_start (P0, P1, P2), so every node is
-// evaluated once.  `loc` holds 12 slots per maturity for the panel
-// integrals; coef[4 j ..] receives nu1^2, nu2^2, eta1, eta2^2 and then the
-// polynomial of maturity j.
+// C = int nu^2), so no difference of large terms is formed.
+//
+// A chain's L lanes take whole panels; at a node only nu and rho are evaluated
+// (two 2^x), G inside a sub-panel comes from the Gauss-Legendre integration
+// matrix, and G at a panel's start from a scan.  With G = G_start + g(t), the
+// panel's integrals of G^2 are kept as coefficients of a quadratic in G_start
+// (P0, P1, P2), so every node is evaluated once.  The scan is that of VL
+// lanes (rounds of VL panels, Hillis-Steele within a round), played by the L
+// lanes, so the sums do not depend on L.  The recurrences are four
+// independent ones -- (A, B, C), (D, E), (H, N), (K, I) -- and four lanes take
+// one each; then every lane forms the polynomials of its own maturities.
+//
+// A maturity's record (16 floats): [0..3] first P1, P2, Q1, Q2, then A, D, H,
+// K, then the polynomial; [4..6] a, b, c; [7..8] d, e; [9..10] h, n; [11..12]
+// int (T_j - t) G^2, int G^2 over the panel; [13..14] P0, Q0.
 __device__ __forceinline__ void case2_group_coef_rule(const float* xp, int n_mats, float l2f,
-                                                      const SmemQuotes<float>& sq, float* coef, float* loc, int lane,
-                                                      int G, unsigned gmask) {
+                                                      const SmemQuotes<float>& sq, float* rec, int lane, int L,
+                                                      int VL, unsigned gmask) {
+  constexpr int CS = 16;
   const float rho0 = xp[2], nu0 = xp[3], dr = xp[6], dn = xp[7], qr = xp[8], qn = xp[9];
   const float na2 = -xp[4] * 1.4426950408889634f, nb2 = -xp[5] * 1.4426950408889634f;
-  float carry = 0.0f;  // G at the start of this round's first panel
-  for (int r0 = 0; r0 < n_mats; r0 += G) {
-    const int j = r0 + lane;
+  for (int j = lane; j < n_mats; j += L) {
     float c_ = 0.f, e_ = 0.f, b_ = 0.f, a_ = 0.f, d_ = 0.f, n_ = 0.f, h_ = 0.f;
     float P0 = 0.f, P1 = 0.f, P2 = 0.f, Q0 = 0.f, Q1 = 0.f, Q2 = 0.f;
-    if (j < n_mats) {
-      const int2 pr = sq.c2_panel[j];
-      for (int sbi = pr.x; sbi < pr.x + pr.y; ++sbi) {
-        const float4 sub = sq.c2_sub[sbi];  // half width, sum W, sum tau W
-        const float cin = n_;               // int of nu rho from the panel start
-        const float4* nd = sq.c2_node + kC2Nodes * sbi;
-        float f[kC2Nodes];
+    const int2 pr = sq.c2_panel[j];
+    for (int sbi = pr.x; sbi < pr.x + pr.y; ++sbi) {
+      const float4 sub = sq.c2_sub[sbi];  // half width, sum W, sum tau W
+      const float cin = n_;               // int of nu rho from the panel start
+      const float4* nd = sq.c2_node + kC2Nodes * sbi;
+      float f[kC2Nodes];
 #pragma unroll
-        for (int k = 0; k < kC2Nodes; ++k) {
-          const float4 q = nd[k];  // u, W, tau
-          const float eb = ex2_approx(nb2 * q.x), ea = ex2_approx(na2 * q.x);
-          const float nu = fmaf(fmaf(qn, q.x, nu0), eb, dn);
-          const float rho = fmaf(fmaf(qr, q.x, rho0), ea, dr);
-          f[k] = nu * rho;
-          const float wn = q.y * nu * nu;
-          c_ += wn;
-          e_ = fmaf(q.x, wn, e_);
-          b_ = fmaf(q.z, wn, b_);
-          const float twn = q.z * wn;
-          a_ = fmaf(q.z, twn, a_);
-          d_ = fmaf(q.x, twn, d_);
-          const float wf = q.y * f[k];
-          n_ += wf;
-          h_ = fmaf(q.z, wf, h_);
-        }
-        float s1 = 0.f, s2 = 0.f, t1 = 0.f, t2 = 0.f;
-#pragma unroll
-        for (int k = 0; k < kC2Nodes; ++k) {
-          float g = 0.f;
-#pragma unroll
-          for (int i = 0; i < kC2Nodes; ++i) g = fmaf(kC2.S[k][i], f[i], g);
-          g *= sub.x;
-          const float4 q = nd[k];
-          const float wg = q.y * g, twg = q.z * wg;
-          s1 += wg;
-          s2 = fmaf(wg, g, s2);
-          t1 += twg;
-          t2 = fmaf(twg, g, t2);
-        }
-        // int W (Gs + cin + g)^2 as a quadratic in Gs, the G at the panel start
-        P0 += sub.y;
-        P1 += fmaf(cin, sub.y, s1);
-        P2 += fmaf(cin, fmaf(cin, sub.y, 2.0f * s1), s2);
-        Q0 += sub.z;
-        Q1 += fmaf(cin, sub.z, t1);
-        Q2 += fmaf(cin, fmaf(cin, sub.z, 2.0f * t1), t2);
+      for (int k = 0; k < kC2Nodes; ++k) {
+        const float4 q = nd[k];  // u, W, tau
+        const float eb = ex2_approx(nb2 * q.x), ea = ex2_approx(na2 * q.x);
+        const float nu = fmaf(fmaf(qn, q.x, nu0), eb, dn);
+        const float rho = fmaf(fmaf(qr, q.x, rho0), ea, dr);
+        f[k] = nu * rho;
+        const float wn = q.y * nu * nu;
+        c_ += wn;
+        e_ = fmaf(q.x, wn, e_);
+        b_ = fmaf(q.z, wn, b_);
+        const float twn = q.z * wn;
+        a_ = fmaf(q.z, twn, a_);
+        d_ = fmaf(q.x, twn, d_);
+        const float wf = q.y * f[k];
+        n_ += wf;
+        h_ = fmaf(q.z, wf, h_);
       }
+      float s1 = 0.f, s2 = 0.f, t1 = 0.f, t2 = 0.f;
+#pragma unroll
+      for (int k = 0; k < kC2Nodes; ++k) {
+        float g = 0.f;
+#pragma unroll
+        for (int i = 0; i < kC2Nodes; ++i) g = fmaf(kC2.S[k][i], f[i], g);
+        g *= sub.x;
+        const float4 q = nd[k];
+        const float wg = q.y * g, twg = q.z * wg;
+        s1 += wg;
+        s2 = fmaf(wg, g, s2);
+        t1 += twg;
+        t2 = fmaf(twg, g, t2);
+      }
+      // int W (Gs + cin + g)^2 as a quadratic in Gs, the G at the panel start
+      P0 += sub.y;
+      P1 += fmaf(cin, sub.y, s1);
+      P2 += fmaf(cin, fmaf(cin, sub.y, 2.0f * s1), s2);
+      Q0 += sub.z;
+      Q1 += fmaf(cin, sub.z, t1);
+      Q2 += fmaf(cin, fmaf(cin, sub.z, 2.0f * t1), t2);
     }
-    // G at each panel's start: exclusive scan of the panels' int nu rho
-    float incl = n_;
-    for (int off = 1; off < G; off <<= 1) {
-      const float y = __shfl_up_sync(gmask, incl, off, G);
-      if (lane >= off) incl += y;
-    }
-    const float Gs = carry + (incl - n_);
-    carry += __shfl_sync(gmask, incl, G - 1, G);
-    if (j < n_mats) {
-      float* L = loc + 12 * j;
-      L[0] = c_;
-      L[1] = e_;
-      L[2] = b_;
-      L[3] = a_;
-      L[4] = d_;
-      L[5] = n_;
-      L[6] = h_;
-      L[7] = fmaf(Gs, fmaf(Gs, P0, 2.0f * P1), P2);  // int G^2 over the panel
-      L[8] = fmaf(Gs, fmaf(Gs, Q0, 2.0f * Q1), Q2);  // int (T_j - t) G^2
+    float4* r = reinterpret_cast<float4*>(rec + CS * j);
+    r[0] = make_float4(P1, P2, Q1, Q2);
+    r[1] = make_float4(a_, b_, c_, d_);
+    r[2] = make_float4(e_, h_, n_, 0.0f);
+    rec[CS * j + 13] = P0;
+    rec[CS * j + 14] = Q0;
+  }
+  __syncwarp(gmask);
+  // G at each panel's start
+  switch (VL / L) {
+    case 1: case2_panel_starts<1>(n_mats, rec, lane, L, gmask); break;
+    case 2: case2_panel_starts<2>(n_mats, rec, lane, L, gmask); break;
+    case 4: case2_panel_starts<4>(n_mats, rec, lane, L, gmask); break;
+    default: case2_panel_starts<8>(n_mats, rec, lane, L, gmask); break;
+  }
+  __syncwarp(gmask);
+  // the recurrences X += Delta (m Y + Delta Z) + x, Y += Delta Z + y, Z += z
+  // (Z = 0 and m = 1 but for A), one a lane; the running X goes to the record
+  for (int role = lane; role < 4; role += L) {
+    const int ox = role == 0 ? 4 : (role == 1 ? 7 : (role == 2 ? 9 : 11));
+    const int oy = role == 0 ? 5 : (role == 1 ? 8 : (role == 2 ? 10 : 12));
+    const float m = role == 0 ? 2.0f : 1.0f;
+    float X = 0.f, Y = 0.f, Z = 0.f, Tp = 0.f;
+#pragma unroll 2
+    for (int j = 0; j < n_mats; ++j) {
+      const float T = sq.mT[j], dl = T - Tp;
+      const float* r = rec + CS * j;
+      const float x = r[ox], y = r[oy], z = role == 0 ? r[6] : 0.0f;
+      X += fmaf(dl, fmaf(dl, Z, m * Y), x);
+      Y += fmaf(dl, Z, y);
+      Z += z;
+      Tp = T;
+      rec[CS * j + role] = X;
     }
   }
   __syncwarp(gmask);
-  // the recurrences over the panels (every lane runs them; lane j mod G
-  // forms maturity j's functions and polynomial)
-  float C = 0.f, E = 0.f, B = 0.f, A = 0.f, D = 0.f, N = 0.f, H = 0.f, I = 0.f, K = 0.f, Tp = 0.f;
-  for (int j = 0; j < n_mats; ++j) {
-    const float T = sq.mT[j], dl = T - Tp;
-    const float* L = loc + 12 * j;
-    A += fmaf(dl, fmaf(dl, C, 2.0f * B), L[3]);
-    B += fmaf(dl, C, L[2]);
-    C += L[0];
-    D += fmaf(dl, E, L[4]);
-    E += L[1];
-    H += fmaf(dl, N, L[6]);
-    N += L[5];
-    K += fmaf(dl, I, L[8]);
-    I += L[7];
-    Tp = T;
-    if ((j & (G - 1)) == lane) {
-      const float iT = rcp_approx(T), iT2 = iT * iT;
-      const PolyCoef<float> c = dynamic_poly<float>(xp[0], xp[1], l2f, T, 3.0f * A * iT2 * iT, 6.0f * D * iT2 * iT,
-                                                    2.0f * H * iT2, 12.0f * K * iT2 * iT2);
-      coef[4 * j + 0] = c.c0;
-      coef[4 * j + 1] = c.c1;
-      coef[4 * j + 2] = c.c2;
-    }
+  for (int j = lane; j < n_mats; j += L) {
+    const float T = sq.mT[j];
+    float4* r = reinterpret_cast<float4*>(rec + CS * j);
+    const float4 v = *r;  // A, D, H, K
+    const float iT = rcp_approx(T), iT2 = iT * iT;
+    const PolyCoef<float> c = dynamic_poly<float>(xp[0], xp[1], l2f, T, 3.0f * v.x * iT2 * iT, 6.0f * v.y * iT2 * iT,
+                                                  2.0f * v.z * iT2, 12.0f * v.w * iT2 * iT2);
+    *r = make_float4(c.c0, c.c1, c.c2, 0.0f);
   }
+}
+
+// The misfit of a dynamic model's point in FP32 by the L lanes of a chain:
+// the polynomials of its maturities into the chain's slice `rec`, then the
+// quotes.
+template <int MODEL>
+__device__ __forceinline__ DF dynamic_cost_f32(const float* xp, int n_quotes, int n_mats, float l2f,
+                                               const SmemQuotes<float>& sq, float* rec, int lane, int L, int G,
+                                               unsigned gmask) {
+  constexpr int CS = CoefStride<float, MODEL>::value;
+  if constexpr (MODEL == SABR_DYN_I) {
+    // three maturities a lane side by side while every lane has three (12
+    // maturities on four lanes), then one at a time
+    int r0 = 0;
+    for (; r0 + 3 * L <= n_mats; r0 += 3 * L) {
+      PolyCoef<float> c[3];
+#pragma unroll
+      for (int u = 0; u < 3; ++u) c[u] = dynamic_coef<float, false>(xp, l2f, sq.mT[r0 + u * L + lane]);
+#pragma unroll
+      for (int u = 0; u < 3; ++u)
+        *reinterpret_cast<float4*>(rec + CS * (r0 + u * L + lane)) = make_float4(c[u].c0, c[u].c1, c[u].c2, 0.0f);
+    }
+    for (; r0 < n_mats; r0 += L) {
+      const int j = r0 + lane;
+      const PolyCoef<float> c = dynamic_coef<float, false>(xp, l2f, sq.mT[j < n_mats ? j : 0]);
+      if (j < n_mats) *reinterpret_cast<float4*>(rec + CS * j) = make_float4(c.c0, c.c1, c.c2, 0.0f);
+    }
+  } else {
+    case2_group_coef_rule(xp, n_mats, l2f, sq, rec, lane, L, G, gmask);
+  }
+  __syncwarp(gmask);
+  const DynPoint<CS> pt{rec};
+  const DF f = virtual_lanes_sum<float>(pt, n_quotes, G, lane_split(G, L), sq, gmask);
+  __syncwarp(gmask);
+  return f;
 }
 
 // Cost of point xp evaluated by the G lanes of one chain group.  Lane `lane`
@@ -577,6 +866,7 @@ __device__ __forceinline__ typename CostOf<R>::T group_cost(const R* xp, int n_q
       acc += r * r;
     }
   } else {
+    if constexpr (sizeof(R) == 4) return dynamic_cost_f32<MODEL>(xp, n_quotes, n_mats, l2f, sq, coef, lane, G, G, gmask);
     constexpr int CS = 4;  // polynomial slots per maturity (load_poly)
     if (MODEL == SABR_DYN_I) {
       for (int j = lane; j < n_mats; j += G) {
@@ -585,9 +875,7 @@ __device__ __forceinline__ typename CostOf<R>::T group_cost(const R* xp, int n_q
         coef[CS * j + 1] = c.c1;
         coef[CS * j + 2] = c.c2;
       }
-    } else if constexpr (sizeof(R) == 4) {
-      case2_group_coef_rule(xp, n_mats, l2f, sq, coef, coef + 4 * n_mats, lane, G, gmask);
-    } else {
+    } else if constexpr (sizeof(R) == 8) {
       case2_group_coef<R>(xp, n_mats, l2f, sq, coef, lane, G, gmask);
     }
     __syncwarp(gmask);

@@ -36,6 +36,10 @@ sabr_status formula_prepare(const sabr_problem& pr, const sabr_bounds& b, const 
 // [1, 32]) sets it for every problem; results then differ only by the FP32
 // rounding of the lane sums.
 int choose_lanes(int n_quotes, int n_mats, int model, int prec, long long batch_chains);
+// Lanes that run a chain whose sums are in the order of G (at most G; blocks
+// of `block` threads).
+int choose_run_lanes(int n_quotes, int n_mats, int model, int prec, int G, long long batch_chains, int block);
+int server_run_lanes(int n_quotes, int n_mats, int model, int prec, int G);
 // Dynamic shared memory of a level block (cpb chains) / of an init block;
 // c2_nsub: sub-panels of the FP32 Case II rule (0 otherwise).
 size_t level_smem_bytes(int prec, int model, int Q, int M, int cpb, int c2_nsub = 0);
@@ -45,9 +49,10 @@ size_t init_smem_bytes(const HostProblem& h);
 // Lays out one problem's device region at [off0, end) of an arena: its
 // quotes, schedule, start point, chain state and block partials, filling d.
 // img == nullptr performs a dry run (offsets only).  Returns end.
-// `block`: threads per level block (chains per block = block / G).
+// `block`: threads per level block; L: lanes that run a chain (0: G).  Chains
+// per block = block / L.
 size_t formula_layout(const HostProblem& h, int G, unsigned char* img, unsigned char* base, size_t off0,
-                      ProblemDev& d, sabr_result* dres, int block = kSaBlock);
+                      ProblemDev& d, sabr_result* dres, int block = kSaBlock, int L = 0);
 
 // Kernel launches for (prec, model).
 void set_engine_smem(int prec, int model, size_t bytes);

@@ -121,6 +121,75 @@ __global__ void sa_init_kernel(const ProblemDev* __restrict__ probs, const int* 
 // ---------------------------------------------------------------------------
 // One temperature level for every chain of a launch group.
 // ---------------------------------------------------------------------------
+// The steps of one level of the chains of a warp, FP32, L lanes each, in
+// lockstep: every lane runs every instruction (full-warp masks; lanes whose
+// proposal is rejected unevaluated compute a cost that is dropped), so nothing
+// is set up per chain group around the exchanges.  cost(xp) is called by the
+// whole warp.
+template <int MODEL, int D, class Cost>
+__device__ __forceinline__ void lockstep_level(const ProblemDev& P, uint32_t gchain, int level, bool active, int lane,
+                                               int L, const float* s_lo, const float* s_hi, const float* s_step,
+                                               float inv_Tk, float Tmax, float (&x)[D], DF& fcur, DF& bf, float* cbx,
+                                               unsigned& ev, unsigned& ac, Cost&& cost) {
+  constexpr unsigned kWarp = 0xffffffffu;
+  constexpr int NB = sa_philox_blocks(D);
+  const int S = L >= NB ? L / NB : 1;  // steps per batch of Philox blocks
+  const uint32_t key0 = P.key0, key1 = P.key1;
+  const int first = (threadIdx.x & 31) & ~(L - 1);
+  const int my = lane < S * NB ? lane : 0;
+  const uint32_t my_step = (uint32_t)(my / NB), my_tag = kTagSA + (uint32_t)(my % NB);
+  uint4 wbuf = make_uint4(0u, 0u, 0u, 0u);
+  int s_ctr = 0;  // st mod S
+  for (int st = 0; st < P.chain_len; ++st) {
+    uint32_t wv[4 * NB];
+    if (L >= NB) {
+      if (s_ctr == 0) wbuf = philox4x32_10(make_uint4(gchain, (uint32_t)level, (uint32_t)st + my_step, my_tag), key0, key1);
+      const int base = first + s_ctr * NB;
+      s_ctr = s_ctr + 1 == S ? 0 : s_ctr + 1;
+#pragma unroll
+      for (int i = 0; i < D; ++i) {
+        const uint32_t word = (i & 3) == 0 ? wbuf.x : ((i & 3) == 1 ? wbuf.y : ((i & 3) == 2 ? wbuf.z : wbuf.w));
+        wv[i] = __shfl_sync(kWarp, word, base + (i >> 2));
+      }
+    } else {
+#pragma unroll
+      for (int b = 0; b < NB; ++b) {
+        const uint4 w =
+            philox4x32_10(make_uint4(gchain, (uint32_t)level, (uint32_t)st, kTagSA + (uint32_t)b), key0, key1);
+        wv[4 * b + 0] = w.x;
+        wv[4 * b + 1] = w.y;
+        wv[4 * b + 2] = w.z;
+        wv[4 * b + 3] = w.w;
+      }
+    }
+    const float ua = u01<float>(sa_accept_word(wv[0], wv[1], wv[2]));
+    float xp[D];
+    bool inside = active;
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+      xp[i] = propose(x[i], s_step[i], u01<float>(wv[i]));
+      inside = inside && !(xp[i] < s_lo[i] || xp[i] > s_hi[i]);
+    }
+    if (MODEL == SABR_DYN_II && inside) inside = case2_feasible<float>(xp, Tmax);
+    if (!__any_sync(kWarp, inside)) continue;
+    const DF fp = cost(xp);
+    ev += inside ? 1u : 0u;
+    const bool better = inside && cost_less(fp, bf);
+    const float delta = cost_delta(fp, fcur);
+    const float pacc = ex2_approx(-delta * inv_Tk);
+    const bool acc = inside && (delta <= 0.0f || ua < pacc);
+    bf = better ? fp : bf;
+    if (better && lane == 0) {
+#pragma unroll
+      for (int i = 0; i < D; ++i) cbx[i] = xp[i];
+    }
+#pragma unroll
+    for (int i = 0; i < D; ++i) x[i] = acc ? xp[i] : x[i];
+    fcur = acc ? fp : fcur;
+    ac += acc ? 1u : 0u;
+  }
+}
+
 // Block `blk` of problem P (staged in shared memory) runs level `level`.
 // Every thread of the block calls this.
 // Units of one problem may run on different blocks of one persistent launch,
@@ -128,31 +197,34 @@ __global__ void sa_init_kernel(const ProblemDev* __restrict__ probs, const int* 
 // counters, block minima) is read from L2 (ld.global.cg), never from a
 // possibly stale L1 line.  `q` (plans only) receives the units of the next
 // level when this block closes level `level` of problem `pid`.
-template <class R, int MODEL, int PAIRS = 2, bool SEL = false>
+// ONE (FP32 Hagan): every chain has one lane (G = L = 1); the forms for several
+// lanes are left out, which the register allocation of the one-lane loops,
+// the largest of the kernel, is sensitive to.
+template <class R, int MODEL, int PAIRS = 2, bool SEL = false, bool ONE = false>
 __device__ __forceinline__ void sa_level_block(const ProblemDev& P, int pid, int blk, int level, unsigned char* smem,
                                                const LevelQueue* q) {
   unsigned char* rest;
   const SmemQuotes<R> sq = stage_quotes<R>(P, smem, blockDim.x, threadIdx.x, &rest);
   constexpr int D = Dim<MODEL>::value;
-  const int G = P.G, cpb = P.cpb;
-  const int g = threadIdx.x / G, lane = threadIdx.x % G;
+  // L lanes run a chain; its misfit is summed in the order of G
+  const int G = ONE ? 1 : P.G, L = ONE ? 1 : P.L, cpb = ONE ? (int)blockDim.x : P.cpb;
+  const int g = threadIdx.x / L, lane = threadIdx.x % L;
   // per-maturity polynomial slices exist only for the dynamic models
-  const int coef_m = (MODEL == SABR_DYN_I || MODEL == SABR_DYN_II) ? P.n_mats : 0;
-  constexpr int CS = CoefStride<R, MODEL>::value;
-  R* coef = (R*)rest + (size_t)g * CS * coef_m;
-  double* red_f = (double*)(rest + ((((size_t)cpb * CS * coef_m + 16) * sizeof(R) + 15) & ~(size_t)15));
+  const int slice = coef_slice(sizeof(R) == 8 ? SABR_FP64 : SABR_FP32, MODEL, P.n_mats);
+  R* coef = (R*)rest + (size_t)g * slice;
+  double* red_f = (double*)(rest + ((((size_t)cpb * slice + 16) * sizeof(R) + 15) & ~(size_t)15));
   R* red_x = (R*)(red_f + cpb);
   __syncthreads();
 
   const int chain = blk * cpb + g;
   const bool active = chain < P.n_chains;
   const uint32_t gchain = (uint32_t)(P.chain0 + chain);  // Philox counter word 0
-  const unsigned gmask = group_mask(G);
+  const unsigned gmask = group_mask(L);
 
   // temperature, step widths and box of this level, formed once by thread 0
   // (FP64 division and square root issue at a small fraction of the FP32
   // rate) and shared by the block's chains
-  __shared__ R s_lo[kMaxD], s_hi[kMaxD], s_step[kMaxD];
+  __shared__ __align__(16) R s_lo[kMaxD + 2], s_hi[kMaxD + 2], s_step[kMaxD + 2];
   __shared__ double s_Tk;
   __shared__ float s_invTk;
   if (threadIdx.x == 0) {
@@ -194,7 +266,29 @@ __device__ __forceinline__ void sa_level_block(const ProblemDev& P, int pid, int
   const R l2f = (R)P.l2f;
   const R Tmax = (R)P.Tmax;
 
-  if (active) {
+  // chains in lockstep: the FP32 dynamic models, and FP32 Hagan chains run by
+  // fewer lanes than their sums are ordered by (the server's)
+  constexpr bool kDyn32 = sizeof(R) == 4 && (MODEL == SABR_DYN_I || MODEL == SABR_DYN_II);
+  bool ran = false;
+  if constexpr (kDyn32) {
+    ran = true;
+    lockstep_level<MODEL, D>(P, gchain, level, active, lane, L, s_lo, s_hi, s_step, inv_Tk, Tmax, x, fcur, bf, cbx, ev,
+                             ac, [&](const float* xp) {
+                               return dynamic_cost_f32<MODEL>(xp, P.n_quotes, P.n_mats, l2f, sq, coef, lane, L, G,
+                                                              0xffffffffu);
+                             });
+  } else if constexpr (sizeof(R) == 4 && MODEL == SABR_HAGAN && PAIRS < 5 && !ONE) {
+    if (L < G) {
+      ran = true;
+      const LaneSplit ls = lane_split(G, L);
+      lockstep_level<MODEL, D>(P, gchain, level, active, lane, L, s_lo, s_hi, s_step, inv_Tk, Tmax, x, fcur, bf, cbx,
+                               ev, ac, [&](const float* xp) {
+                                 const StaticPoint<float, SABR_HAGAN> pt(xp, l2f, P.n_quotes);
+                                 return virtual_lanes_sum<float>(pt, (P.n_quotes + 1) >> 1, G, ls, sq, 0xffffffffu);
+                               });
+    }
+  }
+  if (active && !ran) {
     // The FP32 static formulas draw one Philox block per proposal on one lane
     // and keep the ten round keys in registers; the other forms (whose
     // lanes share the draws, or whose register budget is tight) step the
@@ -211,7 +305,7 @@ __device__ __forceinline__ void sa_level_block(const ProblemDev& P, int pid, int
       }
     };
     bool ran_spec = false;
-    if constexpr (MODEL == SABR_HAGAN) {
+    if constexpr (MODEL == SABR_HAGAN && !ONE) {
       if (P.spec) {
         // Speculative acceptance (Hagan, several lanes per chain).
         // Acceptance is the common outcome (about 96% of the evaluated
@@ -336,21 +430,21 @@ __device__ __forceinline__ void sa_level_block(const ProblemDev& P, int pid, int
       constexpr int KIND = decltype(kind)::value;
       uint4 wbuf = make_uint4(0u, 0u, 0u, 0u);
       constexpr int NB = sa_philox_blocks(D);  // Philox blocks per step
-      const int S = G >= NB ? G / NB : 1;  // steps per batch of Philox blocks
+      const int S = L >= NB ? L / NB : 1;  // steps per batch of Philox blocks
       int s_ctr = 0;                         // st mod S
       uint4 wnext = make_uint4(0u, 0u, 0u, 0u);
-      if (NB == 1 && G == 1 && !ran_spec)
+      if (NB == 1 && L == 1 && !ran_spec)
         wnext = draw(make_uint4(gchain, (uint32_t)level, 0u, kTagSA));
       for (int st = 0; st < (ran_spec ? 0 : P.chain_len); ++st) {
         // D Philox words of blocks 0, 1, ... with counter (chain, level, step,
         // tag + block): D move uniforms and, from their unused low bits, the
-        // acceptance uniform (sa_accept_word).  With G >= NB lanes, the chain's
-        // lanes compute the blocks of S = G/NB consecutive steps at once
+        // acceptance uniform (sa_accept_word).  With L >= NB lanes, the chain's
+        // lanes compute the blocks of S = L/NB consecutive steps at once
         // (lane l: step st0 + l/NB, block l%NB) and every step gathers its
         // words by shuffles; otherwise each lane computes all NB blocks of
         // every step.
         uint32_t wv[4 * NB];
-        if (NB == 1 && G == 1) {
+        if (NB == 1 && L == 1) {
           // one lane, one block: no exchange; the block of the next step is
           // formed here, off the critical path of this one (its counter does
           // not depend on this step's outcome)
@@ -360,14 +454,14 @@ __device__ __forceinline__ void sa_level_block(const ProblemDev& P, int pid, int
           wv[1] = w.y;
           wv[2] = w.z;
           wv[3] = w.w;
-        } else if (G >= NB) {
+        } else if (L >= NB) {
           const int s_in = s_ctr;
           s_ctr = s_ctr + 1 == S ? 0 : s_ctr + 1;
           if (s_in == 0) {
             const int l = lane < S * NB ? lane : 0;
             wbuf = draw(make_uint4(gchain, (uint32_t)level, (uint32_t)(st + l / NB), kTagSA + (uint32_t)(l % NB)));
           }
-          const int base = ((threadIdx.x & 31) & ~(G - 1)) + s_in * NB;
+          const int base = ((threadIdx.x & 31) & ~(L - 1)) + s_in * NB;
 #pragma unroll
           for (int i = 0; i < D; ++i) {
             const uint32_t word =
@@ -390,10 +484,21 @@ __device__ __forceinline__ void sa_level_block(const ProblemDev& P, int pid, int
         u[D] = u01<R>(sa_accept_word(wv[0], wv[1], wv[2]));
         R xp[D];
         bool inside = true;
+        if constexpr (ONE) {
+          // three 16-byte loads for the step widths and the box
+          const float4 sw = *(const float4*)s_step, l4 = *(const float4*)s_lo, h4 = *(const float4*)s_hi;
+          const float w[4] = {sw.x, sw.y, sw.z, sw.w}, l[4] = {l4.x, l4.y, l4.z, l4.w}, h[4] = {h4.x, h4.y, h4.z, h4.w};
 #pragma unroll
-        for (int i = 0; i < D; ++i) {
-          xp[i] = propose(x[i], s_step[i], u[i]);
-          inside = inside && !(xp[i] < s_lo[i] || xp[i] > s_hi[i]);
+          for (int i = 0; i < D; ++i) {
+            xp[i] = propose(x[i], w[i], u[i]);
+            inside = inside && !(xp[i] < l[i] || xp[i] > h[i]);
+          }
+        } else {
+#pragma unroll
+          for (int i = 0; i < D; ++i) {
+            xp[i] = propose(x[i], s_step[i], u[i]);
+            inside = inside && !(xp[i] < s_lo[i] || xp[i] > s_hi[i]);
+          }
         }
         if (MODEL == SABR_DYN_II && inside) inside = case2_feasible<R>(xp, Tmax);
         if (!inside) continue;
@@ -463,9 +568,11 @@ __device__ __forceinline__ void sa_level_block(const ProblemDev& P, int pid, int
           default: step_loop(IntTag<8>{}); break;
         }
       }
-    } else {
+    } else if constexpr (!kDyn32) {
       step_loop(IntTag<0>{});
     }
+  }
+  if (active) {
     if (lane == 0) {
       P.chain_bf[chain] = cost_to_double(bf);
       if (level == 0) {
@@ -548,12 +655,12 @@ __device__ __forceinline__ void sa_level_block(const ProblemDev& P, int pid, int
 // level in .z (level < 0), so that one captured launch serves every step
 // whatever its mix of requests.  Both use this one kernel, so a problem's
 // arithmetic is the same machine code in a plan and in the server.
-// Register budget: up to 128 registers for the static formulas' quote loop
-// (pairs of quotes), the dynamic term structures (Case I closed forms, the
-// Case II rule's eight node values and thirteen running sums per panel) and
-// the chain state; the expanded form keeps 80.
+// Register budget: up to 128 registers for the static formulas (the server
+// keeps 16 of their warps an SM), 255 for the dynamic ones, whose chains run on
+// as few lanes as give a scheduler two warps; the expanded form keeps 80.
 template <class R, int MODEL> struct LevelMinBlocks {
-  static constexpr int value = sizeof(R) == 8 ? 1 : (MODEL == SABR_EXPANDED ? 3 : 2);
+  static constexpr int value =
+      sizeof(R) == 8 || MODEL == SABR_DYN_I || MODEL == SABR_DYN_II ? 1 : (MODEL == SABR_EXPANDED ? 3 : 2);
 };
 
 template <class R, int MODEL>
@@ -575,22 +682,22 @@ __global__ void __launch_bounds__(kSaBlock, (LevelMinBlocks<R, MODEL>::value))
 // Every level of a plan's launch group in one launch: each block takes units
 // from the ready queue until all are claimed (or a wait gave up).
 // Resident warps per SM the queue kernel is compiled for (in blocks of
-// kLevelBlock threads): the FP32 static formulas eight (two warps a
-// scheduler, up to 255 registers for the quote-pair loop), the FP32
-// dynamic models sixteen (128 registers; their term structures are
-// latency-bound and want more warps), the expanded form 24 at 80
-// registers, the FP64 form eight.
+// kLevelBlock threads): eight (two warps a scheduler, up to 255 registers),
+// the FP32 expanded form 24 at 80 registers.
 template <class R, int MODEL> struct QueueBlocks {
-  static constexpr int warps =
-      sizeof(R) == 8 ? 8 : ((MODEL == SABR_HAGAN || MODEL == SABR_OBLOJ) ? 8 : (MODEL == SABR_EXPANDED ? 24 : 16));
+  static constexpr int warps = MODEL == SABR_EXPANDED && sizeof(R) == 4 ? 24 : 8;
   static constexpr int value = warps * 32 / kLevelBlock;
 };
 template <class R, int MODEL> struct QueuePairs {
   static constexpr int value = 5;
 };
 
-template <class R, int MODEL>
-__global__ void __launch_bounds__(kLevelBlock, (QueueBlocks<R, MODEL>::value))
+// ONE: the loops for one lane a chain alone, at 198 registers (five blocks an
+// SM; the launch holds four): ten smiles x 4096 chains x 21 quotes, 200 x 100
+// in 24.7 ms, against 25.2-26.3 for the kernel that also holds the forms for
+// several lanes (two warps a scheduler live on the order of the instructions).
+template <class R, int MODEL, bool ONE = false>
+__global__ void __launch_bounds__(kLevelBlock, (ONE ? 5 : QueueBlocks<R, MODEL>::value))
     sa_queue_kernel(const ProblemDev* __restrict__ probs, LevelQueue q) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ ProblemDev P;
@@ -611,7 +718,7 @@ __global__ void __launch_bounds__(kLevelBlock, (QueueBlocks<R, MODEL>::value))
     const int lv = (int)((e >> 23) & (kQueueMaxLevels - 1));
     const int blk = (int)(e & (kQueueMaxBlocks - 1));
     load_problem(probs, pid, &P);
-    sa_level_block<R, MODEL, QueuePairs<R, MODEL>::value>(P, pid, blk, lv, smem, &q);
+    sa_level_block<R, MODEL, QueuePairs<R, MODEL>::value, false, ONE>(P, pid, blk, lv, smem, &q);
     __syncthreads();
   }
 }
@@ -792,14 +899,44 @@ int choose_lanes(int n_quotes, int n_mats, int model, int prec, long long batch_
   return G;
 }
 
+// FP32 dynamic models: a chain runs on fewer lanes than its sums are ordered
+// by, as many as give the GPU's schedulers two warps each -- every lane of a
+// chain repeats the proposal, the feasibility test and the recurrences, and
+// 12 maturities split evenly over 4 lanes and not over 8 (12 x 21 quotes, 40
+// levels x 50; Case I / II ms): 8192 chains 4 lanes 6.6 / 13.2, 8 lanes 9.3 /
+// 21.9 (two waves); 2048 chains 16 lanes 3.7 / 8.1, 32 lanes 6.4 / 12.6, 8
+// lanes 5.1 / 11.5; 1024 chains 32 lanes, 3.0 / 7.5 on 5 maturities.
+int choose_run_lanes(int n_quotes, int n_mats, int model, int prec, int G, long long batch_chains, int block) {
+  if (prec != SABR_FP32 || (model != SABR_DYN_I && model != SABR_DYN_II)) return G;
+  int L = G;
+  while (L > 4 && batch_chains * (L / 2) >= (long long)device_sms() * 4 * 32) L >>= 1;
+  // (the records of a block's chains have to fit in shared memory)
+  while (L < G && level_smem_bytes(prec, model, n_quotes, n_mats, block / L, kMaxC2Sub) > kMaxLevelSmem) L <<= 1;
+  return L;
+}
+
+// The server's steps hold the chains of many requests.  FP32 Hagan: about 12
+// pairs of quotes a lane, so that the chains of requests of every size take
+// about the same time a step and the proposal is repeated by few lanes (19
+// formula requests of 11 to 320 quotes, 1024 chains: 12 pairs a lane 50.6 ms,
+// 6 51.9, 24 62.2, 48 65.7; all lanes, two steps at once, about 95).  Dynamic
+// models: as for a batch of kServerChains chains.
+int server_run_lanes(int n_quotes, int n_mats, int model, int prec, int G) {
+  constexpr long long kServerChains = 4096;
+  if (prec != SABR_FP32 || model != SABR_HAGAN)
+    return choose_run_lanes(n_quotes, n_mats, model, prec, G, kServerChains, kSaBlock);
+  int L = 1;
+  while (L < G && 12 * L < (n_quotes + 1) / 2) L <<= 1;
+  return L;
+}
+
 size_t level_smem_bytes(int prec, int model, int Q, int M, int cpb, int c2_nsub) {
   const size_t rs = prec == SABR_FP64 ? 8 : 4;
-  const size_t cm = (model == SABR_DYN_I || model == SABR_DYN_II) ? (size_t)M : 0;
   size_t b = 4 * rs * ((size_t)Q + 1) + ((size_t)Q + M) * rs;  // pack (or pairs), l2k, mT
   b = align_up(b, 16);
   if (prec == SABR_FP32 && model == SABR_DYN_II)  // Case II rule: nodes, sub-panels, panels
     b = align_up(b + (size_t)c2_nsub * (kC2Nodes + 1) * 16 + (size_t)M * 8, 16);
-  b += (size_t)cpb * coef_stride(prec, model) * cm * rs + 16 * rs;
+  b += (size_t)cpb * coef_slice(prec, model, M) * rs + 16 * rs;
   b = align_up(b, 16) + 16;
   b += (size_t)cpb * 8 + (size_t)cpb * kMaxD * rs;
   return align_up(b, 16) + 64;
@@ -927,7 +1064,7 @@ sabr_status formula_prepare(const sabr_problem& pr, const sabr_bounds& b, const 
 }
 
 size_t formula_layout(const HostProblem& h, int G, unsigned char* img, unsigned char* base, size_t off0,
-                      ProblemDev& d, sabr_result* dres, int block) {
+                      ProblemDev& d, sabr_result* dres, int block, int L) {
   size_t o = off0;
   auto take = [&](size_t bytes) {
     o = align_up(o, 256);
@@ -950,7 +1087,8 @@ size_t formula_layout(const HostProblem& h, int G, unsigned char* img, unsigned 
   d.n_levels = h.n_levels;
   d.chain_len = h.chain_len;
   d.G = G;
-  d.cpb = block / G;
+  d.L = L > 0 ? L : G;
+  d.cpb = block / d.L;
   d.n_blocks = (h.n_chains + d.cpb - 1) / d.cpb;
   d.fwd = h.fwd;
   d.l2f = std::log2(h.fwd);
@@ -1047,7 +1185,7 @@ size_t formula_layout(const HostProblem& h, int G, unsigned char* img, unsigned 
   // latency-bound problems); with one lane per chain (large batches) the two
   // evaluations cost more issue slots than the latency they hide (measured
   // on the benchmark surface: 2.28e10 against 2.53e10 cost-evals/s)
-  d.spec = (h.model == SABR_HAGAN && G > 1 && speculate_enabled()) ? 1 : 0;
+  d.spec = (h.model == SABR_HAGAN && G > 1 && d.L == G && speculate_enabled()) ? 1 : 0;
   return o;
 }
 
@@ -1103,13 +1241,26 @@ void launch_finalize(int prec, int model, const ProblemDev* probs, const int* pl
   SABR_DISPATCH(prec, model, (sa_finalize_kernel<R, M><<<n, kSaBlock, 0, s>>>(probs, plist, queue_err)));
 }
 
+// one: every chain of the group has one lane.
+static bool queue_one(int prec, int model, bool one) { return one && prec == SABR_FP32 && model == SABR_HAGAN; }
+
 static void launch_queue(int prec, int model, const ProblemDev* probs, const LevelQueue& q, int grid, size_t smem,
-                         cudaStream_t s) {
+                         bool one, cudaStream_t s) {
+  if (queue_one(prec, model, one)) {
+    sa_queue_kernel<float, SABR_HAGAN, true><<<grid, kLevelBlock, smem, s>>>(probs, q);
+    return;
+  }
   SABR_DISPATCH(prec, model, (sa_queue_kernel<R, M><<<grid, kLevelBlock, smem, s>>>(probs, q)));
 }
 
-static int queue_blocks_per_sm(int prec, int model, size_t smem) {
+static int queue_blocks_per_sm(int prec, int model, size_t smem, bool one) {
   int nb = 1;
+  if (queue_one(prec, model, one)) {
+    cudaFuncSetAttribute(sa_queue_kernel<float, SABR_HAGAN, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sa_queue_kernel<float, SABR_HAGAN, true>, kLevelBlock, smem);
+    return nb < 1 ? 1 : nb;
+  }
   SABR_DISPATCH(prec, model, (cudaFuncSetAttribute(sa_queue_kernel<R, M>,
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
                               cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sa_queue_kernel<R, M>, kLevelBlock,
@@ -1139,6 +1290,7 @@ struct LaunchGroup {
   unsigned long long* d_level0 = nullptr;
   unsigned long long n0 = 0;
   int queue_grid = 0;
+  bool one_lane = true;  // every chain has one lane
   // few chains: one cooperative launch of sa_small_kernel (small_blocks > 0)
   SmallShape small;
   int small_blocks = 0;
@@ -1217,7 +1369,7 @@ static sabr_status enqueue_plan(sabr_plan* p, cudaStream_t s, bool capturing) {
     if (!g.use_queue || g.q.total == 0) continue;
     queue_reset_kernel<<<(int)std::min<unsigned long long>(1024, (g.q.total + 255) / 256), 256, 0, s>>>(
         g.q, g.d_level0, g.n0);
-    launch_queue(g.prec, g.model, p->d_probs, g.q, g.queue_grid, g.smem_level, s);
+    launch_queue(g.prec, g.model, p->d_probs, g.q, g.queue_grid, g.smem_level, g.one_lane, s);
     launches += 2;
     ++level_launches;
   }
@@ -1318,7 +1470,7 @@ static sabr_status build_plan(int32_t n, const sabr_problem* problems, const sab
   cudaGetDevice(&p->device);
 
   // arena: problem table, results, per-problem regions, launch maps
-  std::vector<int> lanes(nf);
+  std::vector<int> lanes(nf), run_lanes(nf);
   std::vector<ProblemDev> pd(nf);
   size_t o = 0;
   auto take = [&](size_t bytes) {
@@ -1336,13 +1488,16 @@ static sabr_status build_plan(int32_t n, const sabr_problem* problems, const sab
   for (int i = 0; i < nf; ++i) {
     const SmallChoice& sc = small[hp[i].prec * 5 + hp[i].model];
     if (sc.blocks > 0) hp[i].part_rows = 2 * small_blocks(sc.shape, hp[i].n_chains);
-    if (level_smem_bytes(hp[i].prec, hp[i].model, hp[i].n_quotes, hp[i].n_mats, kLevelBlock / lanes[i],
+    const int run = choose_run_lanes(hp[i].n_quotes, hp[i].n_mats, hp[i].model, hp[i].prec, lanes[i], batch_chains,
+                                     kLevelBlock);
+    run_lanes[i] = run;
+    if (level_smem_bytes(hp[i].prec, hp[i].model, hp[i].n_quotes, hp[i].n_mats, kLevelBlock / run,
                          hp[i].c2_nsub) > kMaxLevelSmem) {
       free_plan(p);
       return fail(SABR_EINVAL, "the quotes of a problem exceed one block's shared memory at its precision");
     }
     f_off[i] = align_up(o, 256);
-    o = formula_layout(hp[i], lanes[i], nullptr, nullptr, f_off[i], pd[i], nullptr, kLevelBlock);
+    o = formula_layout(hp[i], lanes[i], nullptr, nullptr, f_off[i], pd[i], nullptr, kLevelBlock, run_lanes[i]);
   }
   for (size_t k = 0; k < p->mc.size(); ++k) mc_off[k] = take(mcsa_arena_bytes(p->mc[k]));
   for (int i = 0; i < nf; ++i) {
@@ -1356,6 +1511,7 @@ static sabr_status build_plan(int32_t n, const sabr_problem* problems, const sab
       g->model = hp[i].model;
     }
     g->problems.push_back(i);
+    g->one_lane = g->one_lane && lanes[i] == 1;
     g->total_blocks += pd[i].n_blocks;
     g->max_levels = std::max(g->max_levels, hp[i].n_levels);
     g->smem_level = std::max(g->smem_level, level_smem_bytes(hp[i].prec, hp[i].model, hp[i].n_quotes, hp[i].n_mats,
@@ -1380,7 +1536,7 @@ static sabr_status build_plan(int32_t n, const sabr_problem* problems, const sab
     for (int pi : g.problems) {
       total += (unsigned long long)hp[pi].n_levels * (unsigned long long)pd[pi].n_blocks;
       for (int b = 0; hp[pi].n_levels > 0 && b < pd[pi].n_blocks; ++b) level0[gi].push_back(queue_entry(pi, 0, b));
-      const double per_step = (double)(hp[pi].n_quotes / lanes[pi] + 1) + 64.0 * hp[pi].n_mats + 64.0;
+      const double per_step = (double)(hp[pi].n_quotes / run_lanes[pi] + 1) + 64.0 * hp[pi].n_mats + 64.0;
       unit_ns = std::max(unit_ns, 100.0 * per_step * (double)hp[pi].chain_len);
     }
     // The queue pays when a level of the group has more units than the
@@ -1392,7 +1548,7 @@ static sabr_status build_plan(int32_t n, const sabr_problem* problems, const sab
     // instead of after a kernel launch (a level's fixed cost on one smile of
     // 64 chains: 13.7 us with a launch per level); larger single problems
     // run level by level.
-    const int per_sm = std::min(workers_per_sm(g.prec, g.model), queue_blocks_per_sm(g.prec, g.model, g.smem_level));
+    const int per_sm = std::min(workers_per_sm(g.prec, g.model), queue_blocks_per_sm(g.prec, g.model, g.smem_level, g.one_lane));
     int grid = std::max(1, std::min(g.total_blocks, sms * per_sm));
     const bool single_small = g.problems.size() == 1 && 2 * g.total_blocks <= sms * per_sm && p->max_levels > 1;
     if (single_small) grid = 2 * g.total_blocks;
@@ -1427,7 +1583,7 @@ static sabr_status build_plan(int32_t n, const sabr_problem* problems, const sab
   unsigned char* base = (unsigned char*)p->arena;
   sabr_result* dres = (sabr_result*)(base + results_off);
   for (int i = 0; i < nf; ++i)
-    formula_layout(hp[i], lanes[i], img.data(), base, f_off[i], pd[i], dres + fidx[i], kLevelBlock);
+    formula_layout(hp[i], lanes[i], img.data(), base, f_off[i], pd[i], dres + fidx[i], kLevelBlock, run_lanes[i]);
   for (size_t k = 0; k < p->mc.size(); ++k) mcsa_layout(p->mc[k], img.data(), base, mc_off[k], dres + p->mc_index[k]);
   if (nf > 0) std::memcpy(img.data() + probs_off, pd.data(), sizeof(ProblemDev) * nf);
   for (size_t gi = 0; gi < p->groups.size(); ++gi) {

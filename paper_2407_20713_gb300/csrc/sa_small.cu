@@ -22,10 +22,8 @@
 //    each level end on one counter: every block writes its minimum, arrives,
 //    and takes the argmin over the minima itself.
 //
-// A chain's misfit is summed in the order that G lanes (ProblemDev::G) give
-// it: virtual lane v sums units v, v + G, ... and the virtual lanes are added
-// by a butterfly.  A lane here plays the virtual lanes v = p, p + P, ..., so
-// the first levels of the butterfly are additions within the lane.
+// The misfit is summed in the order of ProblemDev::G lanes, played by the P
+// lanes of a group (virtual_lanes_sum).
 //
 // FP64: a scheduler issues one FP64 warp instruction in about 76 cycles, so
 // FP64 counts what FP64 instructions cost: box tests compare the numbers'
@@ -42,18 +40,6 @@ namespace sabr {
 constexpr int kRing = 64;        // steps whose proposal words a warp holds
 constexpr int kLevelCache = 32;  // levels whose temperatures a block holds
 constexpr int kSmallBlock = 128;
-
-__device__ __forceinline__ double cost_xor(double v, int off) { return __shfl_xor_sync(0xffffffffu, v, off); }
-__device__ __forceinline__ DF cost_xor(DF v, int off) {
-  return DF{__shfl_xor_sync(0xffffffffu, v.hi, off), __shfl_xor_sync(0xffffffffu, v.lo, off)};
-}
-__device__ __forceinline__ double cost_add(double a, double b) { return a + b; }
-__device__ __forceinline__ DF cost_add(DF a, DF b) { return df_add(a, b); }
-// the first level of a sum: df_add of (a, 0) and (b, 0) is the exact sum
-__device__ __forceinline__ double cost_add_first(double a, double b) { return a + b; }
-__device__ __forceinline__ DF cost_add_first(float a, float b) { return df_two_sum(a, b); }
-__device__ __forceinline__ double lane_cost(double v) { return v; }
-__device__ __forceinline__ DF lane_cost(float v) { return DF{v, 0.0f}; }
 
 // Box tests.  FP64 bounds and numbers are compared as integers that order
 // like the (finite) numbers: 32-bit ALU instructions instead of FP64 compares.
@@ -77,140 +63,6 @@ __device__ __forceinline__ double word_to(float w, double) {
   const uint32_t b = __float_as_uint(w);
   const uint32_t hi = (b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + ((1023u - 127u) << 20));
   return __hiloint2double((int)hi, (int)(b << 29));
-}
-
-// One static formula at one point: constants, and the unit residuals.  A unit
-// is a quote, or for FP32 Hagan a pair of quotes (float2).
-template <class R, int MODEL> struct StaticPoint {
-  static constexpr bool kPair = MODEL == SABR_HAGAN && sizeof(R) == 4;
-  StaticConst<R> sc;
-  PolyCoef<R> c0;
-  R bw;
-  __device__ __forceinline__ StaticPoint(const R* x, R l2f) {
-    if constexpr (MODEL == SABR_EXPANDED) {
-      c0 = expanded_coef<R>(x, l2f, (R)0);
-      bw = expanded_coef<R>(x, l2f, (R)1).c0 - c0.c0;
-    } else {
-      sc = static_setup<R>(x);
-    }
-  }
-  __device__ __forceinline__ R resid_of(int q, const SmemQuotes<R>& sq) const {
-    const QuotePack<R> qp = sq.pack[q];
-    R vol;
-    if constexpr (MODEL == SABR_HAGAN) {
-      vol = vol_hagan<R>(sc, qp.lfk, qp.l2kf, qp.T);
-    } else if constexpr (MODEL == SABR_OBLOJ) {
-      vol = vol_obloj<R>(sc, qp.lfk, qp.l2kf, sq.l2k[q], qp.T);
-    } else {
-      PolyCoef<R> c = c0;
-      c.c0 = c0.c0 + bw * qp.T;
-      vol = vol_poly<R>(c, qp.lfk);
-    }
-    return resid(vol, qp.w);
-  }
-  __device__ __forceinline__ float2 resid_pair_of(int j, int n_quotes, const SmemQuotes<R>& sq) const {
-    const float4 a = sq.pair[2 * j], b = sq.pair[2 * j + 1];
-    return hagan_resid_pair(sc, make_float2(a.x, a.y), make_float2(a.z, a.w), make_float2(b.x, b.y),
-                            make_float2(b.z, b.w), make_float2(1.0f, 2 * j + 1 < n_quotes ? 1.0f : 0.0f));
-  }
-  // sums of N virtual lanes v[0..N-1], the lanes' units side by side.  A unit
-  // past the end is evaluated as unit 0 and counts 0 (adding 0 changes no sum).
-  template <int N>
-  __device__ __forceinline__ void partials(const int (&v)[N], int units, int G, int n_quotes,
-                                           const SmemQuotes<R>& sq, R (&out)[N]) const {
-    if constexpr (kPair) {
-      float2 acc[N];
-#pragma unroll
-      for (int k = 0; k < N; ++k) acc[k] = make_float2(0.0f, 0.0f);
-      for (int j0 = 0; j0 < units; j0 += G) {
-#pragma unroll
-        for (int k = 0; k < N; ++k) {
-          const bool on = j0 + v[k] < units;
-          float2 r = resid_pair_of(on ? j0 + v[k] : 0, n_quotes, sq);
-          r.x = on ? r.x : 0.0f;
-          r.y = on ? r.y : 0.0f;
-          acc[k] = fma2(r, r, acc[k]);
-        }
-      }
-#pragma unroll
-      for (int k = 0; k < N; ++k) out[k] = acc[k].x + acc[k].y;
-    } else {
-#pragma unroll
-      for (int k = 0; k < N; ++k) out[k] = (R)0;
-      for (int j0 = 0; j0 < units; j0 += G) {
-#pragma unroll
-        for (int k = 0; k < N; ++k) {
-          const bool on = j0 + v[k] < units;
-          R r = resid_of(on ? j0 + v[k] : 0, sq);
-          r = on ? r : (R)0;
-          out[k] += r * r;
-        }
-      }
-    }
-  }
-};
-
-// How P lanes play G virtual lanes: pe of them differ (a lane beyond G repeats
-// another's work), V virtual lanes each.
-struct LaneSplit {
-  int pe, V, shift;  // shift = 32 - log2 V
-};
-__device__ __forceinline__ LaneSplit lane_split(int G, int P) {
-  LaneSplit s;
-  s.pe = G < P ? G : P;
-  s.V = G / s.pe;
-  s.shift = 32 - (31 - __clz(s.V));
-  return s;
-}
-
-// The misfit of a point by P lanes of a warp (every lane gets it).
-template <class R, int MODEL>
-__device__ __forceinline__ typename CostOf<R>::T point_cost(const R* x, int n_quotes, int units, R l2f,
-                                                            const SmemQuotes<R>& sq, int G, const LaneSplit& ls) {
-  using C = typename CostOf<R>::T;
-  const StaticPoint<R, MODEL> pt(x, l2f);
-  const int p = threadIdx.x & (ls.pe - 1);
-  C s;
-  int off = ls.pe >> 1;
-  if (ls.V == 1) {
-    const int v[1] = {p};
-    R a[1];
-    pt.template partials<1>(v, units, G, n_quotes, sq, a);
-    if (off > 0) {
-      s = cost_add_first(a[0], __shfl_xor_sync(0xffffffffu, a[0], off));
-      off >>= 1;
-    } else {
-      s = lane_cost(a[0]);
-    }
-  } else {
-    // the virtual lanes' butterfly starts with the farthest pairs: lanes are
-    // added in the order of their bit-reversed index, a binary counter holding
-    // the finished subtrees
-    C stack[5];
-#pragma unroll
-    for (int l = 0; l < 5; ++l) stack[l] = s = lane_cost((R)0);
-    for (int t = 0; t < ls.V; t += 2) {
-      const int i = (int)(__brev((unsigned)t) >> ls.shift);  // bit 0 of t is the farthest pair
-      const int v[2] = {p + ls.pe * i, p + ls.pe * (i + (ls.V >> 1))};
-      R a[2];
-      pt.template partials<2>(v, units, G, n_quotes, sq, a);
-      s = cost_add_first(a[0], a[1]);
-      bool carry = true;
-#pragma unroll
-      for (int l = 1; l < 5; ++l) {
-        if (carry) {
-          carry = ((t >> l) & 1) != 0;
-          if (carry) {
-            s = cost_add(stack[l], s);
-          } else {
-            stack[l] = s;
-          }
-        }
-      }
-    }
-  }
-  for (; off > 0; off >>= 1) s = cost_add(s, cost_xor(s, off));
-  return s;
 }
 
 // Barrier of a chain's NW warps (they are neighbours in the block).
@@ -354,7 +206,8 @@ __global__ void __launch_bounds__(kSmallBlock) sa_small_kernel(const ProblemDev*
           R xs[D];
 #pragma unroll
           for (int i = 0; i < D; ++i) xs[i] = s_x[warp][k_own][i];
-          const C fo = point_cost<R, MODEL>(xs, n_quotes, units, l2f, sq, G, ls);
+          const StaticPoint<R, MODEL> pt(xs, l2f, n_quotes);
+          const C fo = virtual_lanes_sum<R>(pt, units, G, ls, sq, 0xffffffffu);
           C* fb = s_f[cb][parity];
           parity ^= 1;
           if ((lane & (P - 1)) == 0) fb[k_own] = fo;

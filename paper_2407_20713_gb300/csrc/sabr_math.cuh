@@ -613,35 +613,62 @@ __device__ __forceinline__ void case1_coeffs(R nu0, R rho0, R a, R b, R T, R out
   constexpr int N = Tr<R>::kCase1Series;
   const R x = (R)2 * b * T, y = (a + b) * T;
   R g1, g2, g3, g4;
-  if (x < (R)2) {
-    const R mx = -x;
-    R s1 = (R)g1c(N), s2 = (R)g2c(N);
+  if constexpr (sizeof(R) == 4) {
+    // FP32: both forms, then selects -- the lanes of a chain hold different
+    // maturities, so a warp ran both branches nearly always, one after the
+    // other; without branches the four series, the closed forms and other
+    // maturities' evaluations overlap
+    const R mx = -x, my = -y;
+    R s1 = (R)g1c(N), s2 = (R)g2c(N), s3 = (R)g3c(N), s4 = (R)g4c(N);
 #pragma unroll
     for (int k = N - 1; k >= 0; --k) {
       s1 = s1 * mx + (R)g1c(k);
       s2 = s2 * mx + (R)g2c(k);
-    }
-    g1 = s1;
-    g2 = s2;
-  } else {
-    const R e = m_exp(-x), ix = m_rcp(x), ix3 = ix * ix * ix;
-    g1 = ((x * x * (R)0.5 - x + (R)1) - e) * ix3;
-    g2 = ((R)2 * (e - (R)1) + x * (e + (R)1)) * ix3;
-  }
-  if (y < (R)2) {
-    const R my = -y;
-    R s3 = (R)g3c(N), s4 = (R)g4c(N);
-#pragma unroll
-    for (int k = N - 1; k >= 0; --k) {
       s3 = s3 * my + (R)g3c(k);
       s4 = s4 * my + (R)g4c(k);
     }
-    g3 = s3;
-    g4 = s4;
+    const R ex = m_exp(-x), ix = m_rcp(x), ix3 = ix * ix * ix;
+    const R ey = m_exp(-y), iy = m_rcp(y), iy2 = iy * iy;
+    const R c1 = ((x * x * (R)0.5 - x + (R)1) - ex) * ix3;
+    const R c2 = ((R)2 * (ex - (R)1) + x * (ex + (R)1)) * ix3;
+    const R c3 = (ey - (R)1 + y) * iy2;
+    const R c4 = (m_exp(-(R)2 * y) - (R)8 * ey + ((R)7 + (R)2 * y * (y - (R)3))) * iy2 * iy2;
+    const bool sx = x < (R)2, sy = y < (R)2;
+    g1 = sx ? s1 : c1;
+    g2 = sx ? s2 : c2;
+    g3 = sy ? s3 : c3;
+    g4 = sy ? s4 : c4;
   } else {
-    const R e = m_exp(-y), iy = m_rcp(y), iy2 = iy * iy;
-    g3 = (e - (R)1 + y) * iy2;
-    g4 = (m_exp(-(R)2 * y) - (R)8 * e + ((R)7 + (R)2 * y * (y - (R)3))) * iy2 * iy2;
+    if (x < (R)2) {
+      const R mx = -x;
+      R s1 = (R)g1c(N), s2 = (R)g2c(N);
+#pragma unroll
+      for (int k = N - 1; k >= 0; --k) {
+        s1 = s1 * mx + (R)g1c(k);
+        s2 = s2 * mx + (R)g2c(k);
+      }
+      g1 = s1;
+      g2 = s2;
+    } else {
+      const R e = m_exp(-x), ix = m_rcp(x), ix3 = ix * ix * ix;
+      g1 = ((x * x * (R)0.5 - x + (R)1) - e) * ix3;
+      g2 = ((R)2 * (e - (R)1) + x * (e + (R)1)) * ix3;
+    }
+    if (y < (R)2) {
+      const R my = -y;
+      R s3 = (R)g3c(N), s4 = (R)g4c(N);
+#pragma unroll
+      for (int k = N - 1; k >= 0; --k) {
+        s3 = s3 * my + (R)g3c(k);
+        s4 = s4 * my + (R)g4c(k);
+      }
+      g3 = s3;
+      g4 = s4;
+    } else {
+      const R e = m_exp(-y), iy = m_rcp(y), iy2 = iy * iy;
+      g3 = (e - (R)1 + y) * iy2;
+      g4 = (m_exp(-(R)2 * y) - (R)8 * e + ((R)7 + (R)2 * y * (y - (R)3))) * iy2 * iy2;
+    }
   }
   out[0] = (R)6 * nu0 * nu0 * g1;
   out[1] = (R)6 * nu0 * nu0 * g2;

@@ -89,7 +89,7 @@ struct Request {
   bool cancelled_resident = false;
   HostProblem hp;
   McSaHost mh;
-  int G = 1, n_blocks = 0;
+  int G = 1, L = 1, n_blocks = 0;
   size_t bytes = 0, off = 0;
   int slot = -1;
   ProblemDev pd;
@@ -144,25 +144,59 @@ static size_t server_smem(int prec, int model, int max_quotes) {
   // only for M <= 2)
   const size_t rs = prec == SABR_FP64 ? 8 : 4;
   size_t b = level_smem_bytes(prec, SABR_HAGAN, max_quotes, kMaxMats, 256);
-  if (model == SABR_DYN_I || model == SABR_DYN_II) b += 512 * coef_stride(prec, model) * rs + 64;
+  if (model == SABR_DYN_I || model == SABR_DYN_II) b += (512 * coef_stride(prec, model) + 256 * 4) * rs + 64;
   // the FP32 Case II term-structure rule at its largest
   if (model == SABR_DYN_II && prec == SABR_FP32) b += (size_t)kMaxC2Sub * (kC2Nodes + 1) * 16 + kMaxMats * 8 + 16;
   return b;
 }
 
-static void enqueue_step_launches(sabr_server* s, int par, cudaStream_t st) {
-  cudaMemcpyAsync(s->d_nwork[par], s->h_nwork[par], sizeof(int) * kGroups, cudaMemcpyHostToDevice, st);
-  cudaMemcpyAsync(s->d_work[par], s->h_work[par], sizeof(int4) * kWorkPerGroup * kGroups, cudaMemcpyHostToDevice,
-                  st);
-  for (int g = 0; g < kGroups; ++g)
+// Streams and events of a step's parallel branches; they live until the
+// capture that uses them has ended.
+struct StepBranches {
+  cudaStream_t stream[kGroups] = {};
+  cudaEvent_t join[kGroups] = {}, fork = nullptr;
+  cudaError_t create() {
+    cudaError_t e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
+    for (int g = 0; g < kGroups && e == cudaSuccess; ++g) {
+      e = cudaStreamCreateWithFlags(&stream[g], cudaStreamNonBlocking);
+      if (e == cudaSuccess) e = cudaEventCreateWithFlags(&join[g], cudaEventDisableTiming);
+    }
+    return e;
+  }
+  ~StepBranches() {
+    for (int g = 0; g < kGroups; ++g) {
+      if (join[g]) cudaEventDestroy(join[g]);
+      if (stream[g]) cudaStreamDestroy(stream[g]);
+    }
+    if (fork) cudaEventDestroy(fork);
+  }
+};
+
+// A captured step: the work table's upload, then the groups' kernels as
+// parallel branches (a group's requests rarely fill the GPU, and the kernels of
+// empty groups end at once).
+static cudaError_t enqueue_step_launches(sabr_server* s, int par, cudaStream_t st, const StepBranches& br) {
+  cudaError_t e = cudaMemcpyAsync(s->d_nwork[par], s->h_nwork[par], sizeof(int) * kGroups, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(s->d_work[par], s->h_work[par], sizeof(int4) * kWorkPerGroup * kGroups, cudaMemcpyHostToDevice,
+                        st);
+  if (e == cudaSuccess) e = cudaEventRecord(br.fork, st);
+  for (int g = 0; g < kGroups && e == cudaSuccess; ++g) {
+    e = cudaStreamWaitEvent(br.stream[g], br.fork, 0);
+    if (e != cudaSuccess) break;
     launch_persistent(g / 5, g % 5, s->d_probs, s->d_work[par] + (size_t)g * kWorkPerGroup, s->d_nwork[par] + g,
-                      s->grid[g], s->smem[g], st);
+                      s->grid[g], s->smem[g], br.stream[g]);
+    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaEventRecord(br.join[g], br.stream[g]);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(st, br.join[g], 0);
+  }
+  return e;
 }
 
 static sabr_status upload_formula(sabr_server* s, Request& r) {
   std::vector<unsigned char> img(r.bytes, 0);
   unsigned char* base = s->pool + r.off;
-  formula_layout(r.hp, r.G, img.data(), base, 0, r.pd, s->d_results + r.slot);
+  formula_layout(r.hp, r.G, img.data(), base, 0, r.pd, s->d_results + r.slot, kSaBlock, r.L);
   SABR_CUDA(cudaMemcpyAsync(base, img.data(), r.bytes, cudaMemcpyHostToDevice, s->sf));
   SABR_CUDA(cudaMemcpyAsync(s->d_probs + r.slot, &r.pd, sizeof(ProblemDev), cudaMemcpyHostToDevice, s->sf));
   launch_init(r.hp.prec, r.hp.model, s->d_probs, s->d_ident + r.slot, 1, init_smem_bytes(r.hp), s->sf);
@@ -451,12 +485,19 @@ static sabr_status create_server(const sabr_server_config* cfg, sabr_server** ou
     s->grid[g] = sms * persistent_blocks_per_sm(g / 5, g % 5, s->smem[g]);
   }
   if (cfg->use_graph) {
+    StepBranches branches;
+    e = branches.create();
+    if (e != cudaSuccess) {
+      destroy_server(s);
+      return cuda_fail(e, "server graph branches");
+    }
     for (int p = 0; p < 2; ++p) {
       cudaGraph_t graph = nullptr;
       e = cudaStreamBeginCapture(s->sf, cudaStreamCaptureModeThreadLocal);
       if (e == cudaSuccess) {
-        enqueue_step_launches(s, p, s->sf);
+        const cudaError_t le = enqueue_step_launches(s, p, s->sf, branches);
         e = cudaStreamEndCapture(s->sf, &graph);
+        if (le != cudaSuccess) e = le;
       }
       if (e == cudaSuccess) e = cudaGraphInstantiate(&s->graph[p], graph, 0);
       if (graph) cudaGraphDestroy(graph);
@@ -488,14 +529,19 @@ static sabr_status submit(sabr_server* s, const sabr_problem* pr, const sabr_bou
     SABR_TRY(formula_prepare(*pr, *b, *c, seed, r->hp));
     if (r->hp.n_quotes > s->cfg.max_quotes) return fail(SABR_EINVAL, "request has more quotes than max_quotes");
     r->G = choose_lanes(r->hp.n_quotes, r->hp.n_mats, r->hp.model, r->hp.prec, r->hp.n_chains);
+    // a request shares the GPU with others: as few lanes a chain as a full
+    // GPU would give it, where the block's shared memory holds their records
+    const size_t have = s->smem[group_of(r->hp.prec, r->hp.model)];
+    auto need = [&](int L) {
+      return level_smem_bytes(r->hp.prec, r->hp.model, r->hp.n_quotes, r->hp.n_mats, kSaBlock / L, r->hp.c2_nsub);
+    };
+    r->L = server_run_lanes(r->hp.n_quotes, r->hp.n_mats, r->hp.model, r->hp.prec, r->G);
+    while (r->L < r->G && need(r->L) > have) r->L <<= 1;
     ProblemDev tmp;
-    r->bytes = formula_layout(r->hp, r->G, nullptr, nullptr, 0, tmp, nullptr) + 256;
+    r->bytes = formula_layout(r->hp, r->G, nullptr, nullptr, 0, tmp, nullptr, kSaBlock, r->L) + 256;
     r->n_blocks = tmp.n_blocks;
     if (r->n_blocks > kWorkPerGroup) return fail(SABR_EINVAL, "request has too many chains for one step");
-    const size_t need =
-        level_smem_bytes(r->hp.prec, r->hp.model, r->hp.n_quotes, r->hp.n_mats, tmp.cpb, r->hp.c2_nsub);
-    if (need > s->smem[group_of(r->hp.prec, r->hp.model)])
-      return fail(SABR_EINVAL, "request needs more shared memory than the server reserves");
+    if (need(r->L) > have) return fail(SABR_EINVAL, "request needs more shared memory than the server reserves");
   }
   if (r->bytes > (size_t)s->cfg.device_bytes) return fail(SABR_EINVAL, "request larger than the server pool");
   std::lock_guard<std::mutex> lk(s->mu);

@@ -20,6 +20,15 @@ def _stream_handle(stream):
     return ctypes.c_void_p(stream.cuda_stream)
 
 
+_Params = ctypes.c_double * 10
+
+
+def _params_c(params, model):
+    """The ten parameters as a C array (entries the model does not read are 0)."""
+    a = np.asarray(params, dtype=np.float64).ravel()
+    return _Params(*a[: capi.N_PARAMS[model]].tolist())
+
+
 def _params10(params, model):
     p = np.zeros(10, dtype=np.float64)
     a = np.asarray(params, dtype=np.float64).ravel()
@@ -28,8 +37,18 @@ def _params10(params, model):
     return p
 
 
+def _host_array(a, ctype):
+    """A contiguous host array as a C array over the same memory."""
+    if a is None:
+        return None
+    return (ctype * a.size).from_buffer(a) if a.flags.writeable else a.ctypes.data_as(ctypes.POINTER(ctype))
+
+
 def _dev64(x, device):
     if isinstance(x, torch.Tensor):
+        if (device == "cuda" and x.dtype == torch.float64 and x.is_cuda and x.is_contiguous()
+                and x.get_device() == torch.cuda.current_device()):
+            return x
         t = x.to(device=device, dtype=torch.float64)
     else:
         t = torch.as_tensor(np.asarray(x, dtype=np.float64), device=device)
@@ -40,13 +59,13 @@ def implied_vol(model, params, fwd, T, K, prec=FP32, out=None, stream=None, devi
     """Model implied vols of options (T[i], K[i]); returns a float64 CUDA tensor."""
     lib = capi.load()
     Tt = _dev64(T, device)
-    Kt = _dev64(K, device).expand_as(Tt).contiguous() if _dev64(K, device).numel() == 1 else _dev64(K, device)
+    Kt = _dev64(K, device)
+    if Kt.numel() == 1 and Kt.shape != Tt.shape:
+        Kt = Kt.expand_as(Tt).contiguous()
     if out is None:
         out = torch.empty_like(Tt)
-    p = _params10(params, model)
-    st = lib.sabr_implied_vol(model, p.ctypes.data_as(capi.PD), float(fwd), ctypes.c_void_p(Tt.data_ptr()),
-                              ctypes.c_void_p(Kt.data_ptr()), Tt.numel(), ctypes.c_void_p(out.data_ptr()),
-                              prec, _stream_handle(stream))
+    st = lib.sabr_implied_vol(model, _params_c(params, model), float(fwd), Tt.data_ptr(), Kt.data_ptr(), Tt.numel(),
+                              out.data_ptr(), prec, _stream_handle(stream))
     capi.check(st, "sabr_implied_vol")
     return out
 
@@ -63,12 +82,10 @@ def mc_price(model, params, fwd, T, K, is_call=None, discount=None, n_paths=1 <<
     dc = None if discount is None else np.ascontiguousarray(discount, dtype=np.float64).ravel()
     price = torch.empty(T.size, dtype=torch.float64, device=device)
     se = torch.empty(T.size, dtype=torch.float64, device=device)
-    p = _params10(params, model)
-    head = (model, p.ctypes.data_as(capi.PD), float(fwd), T.ctypes.data_as(capi.PD), K.ctypes.data_as(capi.PD),
-            ic.ctypes.data_as(capi.PI8) if ic is not None else None,
-            dc.ctypes.data_as(capi.PD) if dc is not None else None, T.size, int(n_paths), float(steps_per_year),
+    head = (model, _params_c(params, model), float(fwd), _host_array(T, capi.c_double), _host_array(K, capi.c_double),
+            _host_array(ic, capi.c_int8), _host_array(dc, capi.c_double), T.size, int(n_paths), float(steps_per_year),
             int(seed) & 0xFFFFFFFFFFFFFFFF)
-    tail = (ctypes.c_void_p(price.data_ptr()), ctypes.c_void_p(se.data_ptr()), prec, _stream_handle(stream))
+    tail = (price.data_ptr(), se.data_ptr(), prec, _stream_handle(stream))
     if scheme is None:
         capi.check(lib.sabr_mc_price(*head, *tail), "sabr_mc_price")
     else:

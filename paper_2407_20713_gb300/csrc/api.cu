@@ -1,6 +1,9 @@
 // api.cu -- error reporting and argument checks shared by the entry points.
 #include <atomic>
 #include <cmath>
+#include <map>
+#include <mutex>
+#include <utility>
 
 #include "common.h"
 
@@ -19,6 +22,21 @@ void clear_error() { g_error[0] = '\0'; }
 
 // SM count of the current device, queried once per device ordinal and
 // cached (the grid sizes of the kernels are multiples of it).
+cudaError_t allow_smem(const void* kernel, size_t bytes) {
+  static std::mutex mu;
+  static std::map<std::pair<int, const void*>, size_t> allowed;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lock(mu);
+  // (48 KB need no opt-in, the kernel's static shared memory included)
+  size_t& have = allowed.emplace(std::make_pair(dev, kernel), (size_t)32 * 1024).first->second;
+  if (bytes <= have) return cudaSuccess;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e == cudaSuccess) have = bytes;
+  return e;
+}
+
 int device_sms() {
   static std::atomic<int> cache[64];
   int dev = 0;

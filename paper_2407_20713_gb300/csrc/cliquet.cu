@@ -184,10 +184,10 @@ extern "C" sabr_status sabr_mc_cliquet(sabr_model model, const double* params, d
   // Small blocks keep the SMs' shares equal.
   int per_sm = 8;
   if (prec == SABR_FP64) {
-    cudaFuncSetAttribute(cliquet_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem((const void*)cliquet_kernel<double>, smem);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cliquet_kernel<double>, kClqBlock, smem);
   } else {
-    cudaFuncSetAttribute(cliquet_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem((const void*)cliquet_kernel<float>, smem);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cliquet_kernel<float>, kClqBlock, smem);
   }
   per_sm = std::max(per_sm, 1);
@@ -202,42 +202,28 @@ extern "C" sabr_status sabr_mc_cliquet(sabr_model model, const double* params, d
   const size_t tab_bytes = mc_step_table_bytes(h, 1);
   const size_t bytes = tab_off + tab_bytes;
   cudaStream_t s = (cudaStream_t)stream;
-  unsigned char* dev = nullptr;
-  SABR_CUDA(cudaMallocAsync((void**)&dev, bytes, s));
-  std::vector<unsigned char> host(part_off, 0);
+  McScratch w;
+  SABR_TRY(w.acquire(bytes, part_off));
+  unsigned char* dev = w.dev;
   McDev d;
   int *q_value, *q_out;
   double* disc;
-  mc_fill_image(h, host.data(), dev, d, &q_value, &q_out, &disc);
+  mc_fill_image(h, w.host, dev, d, &q_value, &q_out, &disc);
   if (tab_bytes) d.tab = dev + tab_off;
   double p10[kMaxD];
   for (int i = 0; i < kMaxD; ++i) p10[i] = i < n_params(model) ? params[i] : 0.0;
-  std::memcpy(host.data() + params_off, p10, sizeof(p10));
-  // pageable source: the copy has consumed `host` when this returns
-  cudaError_t e = cudaMemcpyAsync(dev, host.data(), part_off, cudaMemcpyHostToDevice, s);
-  if (e != cudaSuccess) {
-    cudaFreeAsync(dev, s);
-    return cuda_fail(e, "cudaMemcpyAsync");
-  }
+  std::memcpy(w.host + params_off, p10, sizeof(p10));
+  SABR_CUDA(cudaMemcpyAsync(dev, w.host, part_off, cudaMemcpyHostToDevice, s));
   double* part = (double*)(dev + part_off);
   const double* dp = (const double*)(dev + params_off);
   if (tab_bytes) mc_launch_steps(h, d, dp, nullptr, 1, s);
-  if (prec == SABR_FP64) {
-    e = cudaFuncSetAttribute(cliquet_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess)
-      cliquet_kernel<double><<<blocks, kClqBlock, smem, s>>>(d, dp, floor_local, cap_local, floor_global,
-                                                            cap_global, part);
-  } else {
-    e = cudaFuncSetAttribute(cliquet_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess)
-      cliquet_kernel<float><<<blocks, kClqBlock, smem, s>>>(d, dp, floor_local, cap_local, floor_global,
-                                                           cap_global, part);
-  }
-  if (e == cudaSuccess) {
-    cliquet_reduce_kernel<<<1, kClqBlock, 0, s>>>(part, blocks, n_paths, discount, price_out, stderr_out);
-    e = cudaGetLastError();
-  }
-  cudaFreeAsync(dev, s);
-  if (e != cudaSuccess) return cuda_fail(e, "cliquet launch");
-  return SABR_OK;
+  if (prec == SABR_FP64)
+    cliquet_kernel<double><<<blocks, kClqBlock, smem, s>>>(d, dp, floor_local, cap_local, floor_global, cap_global,
+                                                          part);
+  else
+    cliquet_kernel<float><<<blocks, kClqBlock, smem, s>>>(d, dp, floor_local, cap_local, floor_global, cap_global,
+                                                         part);
+  cliquet_reduce_kernel<<<1, kClqBlock, 0, s>>>(part, blocks, n_paths, discount, price_out, stderr_out);
+  SABR_CUDA(cudaGetLastError());
+  return w.release(s);
 }

@@ -50,6 +50,12 @@ inline int n_params(int model) {
 // Streaming multiprocessors of the current device (cached per device).
 int device_sms();
 
+// Raises a kernel's dynamic shared memory allowance on the current device to at
+// least `bytes`.  The allowance is never lowered: it belongs to the kernel, and
+// another thread's launch, or a captured graph's, may need more than this
+// call's.
+cudaError_t allow_smem(const void* kernel, size_t bytes);
+
 // Range checks of a parameter vector common to every entry point.
 sabr_status check_params(int model, const double* p);
 

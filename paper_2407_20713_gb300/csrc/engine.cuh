@@ -778,7 +778,12 @@ __device__ __forceinline__ void case2_group_coef_rule(const float* xp, int n_mat
     float4* r = reinterpret_cast<float4*>(rec + CS * j);
     const float4 v = *r;  // A, D, H, K
     const float iT = rcp_approx(T), iT2 = iT * iT;
-    const PolyCoef<float> c = dynamic_poly<float>(xp[0], xp[1], l2f, T, 3.0f * v.x * iT2 * iT, 6.0f * v.y * iT2 * iT,
+    // opaque: hoisted out of the loop, (1 - beta)^2 / 24 and / 12 would be
+    // rounded before they are added, and the polynomial differ in a last bit
+    // from one kernel to another
+    float beta = xp[1];
+    asm volatile("" : "+f"(beta));
+    const PolyCoef<float> c = dynamic_poly<float>(xp[0], beta, l2f, T, 3.0f * v.x * iT2 * iT, 6.0f * v.y * iT2 * iT,
                                                   2.0f * v.z * iT2, 12.0f * v.w * iT2 * iT2);
     *r = make_float4(c.c0, c.c1, c.c2, 0.0f);
   }

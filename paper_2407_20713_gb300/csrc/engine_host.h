@@ -39,7 +39,7 @@ int choose_lanes(int n_quotes, int n_mats, int model, int prec, long long batch_
 // Lanes that run a chain whose sums are in the order of G (at most G; blocks
 // of `block` threads).
 int choose_run_lanes(int n_quotes, int n_mats, int model, int prec, int G, long long batch_chains, int block);
-int server_run_lanes(int n_quotes, int n_mats, int model, int prec, int G);
+int server_base_lanes(int n_quotes, int model, int prec, int G);
 // Dynamic shared memory of a level block (cpb chains) / of an init block;
 // c2_nsub: sub-panels of the FP32 Case II rule (0 otherwise).
 size_t level_smem_bytes(int prec, int model, int Q, int M, int cpb, int c2_nsub = 0);

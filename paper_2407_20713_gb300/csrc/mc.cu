@@ -384,7 +384,7 @@ static McPathsFn mc_paths_fn(const McHost& h, bool split, size_t* smem) {
                                              : mc_paths_kernel<float, SABR_MC_LOG_EULER, false>);
     *smem = mc_smem_layout<float>(S, h.n_quotes, M, h.n_slots, split).total;
   }
-  cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem);
+  allow_smem((const void*)fn, *smem);
   return fn;
 }
 
@@ -473,9 +473,12 @@ sabr_status mc_launch(const McHost& h, const McDev& d, const double* set_params,
   return SABR_OK;
 }
 
-// Library-owned scratch of sabr_mc_price, one per device, reused by every
-// call on that device (calls are serialised by a mutex and by waiting for the
-// previous call's kernels before the scratch is rewritten).
+// Library-owned scratch of the pricers: two per device, taken in turn, so that a
+// call's tables are laid out and copied while the kernels of the call before it
+// run (2^16 paths: the GPU waited about 15 us between calls).  Calls are
+// serialised by the mutex and by waiting, before a scratch is rewritten, for
+// the kernels that last used it; calls on several streams therefore never
+// share one in flight.  A scratch grows to what its calls need and stays.
 struct McWorkspace {
   void* dev = nullptr;
   size_t dev_bytes = 0;
@@ -483,8 +486,12 @@ struct McWorkspace {
   size_t host_bytes = 0;
   cudaEvent_t done = nullptr;
 };
+struct McWorkspaces {
+  McWorkspace ws[2];
+  int next = 0;
+};
 static std::mutex g_mc_mutex;
-static std::vector<McWorkspace> g_mc_ws;
+static std::vector<McWorkspaces> g_mc_ws;
 
 static sabr_status ensure_ws(McWorkspace& w, size_t dev_bytes, size_t host_bytes) {
   if (!w.done) SABR_CUDA(cudaEventCreateWithFlags(&w.done, cudaEventDisableTiming));
@@ -503,6 +510,25 @@ static sabr_status ensure_ws(McWorkspace& w, size_t dev_bytes, size_t host_bytes
     SABR_CUDA(cudaMallocHost(&w.host, host_bytes));
     w.host_bytes = host_bytes;
   }
+  return SABR_OK;
+}
+
+sabr_status McScratch::acquire(size_t dev_bytes, size_t host_bytes) {
+  lock_ = std::unique_lock<std::mutex>(g_mc_mutex);
+  int d = 0;
+  SABR_CUDA(cudaGetDevice(&d));
+  if ((int)g_mc_ws.size() <= d) g_mc_ws.resize(d + 1);
+  McWorkspaces& all = g_mc_ws[d];
+  McWorkspace& w = all.ws[all.next];
+  all.next ^= 1;
+  SABR_TRY(ensure_ws(w, dev_bytes, host_bytes));
+  dev = (unsigned char*)w.dev;
+  host = w.host;
+  done_ = w.done;
+  return SABR_OK;
+}
+sabr_status McScratch::release(cudaStream_t s) {
+  SABR_CUDA(cudaEventRecord(done_, s));
   return SABR_OK;
 }
 
@@ -529,17 +555,13 @@ static sabr_status mc_price(sabr_model model, const double* params, double fwd, 
   const size_t tab_off = part_off + sizeof(double) * (size_t)bps * h.n_slots * 32;
   const size_t tab_bytes = mc_step_table_bytes(h, 1);
   const size_t dev_bytes = tab_off + tab_bytes;
-  std::lock_guard<std::mutex> lock(g_mc_mutex);
-  int dev = 0;
-  SABR_CUDA(cudaGetDevice(&dev));
-  if ((int)g_mc_ws.size() <= dev) g_mc_ws.resize(dev + 1);
-  McWorkspace& w = g_mc_ws[dev];
-  SABR_TRY(ensure_ws(w, dev_bytes, part_off));
+  McScratch w;
+  SABR_TRY(w.acquire(dev_bytes, part_off));
   McDev d;
   int* q_value;
   int* q_out;
   double* disc;
-  unsigned char* base = (unsigned char*)w.dev;
+  unsigned char* base = w.dev;
   mc_fill_image(h, w.host, base, d, &q_value, &q_out, &disc);
   if (tab_bytes) d.tab = base + tab_off;
   double p10[kMaxD];
@@ -549,8 +571,7 @@ static sabr_status mc_price(sabr_model model, const double* params, double fwd, 
   SABR_CUDA(cudaMemcpyAsync(w.dev, w.host, part_off, cudaMemcpyHostToDevice, s));
   SABR_TRY(mc_launch(h, d, (const double*)(base + params_off), nullptr, 1, bps, (double*)(base + part_off), q_value,
                      q_out, disc, price_out, stderr_out, (int)n, s));
-  SABR_CUDA(cudaEventRecord(w.done, s));
-  return SABR_OK;
+  return w.release(s);
 }
 
 }  // namespace sabr
@@ -598,21 +619,15 @@ static sabr_status mc_shard_prepare(sabr_model model, const double* params, doub
   return SABR_OK;
 }
 
-// Uploads the tables and parameters into the per-device workspace; returns
-// the device image and the workspace (whose `done` event the caller records).
-static sabr_status mc_shard_upload(const McShardCall& c, const double* params, cudaStream_t s, McDev& d,
-                                   int** q_value, int** q_out, double** disc, const double** dparams,
-                                   McWorkspace** ws) {
+// Uploads the tables and parameters into a scratch; returns the device image.
+static sabr_status mc_shard_upload(const McShardCall& c, const double* params, cudaStream_t s, McScratch& w, McDev& d,
+                                   int** q_value, int** q_out, double** disc, const double** dparams) {
   const size_t img = mc_image_bytes(c.h);
   const size_t params_off = (img + 255) & ~(size_t)255;
   const size_t part_off = params_off + 256;
-  int dev = 0;
-  SABR_CUDA(cudaGetDevice(&dev));
-  if ((int)g_mc_ws.size() <= dev) g_mc_ws.resize(dev + 1);
-  McWorkspace& w = g_mc_ws[dev];
   const size_t tab_bytes = mc_step_table_bytes(c.h, 1);
-  SABR_TRY(ensure_ws(w, part_off + tab_bytes, part_off));
-  unsigned char* base = (unsigned char*)w.dev;
+  SABR_TRY(w.acquire(part_off + tab_bytes, part_off));
+  unsigned char* base = w.dev;
   mc_fill_image(c.h, w.host, base, d, q_value, q_out, disc);
   if (tab_bytes) d.tab = base + part_off;
   double p10[kMaxD];
@@ -620,7 +635,6 @@ static sabr_status mc_shard_upload(const McShardCall& c, const double* params, c
   std::memcpy(w.host + params_off, p10, sizeof(p10));
   SABR_CUDA(cudaMemcpyAsync(w.dev, w.host, part_off, cudaMemcpyHostToDevice, s));
   *dparams = (const double*)(base + params_off);
-  *ws = &w;
   return SABR_OK;
 }
 
@@ -649,7 +663,6 @@ extern "C" sabr_status sabr_mc_shard_partials(sabr_model model, const double* pa
   using namespace sabr;
   clear_error();
   if (!partials_out) return fail(SABR_EINVAL, "partials_out is NULL");
-  std::lock_guard<std::mutex> lock(g_mc_mutex);
   McShardCall c;
   SABR_TRY(mc_shard_prepare(model, params, fwd, T, K, is_call, discount, n, n_paths, steps_per_year, seed, prec, c));
   if (total_blocks < 1 || block_count < 1 || block_begin < 0 || (int64_t)block_begin + block_count > total_blocks)
@@ -659,12 +672,11 @@ extern "C" sabr_status sabr_mc_shard_partials(sabr_model model, const double* pa
   int *q_value, *q_out;
   double* disc;
   const double* dp;
-  McWorkspace* w;
-  SABR_TRY(mc_shard_upload(c, params, s, d, &q_value, &q_out, &disc, &dp, &w));
+  McScratch w;
+  SABR_TRY(mc_shard_upload(c, params, s, w, d, &q_value, &q_out, &disc, &dp));
   launch_paths(c.h, d, dp, nullptr, dim3(block_count, 1), partials_out, block_begin, total_blocks, s);
   SABR_CUDA(cudaGetLastError());
-  SABR_CUDA(cudaEventRecord(w->done, s));
-  return SABR_OK;
+  return w.release(s);
 }
 
 extern "C" sabr_status sabr_mc_shard_reduce(sabr_model model, const double* params, double fwd, const double* T,
@@ -675,7 +687,6 @@ extern "C" sabr_status sabr_mc_shard_reduce(sabr_model model, const double* para
   using namespace sabr;
   clear_error();
   if (!partials || !price_out) return fail(SABR_EINVAL, "NULL partials or price_out");
-  std::lock_guard<std::mutex> lock(g_mc_mutex);
   McShardCall c;
   SABR_TRY(mc_shard_prepare(model, params, fwd, T, K, is_call, discount, n, n_paths, steps_per_year, seed, prec, c));
   if (total_blocks < 1) return fail(SABR_EINVAL, "total_blocks must be >= 1");
@@ -684,10 +695,9 @@ extern "C" sabr_status sabr_mc_shard_reduce(sabr_model model, const double* para
   int *q_value, *q_out;
   double* disc;
   const double* dp;
-  McWorkspace* w;
-  SABR_TRY(mc_shard_upload(c, params, s, d, &q_value, &q_out, &disc, &dp, &w));
+  McScratch w;
+  SABR_TRY(mc_shard_upload(c, params, s, w, d, &q_value, &q_out, &disc, &dp));
   launch_reduce(d, 1, total_blocks, partials, q_value, q_out, disc, nullptr, price_out, stderr_out, (int)n, s);
   SABR_CUDA(cudaGetLastError());
-  SABR_CUDA(cudaEventRecord(w->done, s));
-  return SABR_OK;
+  return w.release(s);
 }

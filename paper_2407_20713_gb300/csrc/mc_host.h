@@ -2,6 +2,7 @@
 // by sabr_mc_price and the Technique II (MC-cost) calibration engine.
 #pragma once
 #include <cstdint>
+#include <mutex>
 #include <vector>
 
 #include "common.h"
@@ -19,6 +20,21 @@ struct McHost {
   std::vector<double> mats, K, disc, step_t, step_h;
   std::vector<int> mat_q0, mat_nq, mat_slot, step_mat, q_out, q_value;
   std::vector<int8_t> call;
+};
+
+// A call's hold on the pricers' scratch of the current device: acquire() waits
+// for the kernels that last used it and holds the pricers' lock until the call
+// has enqueued its work; release() marks that work on the stream.
+class McScratch {
+ public:
+  sabr_status acquire(size_t dev_bytes, size_t host_bytes);
+  sabr_status release(cudaStream_t s);
+  unsigned char* dev = nullptr;
+  unsigned char* host = nullptr;  // pinned
+
+ private:
+  std::unique_lock<std::mutex> lock_;
+  cudaEvent_t done_ = nullptr;
 };
 
 // Validates the option set and builds the step grid (options sorted by

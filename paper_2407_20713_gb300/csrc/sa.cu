@@ -306,7 +306,7 @@ __device__ __forceinline__ void sa_level_block(const ProblemDev& P, int pid, int
     };
     bool ran_spec = false;
     if constexpr (MODEL == SABR_HAGAN && !ONE) {
-      if (P.spec) {
+      if (P.spec && L == G) {
         // Speculative acceptance (Hagan, several lanes per chain).
         // Acceptance is the common outcome (about 96% of the evaluated
         // proposals on the benchmark smiles), so each iteration forms step
@@ -674,6 +674,14 @@ __global__ void __launch_bounds__(kSaBlock, (LevelMinBlocks<R, MODEL>::value))
     const int4 it = work[w];
     const int lv = level >= 0 ? level : it.z;
     load_problem(probs, it.x, &P);
+    if (it.w != 0) {  // the step's own lanes per chain
+      if (threadIdx.x == 0) {
+        P.L = it.w;
+        P.cpb = (int)blockDim.x / it.w;
+        P.n_blocks = (P.n_chains + P.cpb - 1) / P.cpb;
+      }
+      __syncthreads();
+    }
     if (lv < P.n_levels) sa_level_block<R, MODEL, 2, true>(P, it.x, it.y, lv, smem, nullptr);
     __syncthreads();
   }
@@ -915,16 +923,17 @@ int choose_run_lanes(int n_quotes, int n_mats, int model, int prec, int G, long 
   return L;
 }
 
-// The server's steps hold the chains of many requests.  FP32 Hagan: about 12
-// pairs of quotes a lane, so that the chains of requests of every size take
-// about the same time a step and the proposal is repeated by few lanes (19
-// formula requests of 11 to 320 quotes, 1024 chains: 12 pairs a lane 50.6 ms,
-// 6 51.9, 24 62.2, 48 65.7; all lanes, two steps at once, about 95).  Dynamic
-// models: as for a batch of kServerChains chains.
-int server_run_lanes(int n_quotes, int n_mats, int model, int prec, int G) {
-  constexpr long long kServerChains = 4096;
-  if (prec != SABR_FP32 || model != SABR_HAGAN)
-    return choose_run_lanes(n_quotes, n_mats, model, prec, G, kServerChains, kSaBlock);
+// The server's steps hold the chains of many requests, and each step may give
+// a request's chains other lanes (level_lanes in server.cu); these are those of
+// a full GPU.  FP32 Hagan: about 12 pairs of quotes a lane, so that the chains
+// of requests of every size take about the same time a step and the proposal
+// is repeated by few lanes (19 formula requests of 11 to 320 quotes, 1024
+// chains: 12 pairs a lane 50.6 ms, 6 51.9, 24 62.2, 48 65.7; all lanes, two
+// steps at once, about 95).
+int server_base_lanes(int n_quotes, int model, int prec, int G) {
+  if (prec != SABR_FP32) return G;
+  if (model == SABR_DYN_I || model == SABR_DYN_II) return std::min(G, 4);
+  if (model != SABR_HAGAN) return G;
   int L = 1;
   while (L < G && 12 * L < (n_quotes + 1) / 2) L <<= 1;
   return L;
@@ -1192,8 +1201,8 @@ size_t formula_layout(const HostProblem& h, int G, unsigned char* img, unsigned 
 // ---- launch wrappers ------------------------------------------------------
 template <class R, int MODEL>
 static void set_smem_one(size_t bytes) {
-  cudaFuncSetAttribute(sa_level_kernel<R, MODEL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  cudaFuncSetAttribute(sa_init_kernel<R, MODEL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  allow_smem((const void*)sa_level_kernel<R, MODEL>, bytes);
+  allow_smem((const void*)sa_init_kernel<R, MODEL>, bytes);
 }
 
 #define SABR_DISPATCH(prec, model, CALL)                              \
@@ -1256,13 +1265,11 @@ static void launch_queue(int prec, int model, const ProblemDev* probs, const Lev
 static int queue_blocks_per_sm(int prec, int model, size_t smem, bool one) {
   int nb = 1;
   if (queue_one(prec, model, one)) {
-    cudaFuncSetAttribute(sa_queue_kernel<float, SABR_HAGAN, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
+    allow_smem((const void*)sa_queue_kernel<float, SABR_HAGAN, true>, smem);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sa_queue_kernel<float, SABR_HAGAN, true>, kLevelBlock, smem);
     return nb < 1 ? 1 : nb;
   }
-  SABR_DISPATCH(prec, model, (cudaFuncSetAttribute(sa_queue_kernel<R, M>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+  SABR_DISPATCH(prec, model, (allow_smem((const void*)sa_queue_kernel<R, M>, smem),
                               cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sa_queue_kernel<R, M>, kLevelBlock,
                                                                             smem)));
   return nb < 1 ? 1 : nb;
@@ -1341,6 +1348,9 @@ struct sabr_plan {
   int64_t launches = 0;
   int64_t level_launches = 0;
   bool ran = false;
+  bool blocking = false;   // of a blocking call: buffers kept (KeptBuffers)
+  size_t arena_bytes = 0;  // allocated
+  int h_count = 0;
   std::vector<sabr::McSaHost> mc;  // Technique II problems
   std::vector<int> mc_index;       // their batch index
 };
@@ -1401,8 +1411,55 @@ static sabr_status enqueue_plan(sabr_plan* p, cudaStream_t s, bool capturing) {
   return SABR_OK;
 }
 
+// The buffers of the blocking calls (sabr_calibrate, sabr_calibrate_batch): one
+// set per device is kept from one call to the next, up to kKeptArena bytes --
+// allocating and freeing device and pinned memory took 0.8 ms of a smile's
+// 4.7.  A call that finds the set in use (another thread's call) or too small
+// allocates its own and leaves the larger of the two behind.
+struct KeptBuffers {
+  void* arena = nullptr;
+  size_t bytes = 0;
+  sabr_result* results = nullptr;
+  int n = 0;
+};
+constexpr size_t kKeptArena = 64u << 20;
+constexpr int kKeptResults = 4096;
+static std::mutex g_kept_mutex;
+static std::vector<KeptBuffers> g_kept;
+
+static KeptBuffers take_kept(int device) {
+  std::lock_guard<std::mutex> lock(g_kept_mutex);
+  if ((int)g_kept.size() <= device) g_kept.resize(device + 1);
+  KeptBuffers k = g_kept[device];
+  g_kept[device] = KeptBuffers();
+  return k;
+}
+// Returns the buffers to keep or frees them (no work of theirs is in flight).
+static void give_kept(int device, KeptBuffers k) {
+  {
+    std::lock_guard<std::mutex> lock(g_kept_mutex);
+    KeptBuffers& slot = g_kept[device];
+    if (k.bytes <= kKeptArena && k.bytes >= slot.bytes) std::swap(slot.arena, k.arena), std::swap(slot.bytes, k.bytes);
+    if (k.n <= kKeptResults && k.n >= slot.n) std::swap(slot.results, k.results), std::swap(slot.n, k.n);
+  }
+  if (k.arena) cudaFree(k.arena);
+  if (k.results) cudaFreeHost(k.results);
+}
+
 static void free_plan(sabr_plan* p) {
   if (!p) return;
+  // (a run that failed half way may have kernels in flight: its buffers are
+  // freed, which waits for them)
+  if (p->blocking && p->ran && cudaEventSynchronize(p->ev_done) == cudaSuccess) {
+    KeptBuffers k;
+    k.arena = p->arena;
+    k.bytes = p->arena_bytes;
+    k.results = p->h_results;
+    k.n = p->h_count;
+    give_kept(p->device, k);
+    p->arena = nullptr;
+    p->h_results = nullptr;
+  }
   if (p->exec) cudaGraphExecDestroy(p->exec);
   if (p->ev_lv0) cudaEventDestroy(p->ev_lv0);
   if (p->ev_lv1) cudaEventDestroy(p->ev_lv1);
@@ -1442,7 +1499,7 @@ static std::vector<SmallChoice> choose_small(const std::vector<HostProblem>& hp,
 
 static sabr_status build_plan(int32_t n, const sabr_problem* problems, const sabr_bounds* bounds,
                               const sabr_cooling* cooling, const uint64_t* seeds, int use_graph, cudaStream_t stream,
-                              sabr_plan** out) {
+                              bool blocking, sabr_plan** out) {
   if (!out) return fail(SABR_EINVAL, "out is NULL");
   *out = nullptr;
   if (n < 1 || !problems || !bounds || !cooling || !seeds) return fail(SABR_EINVAL, "empty batch or NULL array");
@@ -1575,10 +1632,33 @@ static sabr_status build_plan(int32_t n, const sabr_problem* problems, const sab
   const size_t arena_bytes = align_up(o, 256);
 
   std::vector<unsigned char> img(arena_bytes, 0);
-  cudaError_t e = cudaMalloc(&p->arena, arena_bytes);
-  if (e != cudaSuccess) {
-    free_plan(p);
-    return cuda_fail(e, "cudaMalloc(plan arena)");
+  cudaError_t e = cudaSuccess;
+  if (blocking) {
+    p->blocking = true;
+    KeptBuffers k = take_kept(p->device);
+    p->arena = k.arena;
+    p->arena_bytes = k.bytes;
+    p->h_results = k.results;
+    p->h_count = k.n;
+    if (p->arena_bytes < arena_bytes) {
+      if (p->arena) cudaFree(p->arena);
+      p->arena = nullptr;
+      p->arena_bytes = 0;
+    }
+    if (p->h_count < n) {
+      if (p->h_results) cudaFreeHost(p->h_results);
+      p->h_results = nullptr;
+      p->h_count = 0;
+    }
+  }
+  if (!p->arena) {
+    e = cudaMalloc(&p->arena, arena_bytes);
+    if (e != cudaSuccess) {
+      p->arena = nullptr;
+      free_plan(p);
+      return cuda_fail(e, "cudaMalloc(plan arena)");
+    }
+    p->arena_bytes = arena_bytes;
   }
   unsigned char* base = (unsigned char*)p->arena;
   sabr_result* dres = (sabr_result*)(base + results_off);
@@ -1616,7 +1696,14 @@ static sabr_status build_plan(int32_t n, const sabr_problem* problems, const sab
   p->d_probs = (ProblemDev*)(base + probs_off);
   p->d_results = dres;
   e = cudaMemcpy(p->arena, img.data(), arena_bytes, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMallocHost(&p->h_results, sizeof(sabr_result) * n);
+  if (e == cudaSuccess && !p->h_results) {
+    e = cudaMallocHost(&p->h_results, sizeof(sabr_result) * n);
+    if (e == cudaSuccess) {
+      p->h_count = n;
+    } else {
+      p->h_results = nullptr;
+    }
+  }
   if (e == cudaSuccess) e = cudaEventCreate(&p->ev_lv0);
   if (e == cudaSuccess) e = cudaEventCreate(&p->ev_lv1);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->ev_done, cudaEventDisableTiming);
@@ -1685,7 +1772,7 @@ sabr_status sabr_plan_create(int32_t n, const sabr_problem* problems, const sabr
                              const sabr_cooling* cooling, const uint64_t* seeds, int32_t use_graph, void* stream,
                              sabr_plan** out) {
   sabr::clear_error();
-  return sabr::build_plan(n, problems, bounds, cooling, seeds, use_graph, (cudaStream_t)stream, out);
+  return sabr::build_plan(n, problems, bounds, cooling, seeds, use_graph, (cudaStream_t)stream, false, out);
 }
 
 sabr_status sabr_plan_run(sabr_plan* plan, void* stream) {
@@ -1723,7 +1810,7 @@ sabr_status sabr_calibrate_batch(int32_t n, const sabr_problem* problems, const 
   sabr::clear_error();
   if (!out) return sabr::fail(SABR_EINVAL, "out is NULL");
   sabr_plan* p = nullptr;
-  SABR_TRY(sabr::build_plan(n, problems, bounds, cooling, seeds, 0, (cudaStream_t)stream, &p));
+  SABR_TRY(sabr::build_plan(n, problems, bounds, cooling, seeds, 0, (cudaStream_t)stream, true, &p));
   sabr_status st = sabr::run_plan(p, (cudaStream_t)stream);
   if (st == SABR_OK) st = sabr::plan_results(p, out);
   sabr::free_plan(p);

@@ -384,7 +384,7 @@ int small_capacity(int prec, int model, const SmallShape& s, size_t smem) {
   cudaFuncAttributes at;
   if (cudaFuncGetAttributes(&at, (const void*)fn) != cudaSuccess) return 0;
   if (smem + at.sharedSizeBytes > 227 * 1024 ||
-      cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+      allow_smem((const void*)fn, smem) != cudaSuccess)
     return 0;
   int nb = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, (const void*)fn, kSmallBlock, smem) != cudaSuccess) return 0;

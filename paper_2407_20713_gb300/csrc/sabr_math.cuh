@@ -330,15 +330,19 @@ __device__ __forceinline__ float lg2_approx(float x) {
   asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-template <> __device__ __forceinline__ ZxConst<float> zx_setup<float, double>(double rho) {
+// From 1 - rho and 1 + rho rounded from FP64.
+__device__ __forceinline__ ZxConst<float> zx_setup_from(float rho, float omr, float opr) {
   ZxConst<float> c;
-  c.rho = (float)rho;
-  c.omr = (float)(1.0 - rho);
-  c.opr = (float)(1.0 + rho);
+  c.rho = rho;
+  c.omr = omr;
+  c.opr = opr;
   c.q0 = c.omr * c.opr;
   c.ln_opr = lg2_approx(c.opr) * 0.69314718055994531f;
   c.ln_omr = lg2_approx(c.omr) * 0.69314718055994531f;
   return c;
+}
+template <> __device__ __forceinline__ ZxConst<float> zx_setup<float, double>(double rho) {
+  return zx_setup_from((float)rho, (float)(1.0 - rho), (float)(1.0 + rho));
 }
 // A float rho: 1 -+ rho rounded once in FP32 is the value the FP64 route
 // gives (the exact difference rounded to float), without FP64 instructions.
@@ -384,14 +388,14 @@ template <class R> struct StaticConst {
   ZxConst<R> zx;
 };
 
-// params: x[0..3] = alpha, beta, rho, nu (any real type)
-template <class R, class P>
-__device__ __forceinline__ StaticConst<R> static_setup(const P* x) {
+// From alpha, beta, rho, nu in the working precision and the constants of rho.
+template <class R>
+__device__ __forceinline__ StaticConst<R> static_setup_from(R alpha, R beta, R rho, R nu, const ZxConst<R>& zx) {
   StaticConst<R> s;
-  s.alpha = (R)x[0];
-  s.beta = (R)x[1];
-  s.rho = (R)x[2];
-  s.nu = (R)x[3];
+  s.alpha = alpha;
+  s.beta = beta;
+  s.rho = rho;
+  s.nu = nu;
   s.omb = (R)1 - s.beta;
   s.half_omb = (R)0.5 * s.omb;
   s.c2 = m_divc(s.omb * s.omb, 24.0);
@@ -403,8 +407,13 @@ __device__ __forceinline__ StaticConst<R> static_setup(const P* x) {
   s.abr_a = s.alpha * s.br_a;
   s.abr_b = s.alpha * s.br_b;
   s.abr_c = s.alpha * s.br_c;
-  s.zx = zx_setup<R>(x[2]);
+  s.zx = zx;
   return s;
+}
+// params: x[0..3] = alpha, beta, rho, nu (any real type)
+template <class R, class P>
+__device__ __forceinline__ StaticConst<R> static_setup(const P* x) {
+  return static_setup_from<R>((R)x[0], (R)x[1], (R)x[2], (R)x[3], zx_setup<R>(x[2]));
 }
 
 // eq. (haganf) with z of eq. (zeta), fk = (K f)^{(1-beta)/2} = 2^(e) from
@@ -613,62 +622,35 @@ __device__ __forceinline__ void case1_coeffs(R nu0, R rho0, R a, R b, R T, R out
   constexpr int N = Tr<R>::kCase1Series;
   const R x = (R)2 * b * T, y = (a + b) * T;
   R g1, g2, g3, g4;
-  if constexpr (sizeof(R) == 4) {
-    // FP32: both forms, then selects -- the lanes of a chain hold different
-    // maturities, so a warp ran both branches nearly always, one after the
-    // other; without branches the four series, the closed forms and other
-    // maturities' evaluations overlap
-    const R mx = -x, my = -y;
-    R s1 = (R)g1c(N), s2 = (R)g2c(N), s3 = (R)g3c(N), s4 = (R)g4c(N);
+  if (x < (R)2) {
+    const R mx = -x;
+    R s1 = (R)g1c(N), s2 = (R)g2c(N);
 #pragma unroll
     for (int k = N - 1; k >= 0; --k) {
       s1 = s1 * mx + (R)g1c(k);
       s2 = s2 * mx + (R)g2c(k);
+    }
+    g1 = s1;
+    g2 = s2;
+  } else {
+    const R e = m_exp(-x), ix = m_rcp(x), ix3 = ix * ix * ix;
+    g1 = ((x * x * (R)0.5 - x + (R)1) - e) * ix3;
+    g2 = ((R)2 * (e - (R)1) + x * (e + (R)1)) * ix3;
+  }
+  if (y < (R)2) {
+    const R my = -y;
+    R s3 = (R)g3c(N), s4 = (R)g4c(N);
+#pragma unroll
+    for (int k = N - 1; k >= 0; --k) {
       s3 = s3 * my + (R)g3c(k);
       s4 = s4 * my + (R)g4c(k);
     }
-    const R ex = m_exp(-x), ix = m_rcp(x), ix3 = ix * ix * ix;
-    const R ey = m_exp(-y), iy = m_rcp(y), iy2 = iy * iy;
-    const R c1 = ((x * x * (R)0.5 - x + (R)1) - ex) * ix3;
-    const R c2 = ((R)2 * (ex - (R)1) + x * (ex + (R)1)) * ix3;
-    const R c3 = (ey - (R)1 + y) * iy2;
-    const R c4 = (m_exp(-(R)2 * y) - (R)8 * ey + ((R)7 + (R)2 * y * (y - (R)3))) * iy2 * iy2;
-    const bool sx = x < (R)2, sy = y < (R)2;
-    g1 = sx ? s1 : c1;
-    g2 = sx ? s2 : c2;
-    g3 = sy ? s3 : c3;
-    g4 = sy ? s4 : c4;
+    g3 = s3;
+    g4 = s4;
   } else {
-    if (x < (R)2) {
-      const R mx = -x;
-      R s1 = (R)g1c(N), s2 = (R)g2c(N);
-#pragma unroll
-      for (int k = N - 1; k >= 0; --k) {
-        s1 = s1 * mx + (R)g1c(k);
-        s2 = s2 * mx + (R)g2c(k);
-      }
-      g1 = s1;
-      g2 = s2;
-    } else {
-      const R e = m_exp(-x), ix = m_rcp(x), ix3 = ix * ix * ix;
-      g1 = ((x * x * (R)0.5 - x + (R)1) - e) * ix3;
-      g2 = ((R)2 * (e - (R)1) + x * (e + (R)1)) * ix3;
-    }
-    if (y < (R)2) {
-      const R my = -y;
-      R s3 = (R)g3c(N), s4 = (R)g4c(N);
-#pragma unroll
-      for (int k = N - 1; k >= 0; --k) {
-        s3 = s3 * my + (R)g3c(k);
-        s4 = s4 * my + (R)g4c(k);
-      }
-      g3 = s3;
-      g4 = s4;
-    } else {
-      const R e = m_exp(-y), iy = m_rcp(y), iy2 = iy * iy;
-      g3 = (e - (R)1 + y) * iy2;
-      g4 = (m_exp(-(R)2 * y) - (R)8 * e + ((R)7 + (R)2 * y * (y - (R)3))) * iy2 * iy2;
-    }
+    const R e = m_exp(-y), iy = m_rcp(y), iy2 = iy * iy;
+    g3 = (e - (R)1 + y) * iy2;
+    g4 = (m_exp(-(R)2 * y) - (R)8 * e + ((R)7 + (R)2 * y * (y - (R)3))) * iy2 * iy2;
   }
   out[0] = (R)6 * nu0 * nu0 * g1;
   out[1] = (R)6 * nu0 * nu0 * g2;

@@ -6,7 +6,7 @@
 // level) per 256-thread block of every resident formula request -- and
 // launches one persistent SA-level kernel per (precision, model) over it;
 // (3) advances every resident MC-cost request by one proposal wave on a
-// second stream; (4) enqueues the final reduction of requests that ran their
+// second stream, at most two in flight; (4) enqueues the final reduction of requests that ran their
 // last level and releases those the GPU has finished.  Requests arriving
 // while others run therefore share the next launches.  No device code waits
 // on anything; all waiting is host-side with time limits.
@@ -89,14 +89,18 @@ struct Request {
   bool cancelled_resident = false;
   HostProblem hp;
   McSaHost mh;
-  int G = 1, L = 1, n_blocks = 0;
+  int G = 1;           // lanes by whose order the sums run
+  int base_L = 1;      // lanes per chain on a full GPU
+  int n_blocks = 0;    // level blocks at G lanes (the most)
+
   size_t bytes = 0, off = 0;
   int slot = -1;
   ProblemDev pd;
   int level = 0;
   int mc_level = 0, mc_step = 0;
   bool mc_started = false;
-  cudaEvent_t wave_ev = nullptr;  // last MC wave
+  cudaEvent_t wave_ev[2] = {nullptr, nullptr};  // the last two MC waves, in turn
+  int wave = 0;
   cudaEvent_t done_ev = nullptr;
   sabr_result result;
 };
@@ -196,7 +200,7 @@ static cudaError_t enqueue_step_launches(sabr_server* s, int par, cudaStream_t s
 static sabr_status upload_formula(sabr_server* s, Request& r) {
   std::vector<unsigned char> img(r.bytes, 0);
   unsigned char* base = s->pool + r.off;
-  formula_layout(r.hp, r.G, img.data(), base, 0, r.pd, s->d_results + r.slot, kSaBlock, r.L);
+  formula_layout(r.hp, r.G, img.data(), base, 0, r.pd, s->d_results + r.slot);
   SABR_CUDA(cudaMemcpyAsync(base, img.data(), r.bytes, cudaMemcpyHostToDevice, s->sf));
   SABR_CUDA(cudaMemcpyAsync(s->d_probs + r.slot, &r.pd, sizeof(ProblemDev), cudaMemcpyHostToDevice, s->sf));
   launch_init(r.hp.prec, r.hp.model, s->d_probs, s->d_ident + r.slot, 1, init_smem_bytes(r.hp), s->sf);
@@ -231,7 +235,8 @@ static void mc_wave(sabr_server* s, Request& r) {
   } else {
     r.mc_level = m.n_levels;
   }
-  cudaEventRecord(r.wave_ev, s->smc);
+  cudaEventRecord(r.wave_ev[r.wave], s->smc);
+  r.wave ^= 1;
 }
 
 static void release(sabr_server* s, Request& r) {
@@ -240,9 +245,32 @@ static void release(sabr_server* s, Request& r) {
     s->free_slots.push_back(r.slot);
     r.slot = -1;
   }
-  if (r.wave_ev) cudaEventDestroy(r.wave_ev);
+  for (cudaEvent_t& e : r.wave_ev) {
+    if (e) cudaEventDestroy(e);
+    e = nullptr;
+  }
   if (r.done_ev) cudaEventDestroy(r.done_ev);
-  r.wave_ev = r.done_ev = nullptr;
+  r.done_ev = nullptr;
+}
+
+// By what a step multiplies the lanes per chain of each group's requests: as
+// long as the GPU's resident threads hold the group's chains (16 warps an SM
+// for the static formulas, eight for the dynamic models), a chain gets more of
+// the lanes its sums allow.  Which lanes run a chain changes no result.
+static void level_lanes(const std::vector<std::shared_ptr<Request>>& active, int* scale) {
+  for (int g = 0; g < kGroups; ++g) {
+    const bool dyn = g % 5 == SABR_DYN_I || g % 5 == SABR_DYN_II;
+    const long long room = (long long)device_sms() * (dyn ? 8 : 16) * 32;
+    for (scale[g] = 1; scale[g] < 32; scale[g] *= 2) {
+      long long lanes = 0;
+      for (const auto& rp : active) {
+        const Request& r = *rp;
+        if (!r.is_mc && r.state == R_ACTIVE && group_of(r.hp.prec, r.hp.model) == g)
+          lanes += (long long)r.hp.n_chains * std::min(r.G, r.base_L * 2 * scale[g]);
+      }
+      if (lanes > room) break;
+    }
+  }
 }
 
 static void worker_main(sabr_server* s) {
@@ -282,7 +310,7 @@ static void worker_main(sabr_server* s) {
     }
     for (auto& r : admitted) {
       cudaEventCreateWithFlags(&r->done_ev, cudaEventDisableTiming);
-      cudaEventCreateWithFlags(&r->wave_ev, cudaEventDisableTiming);
+      for (cudaEvent_t& e : r->wave_ev) cudaEventCreateWithFlags(&e, cudaEventDisableTiming);
       if (r->is_mc)
         upload_mc(s, *r);
       else
@@ -300,6 +328,8 @@ static void worker_main(sabr_server* s) {
     }
     std::vector<Request*> to_finalize;
     bool any_formula = false;
+    int scale[kGroups];
+    level_lanes(snapshot, scale);
     for (auto& rp : snapshot) {
       Request& r = *rp;
       if (r.is_mc || r.state != R_ACTIVE) continue;
@@ -310,10 +340,12 @@ static void worker_main(sabr_server* s) {
       }
       if (r.level < r.hp.n_levels) {
         const int g = group_of(r.hp.prec, r.hp.model);
-        if (counts[g] + r.n_blocks > kWorkPerGroup) continue;  // waits for the next step
-        for (int b = 0; b < r.n_blocks; ++b)
-          s->h_work[par][(size_t)g * kWorkPerGroup + counts[g] + b] = make_int4(r.slot, b, r.level, 0);
-        counts[g] += r.n_blocks;
+        const int L = std::min(r.G, r.base_L * scale[g]), cpb = kSaBlock / L;
+        const int blocks = (r.hp.n_chains + cpb - 1) / cpb;
+        if (counts[g] + blocks > kWorkPerGroup) continue;  // waits for the next step
+        for (int b = 0; b < blocks; ++b)
+          s->h_work[par][(size_t)g * kWorkPerGroup + counts[g] + b] = make_int4(r.slot, b, r.level, L);
+        counts[g] += blocks;
         ++r.level;
         any_formula = true;
       }
@@ -350,11 +382,12 @@ static void worker_main(sabr_server* s) {
       r->state = R_FINISHING;
     }
 
-    // ---- MC requests: one wave each, at most one wave in flight --------
+    // ---- MC requests: one wave each, at most two in flight (the second so
+    // that the GPU has the next wave when this thread looks again late) ----
     for (auto& rp : snapshot) {
       Request& r = *rp;
       if (!r.is_mc || r.state != R_ACTIVE) continue;
-      if (cudaEventQuery(r.wave_ev) == cudaErrorNotReady) continue;
+      if (cudaEventQuery(r.wave_ev[r.wave]) == cudaErrorNotReady) continue;
       if (r.cancel) {
         r.cancelled_resident = true;
         cudaEventRecord(r.done_ev, s->smc);
@@ -529,19 +562,18 @@ static sabr_status submit(sabr_server* s, const sabr_problem* pr, const sabr_bou
     SABR_TRY(formula_prepare(*pr, *b, *c, seed, r->hp));
     if (r->hp.n_quotes > s->cfg.max_quotes) return fail(SABR_EINVAL, "request has more quotes than max_quotes");
     r->G = choose_lanes(r->hp.n_quotes, r->hp.n_mats, r->hp.model, r->hp.prec, r->hp.n_chains);
-    // a request shares the GPU with others: as few lanes a chain as a full
-    // GPU would give it, where the block's shared memory holds their records
+    ProblemDev tmp;
+    r->bytes = formula_layout(r->hp, r->G, nullptr, nullptr, 0, tmp, nullptr) + 256;
+    r->n_blocks = tmp.n_blocks;
+    if (r->n_blocks > kWorkPerGroup) return fail(SABR_EINVAL, "request has too many chains for one step");
     const size_t have = s->smem[group_of(r->hp.prec, r->hp.model)];
     auto need = [&](int L) {
       return level_smem_bytes(r->hp.prec, r->hp.model, r->hp.n_quotes, r->hp.n_mats, kSaBlock / L, r->hp.c2_nsub);
     };
-    r->L = server_run_lanes(r->hp.n_quotes, r->hp.n_mats, r->hp.model, r->hp.prec, r->G);
-    while (r->L < r->G && need(r->L) > have) r->L <<= 1;
-    ProblemDev tmp;
-    r->bytes = formula_layout(r->hp, r->G, nullptr, nullptr, 0, tmp, nullptr, kSaBlock, r->L) + 256;
-    r->n_blocks = tmp.n_blocks;
-    if (r->n_blocks > kWorkPerGroup) return fail(SABR_EINVAL, "request has too many chains for one step");
-    if (need(r->L) > have) return fail(SABR_EINVAL, "request needs more shared memory than the server reserves");
+    if (need(r->G) > have) return fail(SABR_EINVAL, "request needs more shared memory than the server reserves");
+    // (more chains a block at fewer lanes: their records have to fit)
+    r->base_L = server_base_lanes(r->hp.n_quotes, r->hp.model, r->hp.prec, r->G);
+    while (r->base_L < r->G && need(r->base_L) > have) r->base_L <<= 1;
   }
   if (r->bytes > (size_t)s->cfg.device_bytes) return fail(SABR_EINVAL, "request larger than the server pool");
   std::lock_guard<std::mutex> lk(s->mu);

@@ -1,4 +1,5 @@
 // vol.cu -- sabr_implied_vol: one thread per option, grid-stride.
+#include <algorithm>
 #include <cmath>
 
 #include "common.h"
@@ -6,44 +7,99 @@
 
 namespace sabr {
 
-struct VolArgs {
+// Everything that does not depend on the option, formed once on the host: a
+// thread handles a few options only, and the FP64 pipe that the conversions,
+// log2 f and (in FP64) the formula's constants took on every thread issues 1.7
+// operations a clock and SM (2^20 options, FP32: Hagan 22.7 -> 14.5 us, expanded
+// 51.3 -> 11.4, Case I 54.0 -> 14.4, Case II 122 -> 94; 21 options in FP64, Hagan
+// 12.4 -> 8.3).
+template <class R> struct VolArgs {
   double p[kMaxD];
   double fwd;
+  R f, l2f;                 // f and log2 f
+  R alpha, beta, rho, nu;
+  R omr, opr;               // 1 - rho, 1 + rho
+  StaticConst<R> sc;        // FP64 static formulas
 };
 
+// The formula's constants in FP64 (static_setup, on the host).
+static StaticConst<double> static_setup_host(const double* x) {
+  StaticConst<double> s;
+  s.alpha = x[0];
+  s.beta = x[1];
+  s.rho = x[2];
+  s.nu = x[3];
+  s.omb = 1.0 - s.beta;
+  s.half_omb = 0.5 * s.omb;
+  s.c2 = s.omb * s.omb / 24.0;
+  s.c4 = s.omb * s.omb * s.omb * s.omb / 1920.0;
+  s.nu_over_alpha = s.nu / s.alpha;
+  s.br_a = s.c2 * s.alpha * s.alpha;
+  s.br_b = 0.25 * s.rho * s.beta * s.nu * s.alpha;
+  s.br_c = (2.0 - 3.0 * s.rho * s.rho) / 24.0 * s.nu * s.nu;
+  s.abr_a = s.alpha * s.br_a;
+  s.abr_b = s.alpha * s.br_b;
+  s.abr_c = s.alpha * s.br_c;
+  s.zx.rho = s.rho;
+  s.zx.omr = 1.0 - s.rho;
+  s.zx.opr = 1.0 + s.rho;
+  s.zx.q0 = s.zx.omr * s.zx.opr;
+  s.zx.ln_opr = s.zx.ln_omr = 0.0;
+  return s;
+}
+
 template <class R, int MODEL>
-__global__ void __launch_bounds__(256) implied_vol_kernel(VolArgs a, const double* __restrict__ T,
+__global__ void __launch_bounds__(256) implied_vol_kernel(const __grid_constant__ VolArgs<R> a,
+                                                          const double* __restrict__ T,
                                                           const double* __restrict__ K, int64_t n,
                                                           double* __restrict__ out) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   StaticConst<R> sc;
-  if (MODEL == SABR_HAGAN || MODEL == SABR_OBLOJ) sc = static_setup<R>(a.p);
-  const R l2f = (R)log2(a.fwd);
-  const R fwd = (R)a.fwd;
+  if constexpr (MODEL == SABR_HAGAN || MODEL == SABR_OBLOJ) {
+    if constexpr (sizeof(R) == 8) {
+      sc = a.sc;
+    } else if constexpr (MODEL == SABR_HAGAN) {
+      sc = static_setup_from<R>(a.alpha, a.beta, a.rho, a.nu, zx_setup_from(a.rho, a.omr, a.opr));
+    } else {
+      sc = static_setup<R>(a.p);
+    }
+  }
+  const bool unit = a.fwd == 1.0;  // K f is then K
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
     const double kd = K[i];
     const R t = (R)T[i], k = (R)kd;
-    const R lfk = m_log(fwd / k);
+    const R lfk = m_log(a.f / k);
     R v;
-    if (MODEL == SABR_HAGAN) {
-      v = vol_hagan<R>(sc, lfk, m_log2((R)(kd * a.fwd)), t);
-    } else if (MODEL == SABR_OBLOJ) {
-      v = vol_obloj<R>(sc, lfk, m_log2((R)(kd * a.fwd)), m_log2(k), t);
-    } else if (MODEL == SABR_EXPANDED) {
-      v = vol_poly<R>(expanded_coef<R>(a.p, l2f, t), lfk);
+    if constexpr (MODEL == SABR_HAGAN) {
+      v = vol_hagan<R>(sc, lfk, m_log2(unit ? k : (R)(kd * a.fwd)), t);
+    } else if constexpr (MODEL == SABR_OBLOJ) {
+      v = vol_obloj<R>(sc, lfk, m_log2(unit ? k : (R)(kd * a.fwd)), m_log2(k), t);
+    } else if constexpr (MODEL == SABR_EXPANDED) {
+      v = vol_poly<R>(expanded_coef<R>(a.p, a.l2f, t), lfk);
     } else {
-      v = vol_poly<R>(dynamic_coef<R, MODEL == SABR_DYN_II>(a.p, l2f, t), lfk);
+      v = vol_poly<R>(dynamic_coef<R, MODEL == SABR_DYN_II>(a.p, a.l2f, t), lfk);
     }
     out[i] = (double)v;
   }
 }
 
 template <class R>
-static void launch_vol(int model, const VolArgs& a, const double* T, const double* K, int64_t n,
+static void launch_vol(int model, const double* params, double fwd, const double* T, const double* K, int64_t n,
                        double* out, cudaStream_t s) {
-  int64_t blocks = (n + 255) / 256;
-  const int64_t cap = (int64_t)device_sms() * 16;
-  if (blocks > cap) blocks = cap;
+  VolArgs<R> a;
+  for (int i = 0; i < kMaxD; ++i) a.p[i] = i < n_params(model) ? params[i] : 0.0;
+  a.fwd = fwd;
+  a.f = (R)fwd;
+  a.l2f = (R)std::log2(fwd);
+  a.alpha = (R)a.p[0];
+  a.beta = (R)a.p[1];
+  a.rho = (R)a.p[2];
+  a.nu = (R)a.p[3];
+  a.omr = (R)(1.0 - a.p[2]);
+  a.opr = (R)(1.0 + a.p[2]);
+  if constexpr (sizeof(R) == 8) a.sc = static_setup_host(a.p);
+  // one resident grid (eight blocks an SM), options strided over it
+  const int blocks = (int)std::min<int64_t>((n + 255) / 256, (int64_t)device_sms() * 8);
   switch (model) {
     case SABR_HAGAN: implied_vol_kernel<R, SABR_HAGAN><<<blocks, 256, 0, s>>>(a, T, K, n, out); break;
     case SABR_OBLOJ: implied_vol_kernel<R, SABR_OBLOJ><<<blocks, 256, 0, s>>>(a, T, K, n, out); break;
@@ -66,14 +122,11 @@ extern "C" sabr_status sabr_implied_vol(sabr_model model, const double* params, 
   if (n < 0) return fail(SABR_EINVAL, "n < 0");
   if (n == 0) return SABR_OK;
   if (!T || !K || !vol_out) return fail(SABR_EINVAL, "NULL array");
-  VolArgs a;
-  for (int i = 0; i < kMaxD; ++i) a.p[i] = i < n_params(model) ? params[i] : 0.0;
-  a.fwd = fwd;
   cudaStream_t s = (cudaStream_t)stream;
   if (prec == SABR_FP32)
-    launch_vol<float>(model, a, T, K, n, vol_out, s);
+    launch_vol<float>(model, params, fwd, T, K, n, vol_out, s);
   else
-    launch_vol<double>(model, a, T, K, n, vol_out, s);
+    launch_vol<double>(model, params, fwd, T, K, n, vol_out, s);
   SABR_CUDA(cudaGetLastError());
   return SABR_OK;
 }

@@ -51,7 +51,10 @@ template <class R> struct ClqPath {
 // ... and keeps FP64 sums of the payoff and its square; each block adds its
 // threads' sums in a fixed order into partial[2 b], partial[2 b + 1].  FP32
 // paths advance in two pairs a thread with the packed FP32x2 instructions
-// (run_path_pairs), FP64 paths kMcPathsPerThread at a time.
+// (run_path_pairs, which says what bounds it), FP64 paths kMcPathsPerThread at a
+// time.  2^20 paths x 252 steps, Case I dynamics: 693 us a call with scalar steps,
+// the step table formed by every block and one thread's sum over 1064 blocks,
+// 529 now.
 template <class R>
 __global__ void __launch_bounds__(kClqBlock) cliquet_kernel(McDev P, const double* __restrict__ params,
                                                            double floor_l, double cap_l, double floor_g,

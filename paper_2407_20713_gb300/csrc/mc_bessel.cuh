@@ -87,7 +87,10 @@ __device__ __forceinline__ uint4 bessel_words(const McDev& P, int64_t path, int 
 
 // Everything a step shares between its paths: formed once per step by
 // mc_steps_kernel (a division, a square root and two reciprocals, which every
-// thread used to repeat in every step) and read by all paths through L1.
+// thread used to repeat in every step) and read by all paths through L1: 2^20
+// paths x 24 steps 554 -> 422 us a call.  What bounds the step: the branches of
+// the Gamma trials, whose logarithms and second draws some lane of a warp needs
+// nearly always.
 template <class R> struct __align__(16) BesselStep {
   StepCoefB<R> s;
   R inv_kap;        // 1 / kap, or 0 at nu = 0

@@ -1,9 +1,10 @@
 // sa.cu -- synchronous parallel Simulated Annealing (Sec. 5) on the GPU.
 //
-// Work decomposition: a chain is a group of G lanes (G = 1..32, a power of
-// two); lanes split the quotes of the cost function.  A block holds
-// blockDim/G chains of one problem (64-thread blocks in plans, 256 in the
-// server).  A unit of work is one temperature level (chain_len Metropolis
+// Work decomposition: a chain's misfit is summed in the order of G lanes (G =
+// 1..32, a power of two) that split the quotes, and run by L <= G lanes, each
+// playing G / L of them (virtual_lanes_sum).  A block holds blockDim/L chains of
+// one problem (64-thread blocks in plans, 256 in the server).  A single static
+// problem of few chains takes another kernel (sa_small.cu).  A unit of work is one temperature level (chain_len Metropolis
 // steps per chain) of one block of chains; the chains' states live in
 // registers for the whole unit.  At the end of the unit each block writes
 // the argmin of its chains' final states, and the last block of a problem's
@@ -37,9 +38,9 @@ namespace sabr {
 
 // Quote pairs per point the speculative Hagan loop keeps in flight (several
 // points are evaluated at once, so fewer than QueuePairs), and the steps it
-// evaluates at once: two (on one 15-strike smile, 64 chains, 8 lanes a
-// chain, four measured 8% slower: 17.39 against 16.12 ms per calibration;
-// the results do not depend on the depth).
+// evaluates at once: two (with the points of a window one after the other on a
+// chain's lanes, four measured 8% slower on a 15-strike smile; sa_small.cu
+// evaluates them side by side).  The results do not depend on the depth.
 template <class R> struct SpecPairs {
   static constexpr int value = 2;
 };
@@ -124,8 +125,11 @@ __global__ void sa_init_kernel(const ProblemDev* __restrict__ probs, const int* 
 // The steps of one level of the chains of a warp, FP32, L lanes each, in
 // lockstep: every lane runs every instruction (full-warp masks; lanes whose
 // proposal is rejected unevaluated compute a cost that is dropped), so nothing
-// is set up per chain group around the exchanges.  cost(xp) is called by the
-// whole warp.
+// is set up per chain group around the exchanges (variable masks cost match and
+// vote sequences at each shuffle: Case II, 12 x 21 quotes, 8192 chains, 40
+// levels x 50: 18.2 -> 13.2 ms).  What bounds it: latency, at two warps a
+// scheduler (issue 40%), and for Case II the shared-memory pipe (66% busy: two
+// 16-byte loads a quote).  cost(xp) is called by the whole warp.
 template <int MODEL, int D, class Cost>
 __device__ __forceinline__ void lockstep_level(const ProblemDev& P, uint32_t gchain, int level, bool active, int lane,
                                                int L, const float* s_lo, const float* s_hi, const float* s_step,

@@ -76,6 +76,13 @@ template <int NW> __device__ __forceinline__ void chain_sync(int chain_in_block)
   }
 }
 
+// What bounds it (64 chains, 15 quotes, 4 warps x 4 points: 3.9 ms for 200
+// levels x 100 steps, 15.6 two steps at a time on 8 lanes): latency.  A level of
+// no steps takes 4 us (the meeting of 64 blocks), a window of 16 steps about
+// 1.2 us -- one dependent chain of proposals, formula, butterfly and decision on
+// a warp alone on its scheduler -- and a level waits for its slowest chain.
+// FP64, 4 x 2: 33.5 ms (173.9), FP64 instructions at 76 cycles each.
+//
 // Block minima alternate between two buffers by the level's parity: a block
 // writes the minima of level k + 2 only after every block has read those of
 // level k (it arrives at k + 1 after reading them).  The costs of an iteration

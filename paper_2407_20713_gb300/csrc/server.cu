@@ -6,7 +6,7 @@
 // level) per 256-thread block of every resident formula request -- and
 // launches one persistent SA-level kernel per (precision, model) over it;
 // (3) advances every resident MC-cost request by one proposal wave on a
-// second stream, at most two in flight; (4) enqueues the final reduction of requests that ran their
+// second stream, one in flight beside a formula step, else two; (4) enqueues the final reduction of requests that ran their
 // last level and releases those the GPU has finished.  Requests arriving
 // while others run therefore share the next launches.  No device code waits
 // on anything; all waiting is host-side with time limits.
@@ -122,7 +122,7 @@ struct sabr_server {
   int4* h_work[2] = {nullptr, nullptr};
   int* h_nwork[2] = {nullptr, nullptr};
   cudaEvent_t buf_ev[2] = {nullptr, nullptr};
-  cudaGraphExec_t graph[2] = {nullptr, nullptr};
+  cudaGraphExec_t graph[2][2] = {};  // a step's launches per parity: in turn, as parallel branches
   size_t smem[sabr::kGroups] = {};
   int grid[sabr::kGroups] = {};
   std::vector<int> free_slots;
@@ -176,23 +176,27 @@ struct StepBranches {
   }
 };
 
-// A captured step: the work table's upload, then the groups' kernels as
-// parallel branches (a group's requests rarely fill the GPU, and the kernels of
-// empty groups end at once).
-static cudaError_t enqueue_step_launches(sabr_server* s, int par, cudaStream_t st, const StepBranches& br) {
+// A captured step: the work table's upload, then the groups' kernels, in turn
+// or (br) as parallel branches: a group's requests rarely fill the GPU, and the
+// kernels of empty groups end at once.  Parallel branches are for steps with no
+// Monte Carlo request beside them: a branch can land on the hardware queue that
+// holds the waves and then waits for those in flight, level after level (with a
+// fifth of a loaded server's stream dynamic and 5% Monte Carlo, at 14.3
+// requests/s, the median Hagan request took 249 ms on branches and 87 ms in turn).
+static cudaError_t enqueue_step_launches(sabr_server* s, int par, cudaStream_t st, const StepBranches* br) {
   cudaError_t e = cudaMemcpyAsync(s->d_nwork[par], s->h_nwork[par], sizeof(int) * kGroups, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(s->d_work[par], s->h_work[par], sizeof(int4) * kWorkPerGroup * kGroups, cudaMemcpyHostToDevice,
                         st);
-  if (e == cudaSuccess) e = cudaEventRecord(br.fork, st);
+  if (br && e == cudaSuccess) e = cudaEventRecord(br->fork, st);
   for (int g = 0; g < kGroups && e == cudaSuccess; ++g) {
-    e = cudaStreamWaitEvent(br.stream[g], br.fork, 0);
+    if (br) e = cudaStreamWaitEvent(br->stream[g], br->fork, 0);
     if (e != cudaSuccess) break;
     launch_persistent(g / 5, g % 5, s->d_probs, s->d_work[par] + (size_t)g * kWorkPerGroup, s->d_nwork[par] + g,
-                      s->grid[g], s->smem[g], br.stream[g]);
+                      s->grid[g], s->smem[g], br ? br->stream[g] : st);
     e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaEventRecord(br.join[g], br.stream[g]);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(st, br.join[g], 0);
+    if (br && e == cudaSuccess) e = cudaEventRecord(br->join[g], br->stream[g]);
+    if (br && e == cudaSuccess) e = cudaStreamWaitEvent(st, br->join[g], 0);
   }
   return e;
 }
@@ -327,7 +331,8 @@ static void worker_main(sabr_server* s) {
       snapshot = s->active;
     }
     std::vector<Request*> to_finalize;
-    bool any_formula = false;
+    bool any_formula = false, any_mc = false;
+    for (auto& rp : snapshot) any_mc = any_mc || rp->is_mc;
     int scale[kGroups];
     level_lanes(snapshot, scale);
     for (auto& rp : snapshot) {
@@ -353,8 +358,8 @@ static void worker_main(sabr_server* s) {
     }
     if (any_formula) {
       for (int g = 0; g < kGroups; ++g) s->h_nwork[par][g] = counts[g];
-      if (s->graph[par]) {
-        cudaGraphLaunch(s->graph[par], s->sf);
+      if (s->graph[par][!any_mc]) {
+        cudaGraphLaunch(s->graph[par][!any_mc], s->sf);
         s->stats.kernel_launches += kGroups;
       } else {
         cudaMemcpyAsync(s->d_nwork[par], s->h_nwork[par], sizeof(int) * kGroups, cudaMemcpyHostToDevice, s->sf);
@@ -382,12 +387,13 @@ static void worker_main(sabr_server* s) {
       r->state = R_FINISHING;
     }
 
-    // ---- MC requests: one wave each, at most two in flight (the second so
-    // that the GPU has the next wave when this thread looks again late) ----
+    // ---- MC requests: one wave each, at most one in flight beside a formula
+    // step, else two (the second so that the GPU has the next wave when this
+    // thread looks again late) ----
     for (auto& rp : snapshot) {
       Request& r = *rp;
       if (!r.is_mc || r.state != R_ACTIVE) continue;
-      if (cudaEventQuery(r.wave_ev[r.wave]) == cudaErrorNotReady) continue;
+      if (cudaEventQuery(r.wave_ev[any_formula ? r.wave ^ 1 : r.wave]) == cudaErrorNotReady) continue;
       if (r.cancel) {
         r.cancelled_resident = true;
         cudaEventRecord(r.done_ev, s->smc);
@@ -449,7 +455,8 @@ static void destroy_server(sabr_server* s) {
   if (s->smc) cudaStreamSynchronize(s->smc);
   for (auto& kv : s->all) release(s, *kv.second);
   for (int p = 0; p < 2; ++p) {
-    if (s->graph[p]) cudaGraphExecDestroy(s->graph[p]);
+    for (cudaGraphExec_t g : s->graph[p])
+      if (g) cudaGraphExecDestroy(g);
     if (s->buf_ev[p]) cudaEventDestroy(s->buf_ev[p]);
     if (s->h_work[p]) cudaFreeHost(s->h_work[p]);
     if (s->h_nwork[p]) cudaFreeHost(s->h_nwork[p]);
@@ -524,15 +531,16 @@ static sabr_status create_server(const sabr_server_config* cfg, sabr_server** ou
       destroy_server(s);
       return cuda_fail(e, "server graph branches");
     }
-    for (int p = 0; p < 2; ++p) {
+    for (int i = 0; i < 4; ++i) {
+      const int p = i >> 1, parallel = i & 1;
       cudaGraph_t graph = nullptr;
       e = cudaStreamBeginCapture(s->sf, cudaStreamCaptureModeThreadLocal);
       if (e == cudaSuccess) {
-        const cudaError_t le = enqueue_step_launches(s, p, s->sf, branches);
+        const cudaError_t le = enqueue_step_launches(s, p, s->sf, parallel ? &branches : nullptr);
         e = cudaStreamEndCapture(s->sf, &graph);
         if (le != cudaSuccess) e = le;
       }
-      if (e == cudaSuccess) e = cudaGraphInstantiate(&s->graph[p], graph, 0);
+      if (e == cudaSuccess) e = cudaGraphInstantiate(&s->graph[p][parallel], graph, 0);
       if (graph) cudaGraphDestroy(graph);
       if (e != cudaSuccess) {
         destroy_server(s);

@@ -1353,6 +1353,7 @@ struct sabr_plan {
   int64_t level_launches = 0;
   bool ran = false;
   bool blocking = false;   // of a blocking call: buffers kept (KeptBuffers)
+  std::vector<unsigned char> img;  // blocking call: the upload's source, alive until the run is done
   size_t arena_bytes = 0;  // allocated
   int h_count = 0;
   std::vector<sabr::McSaHost> mc;  // Technique II problems
@@ -1635,7 +1636,8 @@ static sabr_status build_plan(int32_t n, const sabr_problem* problems, const sab
   }
   const size_t arena_bytes = align_up(o, 256);
 
-  std::vector<unsigned char> img(arena_bytes, 0);
+  std::vector<unsigned char>& img = p->img;
+  img.assign(arena_bytes, 0);
   cudaError_t e = cudaSuccess;
   if (blocking) {
     p->blocking = true;
@@ -1699,7 +1701,18 @@ static sabr_status build_plan(int32_t n, const sabr_problem* problems, const sab
   }
   p->d_probs = (ProblemDev*)(base + probs_off);
   p->d_results = dres;
-  e = cudaMemcpy(p->arena, img.data(), arena_bytes, cudaMemcpyHostToDevice);
+  // A copy from pageable memory may return once its source is staged, and a
+  // non-blocking stream does not wait for the default one: a blocking call's
+  // upload goes to the stream its kernels run on (the call keeps its source until
+  // the results are there); a plan, which may run on any stream, waits until its
+  // image has landed.
+  if (blocking) {
+    e = cudaMemcpyAsync(p->arena, img.data(), arena_bytes, cudaMemcpyHostToDevice, stream);
+  } else {
+    e = cudaMemcpy(p->arena, img.data(), arena_bytes, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
+    std::vector<unsigned char>().swap(img);
+  }
   if (e == cudaSuccess && !p->h_results) {
     e = cudaMallocHost(&p->h_results, sizeof(sabr_result) * n);
     if (e == cudaSuccess) {

@@ -32,6 +32,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "arrivals.h"
 #include "sa_device.cuh"
 #include "sa_small.cuh"
 
@@ -288,10 +289,10 @@ __global__ void __launch_bounds__(kSmallBlock) sa_small_kernel(const ProblemDev*
         atomicAdd(Pr.arrive, 1u);
         volatile unsigned int* ctr = Pr.arrive;
         volatile unsigned int* err = Pr.arrive + 1;
-        bool ok = *ctr >= target;
+        bool ok = arrived(*ctr, target);
         if (!ok) {
           const unsigned long long t0 = global_ns();
-          while (!(ok = *ctr >= target)) {
+          while (!(ok = arrived(*ctr, target))) {
             if (*err) break;
             if (global_ns() - t0 > wait_ns) {
               atomicExch(Pr.arrive + 1, 1u);

@@ -253,7 +253,10 @@ sabr_status sabr_mc_shard_reduce(sabr_model model, const double* params,
  *   floor_local <= cap_local, floor_global <= cap_global (pass +-1e300 for
  *                no global limits)
  *   price_out    device, double[1]; stderr_out device double[1] or NULL
- * Asynchronous on cuda_stream; device scratch is stream-ordered
+ * Asynchronous on cuda_stream; never waits for other calls, however many are
+ * in flight.  Device scratch is one of a few that the library keeps (4 x 512
+ * KB per device, with pinned memory for the upload, made on first use), or,
+ * when all are in use or the stream is being captured, stream-ordered
  * (cudaMallocAsync / cudaFreeAsync).  EINVAL for bad sizes or limits, more
  * than 8192 time steps, or parameters violating rho(t) in [-1,1],
  * nu(t) > 0 on [0, T].

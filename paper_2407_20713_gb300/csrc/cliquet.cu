@@ -4,8 +4,11 @@
 // path_step as sabr_mc_price, with the reset dates inserted into the grid as
 // landing points.
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstring>
+#include <map>
+#include <mutex>
 #include <vector>
 
 #include "common.h"
@@ -154,6 +157,94 @@ __global__ void __launch_bounds__(kClqBlock) cliquet_reduce_kernel(const double*
   if (se) *se = disc * sqrt(var / N);
 }
 
+// Scratch of one call: a call never waits for another, whatever its stream or
+// thread.  A few fixed-size scratches per device (with pinned memory for the
+// upload) are kept, and a call takes one whose last use the GPU has finished;
+// a call that finds none, or is being captured, takes stream-ordered memory,
+// whose allocation costs a call that is waited for about 200 us.
+class CliquetScratch {
+ public:
+  sabr_status take(size_t dev_bytes, size_t host_bytes, cudaStream_t s);
+  ~CliquetScratch();
+  unsigned char* dev = nullptr;
+  unsigned char* host = nullptr;
+
+ private:
+  static constexpr int kSlots = 4;
+  // 8192 steps take 164 KB of image and 256 KB of table; the block sums 40 KB
+  static constexpr size_t kDevBytes = 512 * 1024, kHostBytes = 192 * 1024;
+  struct Slot {
+    unsigned char *dev = nullptr, *host = nullptr;
+    cudaEvent_t done = nullptr;
+    bool taken = false;
+    bool ready() const { return dev && host && done; }
+  };
+  static std::mutex mu_;
+  static std::map<int, std::array<Slot, kSlots>> slots_;
+  bool take_slot();
+  Slot* slot_ = nullptr;
+  cudaStream_t stream_ = nullptr;
+  std::vector<unsigned char> own_;
+};
+std::mutex CliquetScratch::mu_;
+std::map<int, std::array<CliquetScratch::Slot, CliquetScratch::kSlots>> CliquetScratch::slots_;
+
+bool CliquetScratch::take_slot() {
+  int d = 0;
+  if (cudaGetDevice(&d) != cudaSuccess) return false;
+  // (another thread's capture forbids queries and allocations in its mode)
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return false;
+  {
+    std::lock_guard<std::mutex> lock(mu_);
+    for (Slot& w : slots_[d]) {
+      if (w.taken) continue;
+      if (!w.ready()) {
+        if (!w.done) cudaEventCreateWithFlags(&w.done, cudaEventDisableTiming);
+        if (!w.dev) cudaMalloc(&w.dev, kDevBytes);
+        if (!w.host) cudaMallocHost(&w.host, kHostBytes);
+        if (!w.ready()) break;
+      } else if (cudaEventQuery(w.done) != cudaSuccess) {
+        continue;
+      }
+      w.taken = true;
+      slot_ = &w;
+      break;
+    }
+  }
+  cudaGetLastError();  // a slot that is busy or could not be made is no error
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  return slot_ != nullptr;
+}
+
+sabr_status CliquetScratch::take(size_t dev_bytes, size_t host_bytes, cudaStream_t s) {
+  stream_ = s;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusActive;
+  if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) cudaGetLastError();
+  if (capture == cudaStreamCaptureStatusNone && dev_bytes <= kDevBytes && host_bytes <= kHostBytes && take_slot()) {
+    dev = slot_->dev;
+    host = slot_->host;
+    return SABR_OK;
+  }
+  void* p = nullptr;
+  SABR_CUDA(cudaMallocAsync(&p, dev_bytes, s));
+  dev = (unsigned char*)p;
+  own_.assign(host_bytes, 0);  // pageable: an upload has consumed it when it returns
+  host = own_.data();
+  return SABR_OK;
+}
+
+// Also after an error: what the call has enqueued may still use the memory.
+CliquetScratch::~CliquetScratch() {
+  if (slot_) {
+    const cudaError_t e = cudaEventRecord(slot_->done, stream_);
+    std::lock_guard<std::mutex> lock(mu_);
+    slot_->taken = e != cudaSuccess;
+  } else if (dev) {
+    cudaFreeAsync(dev, stream_);
+  }
+}
+
 }  // namespace sabr
 
 extern "C" sabr_status sabr_mc_cliquet(sabr_model model, const double* params, double fwd, double T,
@@ -205,8 +296,8 @@ extern "C" sabr_status sabr_mc_cliquet(sabr_model model, const double* params, d
   const size_t tab_bytes = mc_step_table_bytes(h, 1);
   const size_t bytes = tab_off + tab_bytes;
   cudaStream_t s = (cudaStream_t)stream;
-  McScratch w;
-  SABR_TRY(w.acquire(bytes, part_off));
+  CliquetScratch w;
+  SABR_TRY(w.take(bytes, part_off, s));
   unsigned char* dev = w.dev;
   McDev d;
   int *q_value, *q_out;
@@ -228,5 +319,5 @@ extern "C" sabr_status sabr_mc_cliquet(sabr_model model, const double* params, d
                                                          part);
   cliquet_reduce_kernel<<<1, kClqBlock, 0, s>>>(part, blocks, n_paths, discount, price_out, stderr_out);
   SABR_CUDA(cudaGetLastError());
-  return w.release(s);
+  return SABR_OK;
 }

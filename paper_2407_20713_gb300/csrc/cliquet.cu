@@ -165,6 +165,9 @@ __global__ void __launch_bounds__(kClqBlock) cliquet_reduce_kernel(const double*
 class CliquetScratch {
  public:
   sabr_status take(size_t dev_bytes, size_t host_bytes, cudaStream_t s);
+  CliquetScratch() = default;
+  CliquetScratch(const CliquetScratch&) = delete;
+  CliquetScratch& operator=(const CliquetScratch&) = delete;
   ~CliquetScratch();
   unsigned char* dev = nullptr;
   unsigned char* host = nullptr;
@@ -237,9 +240,9 @@ sabr_status CliquetScratch::take(size_t dev_bytes, size_t host_bytes, cudaStream
 // Also after an error: what the call has enqueued may still use the memory.
 CliquetScratch::~CliquetScratch() {
   if (slot_) {
-    const cudaError_t e = cudaEventRecord(slot_->done, stream_);
+    if (cudaEventRecord(slot_->done, stream_) != cudaSuccess) cudaStreamSynchronize(stream_);
     std::lock_guard<std::mutex> lock(mu_);
-    slot_->taken = e != cudaSuccess;
+    slot_->taken = false;
   } else if (dev) {
     cudaFreeAsync(dev, stream_);
   }

@@ -2,6 +2,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <map>
 #include <mutex>
 #include <vector>
 
@@ -475,10 +476,11 @@ sabr_status mc_launch(const McHost& h, const McDev& d, const double* set_params,
 
 // Library-owned scratch of the pricers: two per device, taken in turn, so that a
 // call's tables are laid out and copied while the kernels of the call before it
-// run (2^16 paths: the GPU waited about 15 us between calls).  Calls are
-// serialised by the mutex and by waiting, before a scratch is rewritten, for
-// the kernels that last used it; calls on several streams therefore never
-// share one in flight.  A scratch grows to what its calls need and stays.
+// run (2^16 paths: the GPU waited about 15 us between calls).  The calls of a
+// device are serialised by its lock and by waiting, before a scratch is
+// rewritten, for the kernels that last used it; calls on several streams
+// therefore never share one in flight.  A scratch grows to what its calls need
+// and stays.
 struct McWorkspace {
   void* dev = nullptr;
   size_t dev_bytes = 0;
@@ -487,11 +489,17 @@ struct McWorkspace {
   cudaEvent_t done = nullptr;
 };
 struct McWorkspaces {
+  std::mutex mu;
   McWorkspace ws[2];
   int next = 0;
 };
-static std::mutex g_mc_mutex;
-static std::vector<McWorkspaces> g_mc_ws;
+// The scratches of a device (map nodes stay where they are).
+static McWorkspaces& mc_workspaces(int device) {
+  static std::mutex mu;
+  static std::map<int, McWorkspaces> all;
+  std::lock_guard<std::mutex> lock(mu);
+  return all[device];
+}
 
 static sabr_status ensure_ws(McWorkspace& w, size_t dev_bytes, size_t host_bytes) {
   if (!w.done) SABR_CUDA(cudaEventCreateWithFlags(&w.done, cudaEventDisableTiming));
@@ -513,23 +521,24 @@ static sabr_status ensure_ws(McWorkspace& w, size_t dev_bytes, size_t host_bytes
   return SABR_OK;
 }
 
-sabr_status McScratch::acquire(size_t dev_bytes, size_t host_bytes) {
-  lock_ = std::unique_lock<std::mutex>(g_mc_mutex);
+sabr_status McScratch::acquire(size_t dev_bytes, size_t host_bytes, cudaStream_t s) {
   int d = 0;
   SABR_CUDA(cudaGetDevice(&d));
-  if ((int)g_mc_ws.size() <= d) g_mc_ws.resize(d + 1);
-  McWorkspaces& all = g_mc_ws[d];
+  McWorkspaces& all = mc_workspaces(d);
+  lock_ = std::unique_lock<std::mutex>(all.mu);
   McWorkspace& w = all.ws[all.next];
   all.next ^= 1;
   SABR_TRY(ensure_ws(w, dev_bytes, host_bytes));
   dev = (unsigned char*)w.dev;
   host = w.host;
   done_ = w.done;
+  stream_ = s;
   return SABR_OK;
 }
-sabr_status McScratch::release(cudaStream_t s) {
-  SABR_CUDA(cudaEventRecord(done_, s));
-  return SABR_OK;
+// On every way out, errors included: what was enqueued before an error still
+// uses the scratch.
+McScratch::~McScratch() {
+  if (done_ && cudaEventRecord(done_, stream_) != cudaSuccess) cudaStreamSynchronize(stream_);
 }
 
 }  // namespace sabr
@@ -555,8 +564,9 @@ static sabr_status mc_price(sabr_model model, const double* params, double fwd, 
   const size_t tab_off = part_off + sizeof(double) * (size_t)bps * h.n_slots * 32;
   const size_t tab_bytes = mc_step_table_bytes(h, 1);
   const size_t dev_bytes = tab_off + tab_bytes;
+  cudaStream_t s = (cudaStream_t)stream;
   McScratch w;
-  SABR_TRY(w.acquire(dev_bytes, part_off));
+  SABR_TRY(w.acquire(dev_bytes, part_off, s));
   McDev d;
   int* q_value;
   int* q_out;
@@ -567,11 +577,9 @@ static sabr_status mc_price(sabr_model model, const double* params, double fwd, 
   double p10[kMaxD];
   for (int i = 0; i < kMaxD; ++i) p10[i] = i < n_params(model) ? params[i] : 0.0;
   std::memcpy(w.host + params_off, p10, sizeof(p10));
-  cudaStream_t s = (cudaStream_t)stream;
   SABR_CUDA(cudaMemcpyAsync(w.dev, w.host, part_off, cudaMemcpyHostToDevice, s));
-  SABR_TRY(mc_launch(h, d, (const double*)(base + params_off), nullptr, 1, bps, (double*)(base + part_off), q_value,
-                     q_out, disc, price_out, stderr_out, (int)n, s));
-  return w.release(s);
+  return mc_launch(h, d, (const double*)(base + params_off), nullptr, 1, bps, (double*)(base + part_off), q_value,
+                   q_out, disc, price_out, stderr_out, (int)n, s);
 }
 
 }  // namespace sabr
@@ -626,7 +634,7 @@ static sabr_status mc_shard_upload(const McShardCall& c, const double* params, c
   const size_t params_off = (img + 255) & ~(size_t)255;
   const size_t part_off = params_off + 256;
   const size_t tab_bytes = mc_step_table_bytes(c.h, 1);
-  SABR_TRY(w.acquire(part_off + tab_bytes, part_off));
+  SABR_TRY(w.acquire(part_off + tab_bytes, part_off, s));
   unsigned char* base = w.dev;
   mc_fill_image(c.h, w.host, base, d, q_value, q_out, disc);
   if (tab_bytes) d.tab = base + part_off;
@@ -676,7 +684,7 @@ extern "C" sabr_status sabr_mc_shard_partials(sabr_model model, const double* pa
   SABR_TRY(mc_shard_upload(c, params, s, w, d, &q_value, &q_out, &disc, &dp));
   launch_paths(c.h, d, dp, nullptr, dim3(block_count, 1), partials_out, block_begin, total_blocks, s);
   SABR_CUDA(cudaGetLastError());
-  return w.release(s);
+  return SABR_OK;
 }
 
 extern "C" sabr_status sabr_mc_shard_reduce(sabr_model model, const double* params, double fwd, const double* T,
@@ -699,5 +707,5 @@ extern "C" sabr_status sabr_mc_shard_reduce(sabr_model model, const double* para
   SABR_TRY(mc_shard_upload(c, params, s, w, d, &q_value, &q_out, &disc, &dp));
   launch_reduce(d, 1, total_blocks, partials, q_value, q_out, disc, nullptr, price_out, stderr_out, (int)n, s);
   SABR_CUDA(cudaGetLastError());
-  return w.release(s);
+  return SABR_OK;
 }

@@ -23,18 +23,22 @@ struct McHost {
 };
 
 // A call's hold on the pricers' scratch of the current device: acquire() waits
-// for the kernels that last used it and holds the pricers' lock until the call
-// has enqueued its work; release() marks that work on the stream.
+// for the kernels that last used it and holds the device's lock until the call
+// has enqueued its work on s, which the destructor marks there.
 class McScratch {
  public:
-  sabr_status acquire(size_t dev_bytes, size_t host_bytes);
-  sabr_status release(cudaStream_t s);
+  sabr_status acquire(size_t dev_bytes, size_t host_bytes, cudaStream_t s);
+  McScratch() = default;
+  McScratch(const McScratch&) = delete;
+  McScratch& operator=(const McScratch&) = delete;
+  ~McScratch();
   unsigned char* dev = nullptr;
   unsigned char* host = nullptr;  // pinned
 
  private:
   std::unique_lock<std::mutex> lock_;
   cudaEvent_t done_ = nullptr;
+  cudaStream_t stream_ = nullptr;
 };
 
 // Validates the option set and builds the step grid (options sorted by

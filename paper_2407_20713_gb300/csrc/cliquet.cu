@@ -296,7 +296,7 @@ extern "C" sabr_status sabr_mc_cliquet(sabr_model model, const double* params, d
   const size_t params_off = (img + 255) & ~(size_t)255;
   const size_t part_off = params_off + 256;
   const size_t tab_off = (part_off + sizeof(double) * 2 * blocks + 255) & ~(size_t)255;
-  const size_t tab_bytes = mc_step_table_bytes(h, 1);
+  const size_t tab_bytes = mc_blocks_build_steps(h, blocks, kClqBlock) ? 0 : mc_step_table_bytes(h, 1);
   const size_t bytes = tab_off + tab_bytes;
   cudaStream_t s = (cudaStream_t)stream;
   CliquetScratch w;

@@ -439,6 +439,23 @@ static bool mc_split(const McHost& h, int64_t blocks) {
   return h.prec == SABR_FP32 && h.scheme == SABR_MC_LOG_EULER && blocks <= (int64_t)device_sms();
 }
 
+// Whether the blocks of a dynamic model's launch build their step tables
+// themselves: forming one entry is about 80 FP64 instructions, so a table costs
+// an SM about 15 ns an entry for every block on it, and the launch that forms it
+// once costs 4 to 5 us between two kernels.  The line is at 300 entries an SM
+// and two entries a thread (us a call in a row, built by the blocks | by a launch;
+// pricer 70 000 paths x 250 steps, 1 block an SM 67.6 | 70.4; 150 000 x 100, 2
+// blocks 64.2 | 68.3; x 250 100.3 | 96.6; 300 000 x 50, 4 blocks 66.7 | 68.8; x
+// 100 92.5 | 91.5; cliquet, blocks of 64: 20 000 x 100, 1 block 49.0 | 52.5; x 250
+// 67.3 | 65.0; 150 000 x 50, 4 blocks 48.4 | 52.5; 300 000 x 50, 8 blocks 65.0 |
+// 63.9).
+bool mc_blocks_build_steps(const McHost& h, int64_t blocks, int block_threads) {
+  if (h.scheme == SABR_MC_BESSEL) return false;
+  if (h.model != SABR_DYN_I && h.model != SABR_DYN_II) return true;
+  const int64_t sms = device_sms(), per_sm = (blocks + sms - 1) / sms;
+  return per_sm * h.n_steps <= 300 && h.n_steps <= 2 * block_threads;
+}
+
 // Fills d.tab for n_sets sets.
 void mc_launch_steps(const McHost& h, const McDev& d, const double* set_params, const int* set_valid, int n_sets,
                      cudaStream_t s) {
@@ -458,11 +475,15 @@ void mc_launch_steps(const McHost& h, const McDev& d, const double* set_params, 
 
 static void launch_paths(const McHost& h, const McDev& d, const double* set_params, const int* set_valid,
                          dim3 grid, double* partial, int block0, int grid_total, cudaStream_t s) {
-  if (d.tab != nullptr) mc_launch_steps(h, d, set_params, set_valid, (int)grid.y, s);
-  const bool split = mc_split(h, (int64_t)grid.x * grid.y);
+  const int64_t blocks = (int64_t)grid.x * grid.y;
+  const bool split = mc_split(h, blocks);
+  const int threads = split ? 2 * kMcBlock : kMcBlock;
+  McDev k = d;
+  if (mc_blocks_build_steps(h, blocks, kMcBlock)) k.tab = nullptr;
+  if (k.tab != nullptr) mc_launch_steps(h, k, set_params, set_valid, (int)grid.y, s);
   size_t smem = 0;
   const McPathsFn fn = mc_paths_fn(h, split, &smem);
-  fn<<<grid, split ? 2 * kMcBlock : kMcBlock, smem, s>>>(d, set_params, set_valid, partial, block0, grid_total);
+  fn<<<grid, threads, smem, s>>>(k, set_params, set_valid, partial, block0, grid_total);
 }
 
 sabr_status mc_launch(const McHost& h, const McDev& d, const double* set_params, const int* set_valid, int n_sets,

@@ -115,8 +115,9 @@ __device__ __forceinline__ StepCoef<R> dynamic_step_coef(const McDev& P, const d
 // land[m] = the step whose end is maturity m.  A static model's entry is four
 // FP64 products (square roots once per thread or by the host).  A dynamic
 // model's needs two FP64 exponentials and two square roots, about 80
-// instructions on a pipe that takes 1.7 a clock: 12 us a block at 252 steps,
-// for every resident block of an SM, so mc_steps_kernel forms it once per set.
+// instructions on a pipe that takes 1.7 a clock, for every block of an SM, so
+// mc_steps_kernel forms it once per set unless the launch is small
+// (mc_blocks_build_steps).
 template <class R>
 __device__ __forceinline__ void build_steps(const McDev& P, const double* p, int set, StepCoef<R>* tab, int* land) {
   const bool dyn = P.model == SABR_DYN_I || P.model == SABR_DYN_II;

@@ -55,6 +55,9 @@ int mc_blocks_per_set(const McHost& h, int n_sets);
 // where none is used.  A caller without room for them leaves McDev::tab null
 // (log-Euler only): the blocks then build their tables themselves.
 size_t mc_step_table_bytes(const McHost& h, int n_sets);
+// Whether a launch of that many blocks does without the table although there is
+// room for it.
+bool mc_blocks_build_steps(const McHost& h, int64_t blocks, int block_threads);
 // Fills McDev::tab of n_sets parameter sets.
 void mc_launch_steps(const McHost& h, const McDev& d, const double* set_params, const int* set_valid, int n_sets,
                      cudaStream_t s);

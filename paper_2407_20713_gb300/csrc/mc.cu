@@ -20,9 +20,9 @@ struct McSmem {
   size_t tab, land, q0, nq, slot, K, call, wacc, fx, total;
 };
 
-// FP32 log-Euler options are stored as McOption (8 bytes, no call flag);
-// split: the block of 2 kMcBlock threads also needs the exchange buffer of
-// simulate_paths_f32<1>.
+// FP32 log-Euler options are stored as signed strikes (mc.cuh: no call flag
+// is read); split: the block of 2 kMcBlock threads also needs the exchange
+// buffer of simulate_paths_f32<1>.
 template <class R>
 __host__ __device__ inline McSmem mc_smem_layout(int n_steps, int n_quotes, int n_mats, int n_slots, bool split) {
   // (the conditional-Bessel form leaves its step table in global memory and
@@ -36,7 +36,7 @@ __host__ __device__ inline McSmem mc_smem_layout(int n_steps, int n_quotes, int 
   };
   L.wacc = take(sizeof(double) * kMcWarps * n_slots * 32);
   L.tab = take(sizeof(StepCoef<R>) * n_steps);
-  L.K = take(8 * n_quotes);
+  L.K = take(sizeof(R) * n_quotes);
   L.land = take(sizeof(int) * n_mats);
   L.q0 = take(sizeof(int) * n_mats);
   L.nq = take(sizeof(int) * n_mats);
@@ -46,16 +46,6 @@ __host__ __device__ inline McSmem mc_smem_layout(int n_steps, int n_quotes, int 
   L.total = (o + 15) & ~(size_t)15;
   return L;
 }
-// Bytes of a block's tables and accumulators by which problems are refused
-// and grids are sized: strikes at the working precision, as the scalar paths
-// keep them (within 6 KB of what any form of the kernel takes).
-static size_t mc_table_bytes(int prec, int n_steps, int n_quotes, int n_mats, int n_slots) {
-  auto up = [](size_t x) { return (x + 15) & ~(size_t)15; };
-  const size_t rs = prec == SABR_FP64 ? 8 : 4;
-  return up(sizeof(double) * kMcWarps * n_slots * 32) + up(4 * rs * n_steps) + up(rs * n_quotes) +
-         4 * up(sizeof(int) * n_mats) + up(n_quotes);
-}
-
 // grid = (blocks_per_set, n_sets).  Set s prices with set_params[s][0..9];
 // sets whose set_valid flag is 0 are skipped.  Writes, per block, the FP64
 // sums of payoff and payoff^2 of every option to
@@ -86,7 +76,7 @@ __global__ void __launch_bounds__((SPLIT ? 2 * kMcBlock : kMcBlock),
   double* wacc = (double*)(smem + L.wacc);
   StepCoef<R>* tab = (StepCoef<R>*)(smem + L.tab);
   R* sK = (R*)(smem + L.K);
-  McOption* sopt = (McOption*)(smem + L.K);
+  float* sopt = (float*)(smem + L.K);
   int* land = (int*)(smem + L.land);
   int* s_q0 = (int*)(smem + L.q0);
   int* s_nq = (int*)(smem + L.nq);
@@ -107,8 +97,7 @@ __global__ void __launch_bounds__((SPLIT ? 2 * kMcBlock : kMcBlock),
   }
   for (int q = threadIdx.x; q < P.n_quotes; q += blockDim.x) {
     if constexpr (kPairs) {
-      const float K = (float)P.K[q];
-      sopt[q] = P.is_call[q] != 0 ? McOption{1.0f, -K} : McOption{-1.0f, K};
+      sopt[q] = signed_strike((float)P.K[q], P.is_call[q] != 0);
     } else {
       sK[q] = (R)P.K[q];
       scall[q] = P.is_call[q];
@@ -301,7 +290,12 @@ sabr_status mc_prepare(int model, double fwd, const double* T, const double* K, 
   h.n_steps = (int)h.step_t.size();
   if (h.n_steps > kMaxMcSteps) return fail(SABR_EINVAL, "more than 8192 time steps");
   h.Tmax = h.mats.back();
-  const size_t smem = mc_table_bytes(prec, h.n_steps, h.n_quotes, (int)h.mats.size(), h.n_slots);
+  // what a block of the log-Euler kernel takes (the conditional-Bessel kernel
+  // keeps its step table in global memory; the same limit holds for it)
+  const int M = (int)h.mats.size();
+  const size_t smem = prec == SABR_FP64
+                          ? mc_smem_layout<double>(h.n_steps, h.n_quotes, M, h.n_slots, false).total
+                          : mc_smem_layout<float>(h.n_steps, h.n_quotes, M, h.n_slots, false).total;
   if (smem > 220 * 1024) return fail(SABR_EINVAL, "too many time steps and options for one launch");
   h.smem = smem;
   return SABR_OK;

@@ -466,10 +466,12 @@ __device__ __forceinline__ void run_path_pairs(const McDev& P, const StepCoef<fl
 }
 
 // One option in shared memory, FP32: payoff (sgn F + c)^+ with sgn = 1,
-// c = -K for a call and sgn = -1, c = K for a put.
-struct McOption {
-  float sgn, c;
-};
+// c = -K for a call and sgn = -1, c = K for a put.  Only c is stored: its sign
+// bit (set for a call, at K = 0 too) gives sgn.
+__device__ __forceinline__ float signed_strike(float K, bool call) { return call ? -K : K; }
+__device__ __forceinline__ float forward_sign(float c) {
+  return __uint_as_float(0xBF800000u ^ (__float_as_uint(c) & 0x80000000u));
+}
 
 // The FP32 path loop: four paths per virtual thread as two pairs
 // (path_step2); the same path numbering, Philox counters, landing steps and
@@ -485,7 +487,7 @@ struct McOption {
 template <int PAIRS>
 __device__ __forceinline__ void simulate_paths_f32(const McDev& P, const double* p, const StepCoef<float>* tab,
                                                    const int* land, const int* s_q0, const int* s_nq,
-                                                   const int* s_slot, const McOption* opt, int64_t path0,
+                                                   const int* s_slot, const float* opt, int64_t path0,
                                                    int64_t pstride, double* wacc, float* fx) {
   const int lane = threadIdx.x & 31;
   const int vt = threadIdx.x & (kMcBlock - 1), half = PAIRS == 1 ? threadIdx.x / kMcBlock : 0;
@@ -533,10 +535,10 @@ __device__ __forceinline__ void simulate_paths_f32(const McDev& P, const double*
             const int j = (c0 + kk) >> 1;
             float pay = 0.0f, pay2 = 0.0f;
             if (j < nq) {
-              const McOption o = opt[q0 + j];
+              const float c = opt[q0 + j], sgn = forward_sign(c);
 #pragma unroll
               for (int k = 0; k < NF; ++k) {
-                const float x = fmaxf(fmaf(o.sgn, F[k], o.c), 0.0f);
+                const float x = fmaxf(fmaf(sgn, F[k], c), 0.0f);
                 const float y = live[k] ? x : 0.0f;
                 pay += y;
                 pay2 = fmaf(y, y, pay2);

@@ -203,8 +203,9 @@ __device__ __forceinline__ void lockstep_level(const ProblemDev& P, uint32_t gch
 // level when this block closes level `level` of problem `pid`.
 // ONE (FP32 Hagan): every chain has one lane (G = L = 1); the forms for several
 // lanes are left out, which the register allocation of the one-lane loops,
-// the largest of the kernel, is sensitive to.
-template <class R, int MODEL, int PAIRS = 2, bool SEL = false, bool ONE = false>
+// the largest of the kernel, is sensitive to.  LOCK (FP32 Hagan): with the
+// lockstep form of chains on fewer lanes than their sums are ordered by.
+template <class R, int MODEL, int PAIRS, bool LOCK, bool ONE = false>
 __device__ __forceinline__ void sa_level_block(const ProblemDev& P, int pid, int blk, int level, unsigned char* smem,
                                                const LevelQueue* q) {
   unsigned char* rest;
@@ -281,7 +282,7 @@ __device__ __forceinline__ void sa_level_block(const ProblemDev& P, int pid, int
                                return dynamic_cost_f32<MODEL>(xp, P.n_quotes, P.n_mats, l2f, sq, coef, lane, L, G,
                                                               0xffffffffu);
                              });
-  } else if constexpr (sizeof(R) == 4 && MODEL == SABR_HAGAN && PAIRS < 5 && !ONE) {
+  } else if constexpr (sizeof(R) == 4 && MODEL == SABR_HAGAN && LOCK) {
     if (L < G) {
       ran = true;
       const LaneSplit ls = lane_split(G, L);
@@ -360,8 +361,8 @@ __device__ __forceinline__ void sa_level_block(const ProblemDev& P, int pid, int
             bool go = true;
 #pragma unroll
             for (int k = 0; k < SD; ++k) {
-              if constexpr (sizeof(R) == 4 && SEL) {
-                // FP32, SEL: the decisions as selects (as in the one-step
+              if constexpr (sizeof(R) == 4) {
+                // FP32: the decisions as selects (as in the one-step
                 // loop), so that the chains of a warp, whose steps accept and
                 // reject at different points, run the same instructions
                 const bool take = go && st + k < P.chain_len;
@@ -658,7 +659,7 @@ __device__ __forceinline__ void sa_level_block(const ProblemDev& P, int pid, int
 // read from device memory (n_work != nullptr), each item carrying its own
 // level in .z (level < 0), so that one captured launch serves every step
 // whatever its mix of requests.  Both use this one kernel, so a problem's
-// arithmetic is the same machine code in a plan and in the server.
+// arithmetic is the same source in a plan and in the server.
 // Register budget: up to 128 registers for the static formulas (the server
 // keeps 16 of their warps an SM), 255 for the dynamic ones, whose chains run on
 // as few lanes as give a scheduler two warps; the expanded form keeps 80.
@@ -667,7 +668,11 @@ template <class R, int MODEL> struct LevelMinBlocks {
       sizeof(R) == 8 || MODEL == SABR_DYN_I || MODEL == SABR_DYN_II ? 1 : (MODEL == SABR_EXPANDED ? 3 : 2);
 };
 
-template <class R, int MODEL>
+// LOCK: with the lockstep form of FP32 Hagan chains on fewer lanes than their
+// sums are ordered by, which only the server runs; a plan's levels go without it
+// (2000 chains x 126 quotes, 40 x 50: 3.94 ms with, 3.90 without; 4000 x 492
+// 10.64, 10.25).
+template <class R, int MODEL, bool LOCK>
 __global__ void __launch_bounds__(kSaBlock, (LevelMinBlocks<R, MODEL>::value))
     sa_level_kernel(const ProblemDev* __restrict__ probs, const int4* __restrict__ work,
                     const int* __restrict__ n_work, int n_items, int level) {
@@ -686,7 +691,7 @@ __global__ void __launch_bounds__(kSaBlock, (LevelMinBlocks<R, MODEL>::value))
       }
       __syncthreads();
     }
-    if (lv < P.n_levels) sa_level_block<R, MODEL, 2, true>(P, it.x, it.y, lv, smem, nullptr);
+    if (lv < P.n_levels) sa_level_block<R, MODEL, 2, LOCK>(P, it.x, it.y, lv, smem, nullptr);
     __syncthreads();
   }
 }
@@ -704,10 +709,13 @@ template <class R, int MODEL> struct QueuePairs {
   static constexpr int value = 5;
 };
 
-// ONE: the loops for one lane a chain alone, at 198 registers (five blocks an
-// SM; the launch holds four): ten smiles x 4096 chains x 21 quotes, 200 x 100
-// in 24.7 ms, against 25.2-26.3 for the kernel that also holds the forms for
-// several lanes (two warps a scheduler live on the order of the instructions).
+// ONE: the loops for one lane a chain alone, at 162 registers (five blocks an
+// SM; the launch holds four).  Two warps a scheduler live on the order of the
+// instructions, and in one kernel the one-lane loops and the select form of the
+// speculative loop cost each other: ten smiles x 4096 chains x 21 quotes, 200 x
+// 100 take 24.95 ms here and 25.2-26.3 beside the other forms (25.02 where those
+// decide by branches), and one smile x 1600 chains x 15 quotes, 60 x 50 takes 3.44
+// ms with selects, 3.54 with branches.
 template <class R, int MODEL, bool ONE = false>
 __global__ void __launch_bounds__(kLevelBlock, (ONE ? 5 : QueueBlocks<R, MODEL>::value))
     sa_queue_kernel(const ProblemDev* __restrict__ probs, LevelQueue q) {
@@ -1203,9 +1211,13 @@ size_t formula_layout(const HostProblem& h, int G, unsigned char* img, unsigned 
 }
 
 // ---- launch wrappers ------------------------------------------------------
+// (the other kinds have no such form and share one instance)
+template <class R, int MODEL> constexpr bool kPlanLock = !(sizeof(R) == 4 && MODEL == SABR_HAGAN);
+
 template <class R, int MODEL>
 static void set_smem_one(size_t bytes) {
-  allow_smem((const void*)sa_level_kernel<R, MODEL>, bytes);
+  allow_smem((const void*)sa_level_kernel<R, MODEL, kPlanLock<R, MODEL>>, bytes);
+  allow_smem((const void*)sa_level_kernel<R, MODEL, true>, bytes);
   allow_smem((const void*)sa_init_kernel<R, MODEL>, bytes);
 }
 
@@ -1241,12 +1253,12 @@ void launch_init(int prec, int model, const ProblemDev* probs, const int* plist,
 void launch_level(int prec, int model, const ProblemDev* probs, const int4* bmap, int blocks, int level, size_t smem,
                   cudaStream_t s) {
   SABR_DISPATCH(prec, model,
-                (sa_level_kernel<R, M><<<blocks, kLevelBlock, smem, s>>>(probs, bmap, nullptr, blocks, level)));
+                (sa_level_kernel<R, M, kPlanLock<R, M>><<<blocks, kLevelBlock, smem, s>>>(probs, bmap, nullptr, blocks, level)));
 }
 
 void launch_persistent(int prec, int model, const ProblemDev* probs, const int4* work, const int* n_work, int grid,
                        size_t smem, cudaStream_t s) {
-  SABR_DISPATCH(prec, model, (sa_level_kernel<R, M><<<grid, kSaBlock, smem, s>>>(probs, work, n_work, 0, -1)));
+  SABR_DISPATCH(prec, model, (sa_level_kernel<R, M, true><<<grid, kSaBlock, smem, s>>>(probs, work, n_work, 0, -1)));
 }
 
 void launch_finalize(int prec, int model, const ProblemDev* probs, const int* plist, int n, cudaStream_t s,
@@ -1282,7 +1294,7 @@ static int queue_blocks_per_sm(int prec, int model, size_t smem, bool one) {
 int persistent_blocks_per_sm(int prec, int model, size_t smem) {
   int nb = 1;
   SABR_DISPATCH(prec, model,
-                (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sa_level_kernel<R, M>, kSaBlock, smem)));
+                (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sa_level_kernel<R, M, true>, kSaBlock, smem)));
   return nb < 1 ? 1 : nb;
 }
 

@@ -66,6 +66,13 @@ __device__ __forceinline__ SmemQuotes<R> stage_quotes(const ProblemDev& P, unsig
   return sq;
 }
 
+// The quotes that stage_quotes left at `base`, for a function of its own (static
+// models).
+template <class R> __device__ __forceinline__ SmemQuotes<R> staged_quotes(int n_quotes, unsigned char* base) {
+  QuotePack<R>* pack = (QuotePack<R>*)base;
+  return SmemQuotes<R>{pack, (const float4*)base, (R*)(pack + n_quotes + 1), nullptr, nullptr, nullptr, nullptr};
+}
+
 // Lexicographic minimum of (f, i): the smaller f, then the smaller index, so
 // the result does not depend on the order of merging.
 __device__ __forceinline__ void argmin_merge(double& f, int& i, double f2, int i2) {

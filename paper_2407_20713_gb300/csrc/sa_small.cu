@@ -77,6 +77,95 @@ template <int NW> __device__ __forceinline__ void chain_sync(int chain_in_block)
   }
 }
 
+// Words of steps s0 .. s0 + 31 of a chain's level into a warp's ring, a Philox
+// block a lane.
+__device__ __forceinline__ void draw_words(uint32_t gchain, int level, int s0, uint32_t key0, uint32_t key1,
+                                           float (*w)[kRing], float* u) {
+  const int s = s0 + (threadIdx.x & 31), at = s & (kRing - 1);
+  const uint4 b = philox4x32_10(make_uint4(gchain, (uint32_t)level, (uint32_t)s, kTagSA), key0, key1);
+  __syncwarp();  // every lane has read the entries that are replaced
+  w[0][at] = 2.0f * u01<float>(b.x) - 1.0f;
+  w[1][at] = 2.0f * u01<float>(b.y) - 1.0f;
+  w[2][at] = 2.0f * u01<float>(b.z) - 1.0f;
+  w[3][at] = 2.0f * u01<float>(b.w) - 1.0f;
+  u[at] = u01<float>(sa_accept_word(b.x, b.y, b.z));
+  __syncwarp();
+}
+
+// A level one step after the other, by one warp with all its lanes on one point:
+// for chains that accept less than half of what they evaluate (a start
+// temperature far below the costs that a step makes), whose windows would be
+// points evaluated in vain.  20 levels x 50 steps at 1% accepted, ms in windows |
+// so: 64 chains x 15 quotes 1.87 | 0.78, 608 x 492 4.9 | 2.0, 1216 x 492 4.9 | 2.1,
+// Obloj 1216 x 246 6.2 | 2.3; FP64 (6 levels), 64 x 246 20.8 | 11.3, Obloj 152 x 42 9.0
+// | 5.0.  At 20% accepted windows are still the slower by 1.3 to 2.9.
+template <class R> struct ChainState {
+  R x[4], bx[4];
+  typename CostOf<R>::T fcur, bf;
+  unsigned ev, ac;
+};
+template <class R, int MODEL>
+__device__ __forceinline__ void single_steps(const ProblemDev& P, uint32_t gchain, int level, const R* step4, float inv_Tk,
+                                          double Tk, float (*w)[kRing], float* u, ChainState<R>& z) {
+  using C = typename CostOf<R>::T;
+  constexpr int D = 4;
+  extern __shared__ __align__(16) unsigned char smem[];
+  const SmemQuotes<R> sq = staged_quotes<R>(P.n_quotes, smem);
+  const R l2f = (R)P.l2f;
+  const int n_quotes = P.n_quotes, G = P.G, len = P.chain_len;
+  const int units = StaticPoint<R, MODEL>::kPair ? (n_quotes + 1) >> 1 : n_quotes;
+  const LaneSplit ls = lane_split(G, 32);
+  // lane i & 3 forms coordinate i of the proposal and tests it
+  const int ci = threadIdx.x & (D - 1);
+  const R step = step4[ci];
+  const auto lo = BoxKey<R>::of((R)P.lo[ci]), hi = BoxKey<R>::of((R)P.hi[ci]);
+  R x[D], bx[D];
+#pragma unroll
+  for (int i = 0; i < D; ++i) x[i] = z.x[i], bx[i] = z.bx[i];
+  C fcur = z.fcur, bf = z.bf;
+  unsigned ev = z.ev, ac = z.ac;
+  for (int st = 0; st < len; ++st) {
+    if ((st & 31) == 0) draw_words(gchain, level, st, P.key0, P.key1, w, u);
+    const int at = st & (kRing - 1);
+    R xi = x[0];
+#pragma unroll
+    for (int i = 1; i < D; ++i) xi = ci == i ? x[i] : xi;
+    const R y = move_by(xi, step, word_to(w[ci][at], R{}));
+    const auto v = BoxKey<R>::of(y);
+    if (__any_sync(0xffffffffu, v < lo || v > hi)) continue;
+    R xs[D];
+#pragma unroll
+    for (int i = 0; i < D; ++i) xs[i] = __shfl_sync(0xffffffffu, y, i);
+    const StaticPoint<R, MODEL> pt(xs, l2f, n_quotes);
+    const C f = virtual_lanes_sum<R>(pt, units, G, ls, sq, 0xffffffffu);
+    ++ev;
+    if (cost_less(f, bf)) {
+      bf = f;
+#pragma unroll
+      for (int i = 0; i < D; ++i) bx[i] = xs[i];
+    }
+    const auto delta = cost_delta(f, fcur);
+    if (delta <= 0 || metropolis(word_to(u[at], R{}), delta, inv_Tk, Tk)) {
+      ++ac;
+      fcur = f;
+#pragma unroll
+      for (int i = 0; i < D; ++i) x[i] = xs[i];
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < D; ++i) z.x[i] = x[i], z.bx[i] = bx[i];
+  z.fcur = fcur, z.bf = bf, z.ev = ev, z.ac = ac;
+}
+
+// FP32 calls it, so that it takes neither registers nor order from the windows
+// (inlined, 152 chains x 75 quotes take 4% longer); FP64 has registers to spare.
+template <class R, int MODEL>
+__device__ __noinline__ void single_steps_call(const ProblemDev& P, uint32_t gchain, int level, const R* step4,
+                                               float inv_Tk, double Tk, float (*w)[kRing], float* u,
+                                               ChainState<R>& z) {
+  single_steps<R, MODEL>(P, gchain, level, step4, inv_Tk, Tk, w, u, z);
+}
+
 // What bounds it (64 chains, 15 quotes, 4 warps x 4 points: 3.9 ms for 200
 // levels x 100 steps, 15.6 two steps at a time on 8 lanes): latency.  A level of
 // no steps takes 4 us (the meeting of 64 blocks), a window of 16 steps about
@@ -88,10 +177,20 @@ template <int NW> __device__ __forceinline__ void chain_sync(int chain_in_block)
 // writes the minima of level k + 2 only after every block has read those of
 // level k (it arrives at k + 1 after reading them).  The costs of an iteration
 // alternate likewise.
+//
+// A block's chains go step by step (single_steps) in the level after one in
+// which they accepted less than half of the proposals that they evaluated, and
+// back.  The two kinds of levels have a loop each: one loop that asks per level
+// costs the windows 4 to 6% (64 chains x 15 quotes, 200 x 100: 4.01 ms without
+// the single steps, 4.28 in one loop, 3.95 in two).
+//
+// Blocks an SM of the largest launch of a shape (small_shape,
+// small_most_chains); the registers are set by it.
+template <class R, int NW, int KW>
+constexpr int kSmallResident = sizeof(R) == 8 ? 1 : (KW == 2 ? 4 : (NW == 1 ? 2 : 1));
 template <class R, int MODEL, int NW, int KW>
-__global__ void __launch_bounds__(kSmallBlock) sa_small_kernel(const ProblemDev* __restrict__ probs,
-                                                              const int4* __restrict__ work,
-                                                              unsigned long long wait_ns) {
+__global__ void __launch_bounds__(kSmallBlock, (kSmallResident<R, NW, KW>))
+    sa_small_kernel(const ProblemDev* __restrict__ probs, const int4* __restrict__ work, unsigned long long wait_ns) {
   using C = typename CostOf<R>::T;
   using Key = typename BoxKey<R>::T;
   constexpr int D = 4, P = 32 / KW, K = NW * KW, CPB = kSmallBlock / 32 / NW;
@@ -106,6 +205,7 @@ __global__ void __launch_bounds__(kSmallBlock) sa_small_kernel(const ProblemDev*
   __shared__ C s_f[CPB][2][K];                       // their costs
   __shared__ double s_mf[CPB], s_mx[CPB][D], s_new[D + 1];
   __shared__ int s_stop;
+  __shared__ float s_low[CPB];                       // evaluations less twice the acceptances of a level
   const int4 it = work[blockIdx.x];
   load_problem(probs, it.x, &Pr);
   const int blk = it.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -143,7 +243,7 @@ __global__ void __launch_bounds__(kSmallBlock) sa_small_kernel(const ProblemDev*
   int parity = 0;
   __syncthreads();
 
-  for (int level = 0; level < n_levels; ++level) {
+  auto level_begin = [&](int level) {
     // temperatures and step widths of the next kLevelCache levels, a level a
     // lane of warp 0 (FP64 square roots and divisions, off the levels' path)
     if ((level & (kLevelCache - 1)) == 0) {
@@ -157,120 +257,23 @@ __global__ void __launch_bounds__(kSmallBlock) sa_small_kernel(const ProblemDev*
       }
       __syncthreads();
     }
-    if (active) {
-      const R step = s_step[level & (kLevelCache - 1)][ci];
-      const float inv_Tk = s_invTk[level & (kLevelCache - 1)];
-      const double Tk = s_Tk[level & (kLevelCache - 1)];
-      unsigned ev = 0, ac = 0;
-      int filled = 0;  // steps whose words are in the ring
-      int st = 0;
-      while (st < len) {
-        if (filled < len && filled < st + K) {
-          const int s = filled + lane;
-          const uint4 w = philox4x32_10(make_uint4(gchain, (uint32_t)level, (uint32_t)s, kTagSA), key0, key1);
-          __syncwarp();  // every lane has read the entries that are replaced
-          s_w[warp][0][s & (kRing - 1)] = 2.0f * u01<float>(w.x) - 1.0f;
-          s_w[warp][1][s & (kRing - 1)] = 2.0f * u01<float>(w.y) - 1.0f;
-          s_w[warp][2][s & (kRing - 1)] = 2.0f * u01<float>(w.z) - 1.0f;
-          s_w[warp][3][s & (kRing - 1)] = 2.0f * u01<float>(w.w) - 1.0f;
-          s_u[warp][s & (kRing - 1)] = u01<float>(sa_accept_word(w.x, w.y, w.z));
-          filled += 32;
-          __syncwarp();
-        }
-        const int nv = len - st < K ? len - st : K;  // steps of this window
-        const unsigned window = nv == K ? kAll : (1u << nv) - 1u;
-        // the window's points if every proposal inside the box is accepted;
-        // one found outside (skip) is rejected for certain, and the points
-        // after it start from the one before it
-        unsigned skip = 0, out;
-        R xi0 = x[0];
-#pragma unroll
-        for (int i = 1; i < D; ++i) xi0 = ci == i ? x[i] : xi0;
-        R w[K];
-#pragma unroll
-        for (int j = 0; j < K; ++j) w[j] = word_to(s_w[warp][ci][(st + j) & (kRing - 1)], R{});
-        do {
-          R cur = xi0;
-#pragma unroll
-          for (int j = 0; j < K; ++j) {
-            const R y = move_by(cur, step, w[j]);
-            if (lane < D) s_x[warp][j][ci] = y;
-            cur = (skip >> j) & 1u ? cur : y;
-          }
-          __syncwarp();
-          const R* y = s_x[warp][K == 32 ? lane : (lane & (K - 1))];
-          bool in = true;
-#pragma unroll
-          for (int i = 0; i < D; ++i) {
-            const Key v = BoxKey<R>::of(y[i]);
-            in = in && !(v < lo[i] || v > hi[i]);
-          }
-          out = ~__ballot_sync(0xffffffffu, in) & window & ~skip;
-          skip |= out & (0u - out);
-        } while (out);
-        const unsigned in_mask = window & ~skip;
-        unsigned rej = 0;
-        if (in_mask) {
-          R xs[D];
-#pragma unroll
-          for (int i = 0; i < D; ++i) xs[i] = s_x[warp][k_own][i];
-          const StaticPoint<R, MODEL> pt(xs, l2f, n_quotes);
-          const C fo = virtual_lanes_sum<R>(pt, units, G, ls, sq, 0xffffffffu);
-          C* fb = s_f[cb][parity];
-          parity ^= 1;
-          if ((lane & (P - 1)) == 0) fb[k_own] = fo;
-          chain_sync<NW>(cb);
-          // lane k decides step k
-          const int k = lane & (K - 1);
-          const C f = fb[k];
-          const unsigned before = in_mask & ((1u << k) - 1u);  // the nearest earlier step inside the box
-          const C fe = fb[before ? 31 - __clz(before) : 0];
-          const C fp = before ? fe : fcur;
-          const auto delta = cost_delta(f, fp);
-          const R u = word_to(s_u[warp][(st + k) & (kRing - 1)], R{});
-          const bool acc = delta <= 0 || metropolis(u, delta, inv_Tk, Tk);
-          rej = __ballot_sync(0xffffffffu, !acc) & in_mask;
-          const int first = __ffs(rej) - 1;  // the first rejected step
-          const unsigned eval = rej ? in_mask & ((2u << first) - 1u) : in_mask;
-          const unsigned taken = rej ? eval & ~(1u << first) : eval;
-          ev += __popc(eval);
-          ac += __popc(taken);
-          unsigned better = __ballot_sync(0xffffffffu, cost_less(f, bf)) & eval;
-          if (better) {
-            int at = 0;
-            while (better) {
-              const int l = __ffs(better) - 1;
-              better &= better - 1u;
-              if (cost_less(fb[l], bf)) {
-                bf = fb[l];
-                at = l;
-              }
-            }
-#pragma unroll
-            for (int i = 0; i < D; ++i) bx[i] = s_x[warp][at][i];
-          }
-          if (taken) {
-            const int last = 31 - __clz(taken);
-            fcur = fb[last];
-#pragma unroll
-            for (int i = 0; i < D; ++i) x[i] = s_x[warp][last][i];
-          }
-          st += rej ? first + 1 : nv;
-        } else {
-          st += nv;
-        }
-        __syncwarp();  // the points are read before the next window's are written
-      }
-      ev_all += ev;
-      ac_all += ac;
-    }
-    // ---- level end: argmin over the chains of the problem ----------------
+  };
+  bool low = false;  // few of the proposals that the block's chains evaluated in the last level were accepted
+  // argmin over the chains of the problem; false when a wait gave up
+  auto level_end = [&](int level, unsigned ev, unsigned ac, auto single) {
+    ev_all += ev;
+    ac_all += ac;
+    // warps that share windows all know a lone chain's counts
+    constexpr bool kShared = CPB > 1 || decltype(single)::value;
+    const float excess = (float)ev - 2.0f * (float)ac;
+    if (!kShared) low = ac < ev - ac;
     if (wc == 0 && lane == 0) {
       s_mf[cb] = active ? cost_to_double(fcur) : INFINITY;
 #pragma unroll
       for (int i = 0; i < D; ++i) s_mx[cb][i] = (double)x[i];
     }
     __syncthreads();
+    if (kShared && wc == 0 && lane == 0) s_low[cb] = active ? excess : 0.0f;
     target += (unsigned)nb;
     if (warp == 0) {
       double* mf = Pr.part_f + (size_t)(level & 1) * nb;
@@ -322,10 +325,143 @@ __global__ void __launch_bounds__(kSmallBlock) sa_small_kernel(const ProblemDev*
       }
     }
     __syncthreads();
-    if (s_stop) return;
+    if (s_stop) return false;
 #pragma unroll
     for (int i = 0; i < D; ++i) x[i] = (R)s_new[i];
     fcur = cost_from(s_new[D], C{});
+    if (kShared) {
+      float balance = 0.0f;
+#pragma unroll
+      for (int i = 0; i < CPB; ++i) balance += s_low[i];
+      low = balance > 0.0f;
+    }
+    return true;
+  };
+
+  int level = 0;
+  while (level < n_levels) {
+    for (; level < n_levels && !low; ++level) {
+      level_begin(level);
+      unsigned ev = 0, ac = 0;
+      if (active) {
+        const R step = s_step[level & (kLevelCache - 1)][ci];
+        const float inv_Tk = s_invTk[level & (kLevelCache - 1)];
+        const double Tk = s_Tk[level & (kLevelCache - 1)];
+        int filled = 0;  // steps whose words are in the ring
+        int st = 0;
+        while (st < len) {
+          if (filled < len && filled < st + K) {
+            draw_words(gchain, level, filled, key0, key1, s_w[warp], s_u[warp]);
+            filled += 32;
+          }
+          R xi0 = x[0];
+#pragma unroll
+          for (int i = 1; i < D; ++i) xi0 = ci == i ? x[i] : xi0;
+          const int nv = len - st < K ? len - st : K;  // steps of this window
+          const unsigned window = nv == K ? kAll : (1u << nv) - 1u;
+          // the window's points if every proposal inside the box is accepted;
+          // one found outside (skip) is rejected for certain, and the points
+          // after it start from the one before it
+          unsigned skip = 0, out;
+          R w[K];
+#pragma unroll
+          for (int j = 0; j < K; ++j) w[j] = word_to(s_w[warp][ci][(st + j) & (kRing - 1)], R{});
+          do {
+            R cur = xi0;
+#pragma unroll
+            for (int j = 0; j < K; ++j) {
+              const R y = move_by(cur, step, w[j]);
+              if (lane < D) s_x[warp][j][ci] = y;
+              cur = (skip >> j) & 1u ? cur : y;
+            }
+            __syncwarp();
+            const R* y = s_x[warp][K == 32 ? lane : (lane & (K - 1))];
+            bool in = true;
+#pragma unroll
+            for (int i = 0; i < D; ++i) {
+              const Key v = BoxKey<R>::of(y[i]);
+              in = in && !(v < lo[i] || v > hi[i]);
+            }
+            out = ~__ballot_sync(0xffffffffu, in) & window & ~skip;
+            skip |= out & (0u - out);
+          } while (out);
+          const unsigned in_mask = window & ~skip;
+          unsigned rej = 0;
+          if (in_mask) {
+            R xs[D];
+#pragma unroll
+            for (int i = 0; i < D; ++i) xs[i] = s_x[warp][k_own][i];
+            const StaticPoint<R, MODEL> pt(xs, l2f, n_quotes);
+            const C fo = virtual_lanes_sum<R>(pt, units, G, ls, sq, 0xffffffffu);
+            C* fb = s_f[cb][parity];
+            parity ^= 1;
+            if ((lane & (P - 1)) == 0) fb[k_own] = fo;
+            chain_sync<NW>(cb);
+            // lane k decides step k
+            const int k = lane & (K - 1);
+            const C f = fb[k];
+            const unsigned before = in_mask & ((1u << k) - 1u);  // the nearest earlier step inside the box
+            const C fe = fb[before ? 31 - __clz(before) : 0];
+            const C fp = before ? fe : fcur;
+            const auto delta = cost_delta(f, fp);
+            const R u = word_to(s_u[warp][(st + k) & (kRing - 1)], R{});
+            const bool acc = delta <= 0 || metropolis(u, delta, inv_Tk, Tk);
+            rej = __ballot_sync(0xffffffffu, !acc) & in_mask;
+            const int first = __ffs(rej) - 1;  // the first rejected step
+            const unsigned eval = rej ? in_mask & ((2u << first) - 1u) : in_mask;
+            const unsigned taken = rej ? eval & ~(1u << first) : eval;
+            ev += __popc(eval);
+            ac += __popc(taken);
+            unsigned better = __ballot_sync(0xffffffffu, cost_less(f, bf)) & eval;
+            if (better) {
+              int at = 0;
+              while (better) {
+                const int l = __ffs(better) - 1;
+                better &= better - 1u;
+                if (cost_less(fb[l], bf)) {
+                  bf = fb[l];
+                  at = l;
+                }
+              }
+#pragma unroll
+              for (int i = 0; i < D; ++i) bx[i] = s_x[warp][at][i];
+            }
+            if (taken) {
+              const int last = 31 - __clz(taken);
+              fcur = fb[last];
+#pragma unroll
+              for (int i = 0; i < D; ++i) x[i] = s_x[warp][last][i];
+            }
+            st += rej ? first + 1 : nv;
+          } else {
+            st += nv;
+          }
+          __syncwarp();  // the points are read before the next window's are written
+        }
+      }
+      if (!level_end(level, ev, ac, IntTag<0>{})) return;
+    }
+    // the chains' first warps run the levels step by step, and the level end hands
+    // their state to the others, until acceptance is the common outcome again
+    for (; level < n_levels && low; ++level) {
+      level_begin(level);
+      unsigned ev = 0, ac = 0;
+      if (active && wc == 0) {
+        ChainState<R> z;
+#pragma unroll
+        for (int i = 0; i < D; ++i) z.x[i] = x[i], z.bx[i] = bx[i];
+        z.fcur = fcur, z.bf = bf, z.ev = 0, z.ac = 0;
+        const int at = level & (kLevelCache - 1);
+        if constexpr (sizeof(R) == 8)
+          single_steps<R, MODEL>(Pr, gchain, level, s_step[at], s_invTk[at], s_Tk[at], s_w[warp], s_u[warp], z);
+        else
+          single_steps_call<R, MODEL>(Pr, gchain, level, s_step[at], s_invTk[at], s_Tk[at], s_w[warp], s_u[warp], z);
+#pragma unroll
+        for (int i = 0; i < D; ++i) x[i] = z.x[i], bx[i] = z.bx[i];
+        fcur = z.fcur, bf = z.bf, ev = z.ev, ac = z.ac;
+      }
+      if (!level_end(level, ev, ac, IntTag<1>{})) return;
+    }
   }
   if (n_levels > 0 && active && wc == 0 && lane == 0) {
     Pr.chain_bf[chain] = cost_to_double(bf);

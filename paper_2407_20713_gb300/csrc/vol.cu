@@ -10,9 +10,11 @@ namespace sabr {
 // Everything that does not depend on the option, formed once on the host: a
 // thread handles a few options only, and the FP64 pipe that the conversions,
 // log2 f and (in FP64) the formula's constants took on every thread issues 1.7
-// operations a clock and SM (2^20 options, FP32: Hagan 22.7 -> 14.5 us, expanded
-// 51.3 -> 11.4, Case I 54.0 -> 14.4, Case II 122 -> 94; 21 options in FP64, Hagan
-// 12.4 -> 8.3).
+// operations a clock and SM (2^20 options at any forward, FP32, us a launch in a
+// graph: Hagan 20.3 -> 10.9, Obloj 21.2 -> 16.5, expanded 50.3 -> 9.6, Case I 52.5 ->
+// 12.0, Case II 120 -> 93; FP64 Hagan 385 -> 333; 21 options in FP64, Hagan 12.4 ->
+// 8.3).  What is left on that pipe in FP32: three conversions to floats, the
+// product K f, and one back.
 template <class R> struct VolArgs {
   double p[kMaxD];
   double fwd;
@@ -64,16 +66,15 @@ __global__ void __launch_bounds__(256) implied_vol_kernel(const __grid_constant_
       sc = static_setup<R>(a.p);
     }
   }
-  const bool unit = a.fwd == 1.0;  // K f is then K
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
     const double kd = K[i];
     const R t = (R)T[i], k = (R)kd;
     const R lfk = m_log(a.f / k);
     R v;
     if constexpr (MODEL == SABR_HAGAN) {
-      v = vol_hagan<R>(sc, lfk, m_log2(unit ? k : (R)(kd * a.fwd)), t);
+      v = vol_hagan<R>(sc, lfk, m_log2((R)(kd * a.fwd)), t);
     } else if constexpr (MODEL == SABR_OBLOJ) {
-      v = vol_obloj<R>(sc, lfk, m_log2(unit ? k : (R)(kd * a.fwd)), m_log2(k), t);
+      v = vol_obloj<R>(sc, lfk, m_log2((R)(kd * a.fwd)), m_log2(k), t);
     } else if constexpr (MODEL == SABR_EXPANDED) {
       v = vol_poly<R>(expanded_coef<R>(a.p, a.l2f, t), lfk);
     } else {

@@ -88,14 +88,14 @@ __device__ __forceinline__ double m_sqrt(double x) { return sqrt(x); }
 // Hot-loop division and square root: in FP32 the SFU reciprocal / rsqrt
 // forms (about 2 ulp), in FP64 the IEEE operations.
 __device__ __forceinline__ float m_div(float a, float b) { return a * rcp_approx(b); }
-__device__ __forceinline__ double m_div(double a, double b) { return a / b; }
+__host__ __device__ __forceinline__ double m_div(double a, double b) { return a / b; }
 __device__ __forceinline__ float m_sqrt_pos(float x) { return x * rsqrt_approx(x); }  // x > 0
 __device__ __forceinline__ float m_rcp(float x) { return rcp_approx(x); }
 __device__ __forceinline__ double m_rcp(double x) { return 1.0 / x; }
 // Division by a constant: FP32 multiplies by the rounded reciprocal (one
 // extra rounding), FP64 divides as written.
 __device__ __forceinline__ float m_divc(float a, double c) { return a * (float)(1.0 / c); }
-__device__ __forceinline__ double m_divc(double a, double c) { return a / c; }
+__host__ __device__ __forceinline__ double m_divc(double a, double c) { return a / c; }
 __device__ __forceinline__ double m_sqrt_pos(double x) { return sqrt(x); }
 
 // ---------------------------------------------------------------------------
@@ -280,15 +280,18 @@ template <class R> struct ZxConst {
   R rho, omr, opr, q0;  // rho, 1 - rho, 1 + rho, (1 - rho)(1 + rho)
   R ln_opr, ln_omr;     // ln(1 + rho), ln(1 - rho) (FP32 form only)
 };
-// omr = 1 - rho and opr = 1 + rho are formed from the FP64 parameter.
-template <class R, class P> __device__ __forceinline__ ZxConst<R> zx_setup(P rho) {
+template <class R> __host__ __device__ __forceinline__ ZxConst<R> zx_plain(R rho, R omr, R opr) {
   ZxConst<R> c;
-  c.rho = (R)rho;
-  c.omr = (R)(1.0 - (double)rho);
-  c.opr = (R)(1.0 + (double)rho);
+  c.rho = rho;
+  c.omr = omr;
+  c.opr = opr;
   c.q0 = c.omr * c.opr;
   c.ln_opr = c.ln_omr = (R)0;
   return c;
+}
+// omr = 1 - rho and opr = 1 + rho are formed from the FP64 parameter.
+template <class R, class P> __device__ __forceinline__ ZxConst<R> zx_setup(P rho) {
+  return zx_plain<R>((R)rho, (R)(1.0 - (double)rho), (R)(1.0 + (double)rho));
 }
 
 // FP64 form: u is one division of selected operands.  Near z = 0, ln u alone
@@ -388,9 +391,11 @@ template <class R> struct StaticConst {
   ZxConst<R> zx;
 };
 
-// From alpha, beta, rho, nu in the working precision and the constants of rho.
+// From alpha, beta, rho, nu in the working precision and the constants of rho
+// (FP64 on the host too, for the volatility kernel's arguments).
+#pragma nv_exec_check_disable
 template <class R>
-__device__ __forceinline__ StaticConst<R> static_setup_from(R alpha, R beta, R rho, R nu, const ZxConst<R>& zx) {
+__host__ __device__ __forceinline__ StaticConst<R> static_setup_from(R alpha, R beta, R rho, R nu, const ZxConst<R>& zx) {
   StaticConst<R> s;
   s.alpha = alpha;
   s.beta = beta;

@@ -24,32 +24,6 @@ template <class R> struct VolArgs {
   StaticConst<R> sc;        // FP64 static formulas
 };
 
-// The formula's constants in FP64 (static_setup, on the host).
-static StaticConst<double> static_setup_host(const double* x) {
-  StaticConst<double> s;
-  s.alpha = x[0];
-  s.beta = x[1];
-  s.rho = x[2];
-  s.nu = x[3];
-  s.omb = 1.0 - s.beta;
-  s.half_omb = 0.5 * s.omb;
-  s.c2 = s.omb * s.omb / 24.0;
-  s.c4 = s.omb * s.omb * s.omb * s.omb / 1920.0;
-  s.nu_over_alpha = s.nu / s.alpha;
-  s.br_a = s.c2 * s.alpha * s.alpha;
-  s.br_b = 0.25 * s.rho * s.beta * s.nu * s.alpha;
-  s.br_c = (2.0 - 3.0 * s.rho * s.rho) / 24.0 * s.nu * s.nu;
-  s.abr_a = s.alpha * s.br_a;
-  s.abr_b = s.alpha * s.br_b;
-  s.abr_c = s.alpha * s.br_c;
-  s.zx.rho = s.rho;
-  s.zx.omr = 1.0 - s.rho;
-  s.zx.opr = 1.0 + s.rho;
-  s.zx.q0 = s.zx.omr * s.zx.opr;
-  s.zx.ln_opr = s.zx.ln_omr = 0.0;
-  return s;
-}
-
 template <class R, int MODEL>
 __global__ void __launch_bounds__(256) implied_vol_kernel(const __grid_constant__ VolArgs<R> a,
                                                           const double* __restrict__ T,
@@ -98,7 +72,9 @@ static void launch_vol(int model, const double* params, double fwd, const double
   a.nu = (R)a.p[3];
   a.omr = (R)(1.0 - a.p[2]);
   a.opr = (R)(1.0 + a.p[2]);
-  if constexpr (sizeof(R) == 8) a.sc = static_setup_host(a.p);
+  if constexpr (sizeof(R) == 8)
+    a.sc = static_setup_from<double>(a.p[0], a.p[1], a.p[2], a.p[3],
+                                     zx_plain<double>(a.p[2], 1.0 - a.p[2], 1.0 + a.p[2]));
   // one resident grid (eight blocks an SM), options strided over it
   const int blocks = (int)std::min<int64_t>((n + 255) / 256, (int64_t)device_sms() * 8);
   switch (model) {

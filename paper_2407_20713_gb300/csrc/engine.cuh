@@ -798,8 +798,10 @@ __device__ __forceinline__ DF dynamic_cost_f32(const float* xp, int n_quotes, in
                                                unsigned gmask) {
   constexpr int CS = CoefStride<float, MODEL>::value;
   if constexpr (MODEL == SABR_DYN_I) {
-    // three maturities a lane side by side while every lane has three (12
-    // maturities on four lanes), then one at a time
+    // three maturities a lane side by side while every lane has three (from 12
+    // maturities on, on four lanes), then one at a time: two side by side where
+    // every lane has two gains nothing (8192 chains on four lanes, 12 levels x 40,
+    // ms: 8 maturities 1.385 | 1.382, 11 1.600 | 1.639)
     int r0 = 0;
     for (; r0 + 3 * L <= n_mats; r0 += 3 * L) {
       PolyCoef<float> c[3];

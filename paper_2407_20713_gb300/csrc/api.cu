@@ -20,8 +20,6 @@ void set_error(const char* fmt, ...) {
 
 void clear_error() { g_error[0] = '\0'; }
 
-// SM count of the current device, queried once per device ordinal and
-// cached (the grid sizes of the kernels are multiples of it).
 cudaError_t allow_smem(const void* kernel, size_t bytes) {
   static std::mutex mu;
   static std::map<std::pair<int, const void*>, size_t> allowed;
@@ -37,6 +35,8 @@ cudaError_t allow_smem(const void* kernel, size_t bytes) {
   return e;
 }
 
+// SM count of the current device, queried once per device ordinal and
+// cached (the grid sizes of the kernels are multiples of it).
 int device_sms() {
   static std::atomic<int> cache[64];
   int dev = 0;

@@ -180,12 +180,8 @@ __host__ __device__ constexpr int coef_stride(int prec, int model) {
   return (model == SABR_DYN_II && prec == SABR_FP32) ? 16 : 4;
 }
 
-// The polynomial of maturity j from a coefficient slice: one 16-byte load
-// in FP32 (the slice is 16-byte aligned and its stride is 4), two in FP64.
-__device__ __forceinline__ PolyCoef<float> load_poly(const float* coef, int j) {
-  const float4 v = *reinterpret_cast<const float4*>(coef + 4 * j);
-  return PolyCoef<float>{v.x, v.y, v.z};
-}
+// The polynomial of maturity j from an FP64 coefficient slice (16-byte aligned, of
+// stride 4; FP32 reads its records in DynPoint).
 __device__ __forceinline__ PolyCoef<double> load_poly(const double* coef, int j) {
   const double2 v = *reinterpret_cast<const double2*>(coef + 4 * j);
   return PolyCoef<double>{v.x, v.y, coef[4 * j + 2]};
@@ -873,26 +869,29 @@ __device__ __forceinline__ typename CostOf<R>::T group_cost(const R* xp, int n_q
       acc += r * r;
     }
   } else {
-    if constexpr (sizeof(R) == 4) return dynamic_cost_f32<MODEL>(xp, n_quotes, n_mats, l2f, sq, coef, lane, G, G, gmask);
-    constexpr int CS = 4;  // polynomial slots per maturity (load_poly)
-    if (MODEL == SABR_DYN_I) {
-      for (int j = lane; j < n_mats; j += G) {
-        const PolyCoef<R> c = dynamic_coef<R, false>(xp, l2f, sq.mT[j]);
-        coef[CS * j + 0] = c.c0;
-        coef[CS * j + 1] = c.c1;
-        coef[CS * j + 2] = c.c2;
+    if constexpr (sizeof(R) == 4) {
+      return dynamic_cost_f32<MODEL>(xp, n_quotes, n_mats, l2f, sq, coef, lane, G, G, gmask);
+    } else {
+      constexpr int CS = 4;  // polynomial slots per maturity (load_poly)
+      if (MODEL == SABR_DYN_I) {
+        for (int j = lane; j < n_mats; j += G) {
+          const PolyCoef<R> c = dynamic_coef<R, false>(xp, l2f, sq.mT[j]);
+          coef[CS * j + 0] = c.c0;
+          coef[CS * j + 1] = c.c1;
+          coef[CS * j + 2] = c.c2;
+        }
+      } else {
+        case2_group_coef<R>(xp, n_mats, l2f, sq, coef, lane, G, gmask);
       }
-    } else if constexpr (sizeof(R) == 8) {
-      case2_group_coef<R>(xp, n_mats, l2f, sq, coef, lane, G, gmask);
+      __syncwarp(gmask);
+      for (int q = lane; q < n_quotes; q += G) {
+        const QuotePack<R> qp = sq.pack[q];
+        const PolyCoef<R> c = load_poly(coef, mat_of_slot(qp.l2kf));
+        const R r = resid(vol_poly<R>(c, qp.lfk), qp.w);
+        acc += r * r;
+      }
+      __syncwarp(gmask);
     }
-    __syncwarp(gmask);
-    for (int q = lane; q < n_quotes; q += G) {
-      const QuotePack<R> qp = sq.pack[q];
-      const PolyCoef<R> c = load_poly(coef, mat_of_slot(qp.l2kf));
-      const R r = resid(vol_poly<R>(c, qp.lfk), qp.w);
-      acc += r * r;
-    }
-    __syncwarp(gmask);
   }
   return lanes_sum(acc, G, gmask);
 }

@@ -426,9 +426,9 @@ int mc_blocks_per_set(const McHost& h, int n_sets) {
 
 // A launch of at most one block of kMcBlock threads per SM runs the FP32
 // log-Euler form with a pair of paths a thread: two warps a scheduler instead
-// of one (2^15 paths x 504 steps: 158 us a call against 168; from two blocks
-// an SM on, 2^17 paths, two pairs a thread are the faster form, 217 us
-// against 231).
+// of one (504 steps, us a call in a row, one pair a thread | two: 2^15 paths
+// 104.7 | 113.9, 2^16 105.3 | 115.2; from two blocks an SM on two pairs are the
+// faster form, 2^17 171 | 160, 2^18 308 | 292).
 static bool mc_split(const McHost& h, int64_t blocks) {
   return h.prec == SABR_FP32 && h.scheme == SABR_MC_LOG_EULER && blocks <= (int64_t)device_sms();
 }

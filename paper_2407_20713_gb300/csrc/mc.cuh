@@ -402,8 +402,9 @@ template <int PAIRS> struct PathPairs {
 // with one pair, the block before) takes its steps: Philox fills the FMA pipe
 // (a wide multiply holds it four cycles, a packed FP32x2 operation two) and
 // Box-Muller the SFU, and neither waits for the other.  What bounds the loop: a
-// path and step take about 47 cycles of a scheduler's FMA pipe (7.5 wide
-// multiplies 30, packed FP32 14) and 36 of its SFU; 60 are measured.  2^22 paths
+// path and step take about 45 cycles of a scheduler's FMA pipe (7.5 wide
+// multiplies 30, packed FP32 14, the step's key and drift 1) and 36 of its SFU; 60
+// are measured.  2^22 paths
 // x 504 steps: 4.17 ms with 20 multiplies a block and the words formed before
 // the steps, 3.87 with 15, 3.50 side by side.
 template <int PAIRS, int ORDER, class Land>

@@ -166,7 +166,7 @@ __device__ __noinline__ void single_steps_call(const ProblemDev& P, uint32_t gch
   single_steps<R, MODEL>(P, gchain, level, step4, inv_Tk, Tk, w, u, z);
 }
 
-// What bounds it (64 chains, 15 quotes, 4 warps x 4 points: 3.9 ms for 200
+// What bounds it (64 chains, 15 quotes, 4 warps x 4 points: 3.95 ms for 200
 // levels x 100 steps, 15.6 two steps at a time on 8 lanes): latency.  A level of
 // no steps takes 4 us (the meeting of 64 blocks), a window of 16 steps about
 // 1.2 us -- one dependent chain of proposals, formula, butterfly and decision on
@@ -480,15 +480,20 @@ bool small_supported(int prec, int model) {
   return model == SABR_HAGAN || model == SABR_OBLOJ || (model == SABR_EXPANDED && prec == SABR_FP64);
 }
 
-// FP32, ms per calibration on 152 SMs (level kernels and queue | shape chosen):
-//   64 chains, 15 quotes, 200 x 100: 15.6 | 4 warps x 4 points 3.95 (4 x 2 4.11, 2 x 4 4.16, 1 x 4 5.65)
-//   503 chains, 350 quotes, 28 x 97: 6.45 | 4 x 2 3.51 (4 x 4 4.98, 2 x 2 4.05, 1 x 2 5.85)
-//   1000 chains, 11 quotes, 50 x 50: 2.65 | 1 x 4 1.18 (1 x 2 1.52, 2 x 4 1.23)
-//   1024 chains, 200 quotes, 40 x 50: 3.21 | 1 x 4 2.16 (1 x 2 2.17, 2 x 4 2.38)
+// FP32, ms per calibration on 152 SMs (level kernels and queue | shapes, the
+// chosen one first):
+//   64 chains, 15 quotes, 200 x 100: 16.5 | 4 warps x 4 points 3.95, 4 x 2 4.21, 1 x 4 5.30
+//   152 chains, 64 quotes, 50 x 50: 2.96 | 4 x 4 0.97, 4 x 2 0.91, 1 x 4 1.26
+//   152 chains, 80 quotes, 50 x 50: 3.33 | 4 x 2 1.06, 4 x 4 1.23, 1 x 4 1.57
+//   503 chains, 350 quotes, 28 x 97: 4.73 | 4 x 2 2.29, 1 x 4 3.00
+//   600 chains, 21 quotes, 50 x 50: 3.25 | 4 x 2 1.28, 1 x 4 1.18
+//   1000 chains, 11 quotes, 50 x 50: 3.26 | 1 x 4 1.04
+//   1024 chains, 200 quotes, 40 x 50: 3.85 | 1 x 4 2.10
 // A point too deep costs evaluations that are dropped, so few quotes take the
 // deeper window.  FP64, whose time is FP64 instructions a scheduler: two
-// points a warp, as many warps a chain as give every scheduler one (64 chains,
-// 15 quotes, 200 x 100: 173.9 | 4 x 2 33.5; 4 x 4 40.1, 2 x 2 48.7, 1 x 2 80.2).
+// points a warp, as many warps a chain as give every scheduler one (15 quotes, 50
+// levels: 64 chains x 100 steps 47.6 | 4 x 2 8.56, 2 x 2 12.3, 1 x 2 19.9; 300 chains
+// x 50 25.9 | 2 x 2 7.35, 4 x 2 8.58, 1 x 2 10.9; 600 x 50 26.8 | 1 x 2 11.3, 2 x 2 12.2).
 SmallShape small_shape(int prec, int n_quotes, long long chains) {
   const long long sms = device_sms();
   if (prec == SABR_FP64) return SmallShape{chains <= sms ? 4 : (chains <= 2 * sms ? 2 : 1), 2};

@@ -424,13 +424,18 @@ int mc_blocks_per_set(const McHost& h, int n_sets) {
   return (int)best;
 }
 
-// A launch of at most one block of kMcBlock threads per SM runs the FP32
-// log-Euler form with a pair of paths a thread: two warps a scheduler instead
-// of one (504 steps, us a call in a row, one pair a thread | two: 2^15 paths
-// 104.7 | 113.9, 2^16 105.3 | 115.2; from two blocks an SM on two pairs are the
-// faster form, 2^17 171 | 160, 2^18 308 | 292).
+// A launch of at most one block of kMcBlock threads per SM and of many steps runs
+// the FP32 log-Euler form with a pair of paths a thread: two warps a scheduler
+// instead of one (504 steps, us a call in a row, one pair a thread | two: 2^15
+// paths 104.7 | 113.9, 2^16 105.3 | 115.2; from two blocks an SM on two pairs are
+// the faster form, 2^17 171 | 160, 2^18 308 | 292).  Its larger blocks and the
+// exchange at the maturities cost 1 to 2 us a launch, which the steps earn from
+// about 100 on (a Technique II calibration of 30 waves, us: 3 steps 1266 | 1202,
+// 50 2592 | 2592, 63 2799 | 2736, 100 4156 | 4158, 125 4600 | 4597, 250 8113 | 8175).
+constexpr int kSplitSteps = 128;
 static bool mc_split(const McHost& h, int64_t blocks) {
-  return h.prec == SABR_FP32 && h.scheme == SABR_MC_LOG_EULER && blocks <= (int64_t)device_sms();
+  return h.prec == SABR_FP32 && h.scheme == SABR_MC_LOG_EULER && h.n_steps >= kSplitSteps &&
+         blocks <= (int64_t)device_sms();
 }
 
 // Whether the blocks of a dynamic model's launch build their step tables

@@ -20,11 +20,12 @@ struct McSmem {
   size_t tab, land, q0, nq, slot, K, call, wacc, fx, total;
 };
 
-// FP32 log-Euler options are stored as signed strikes (mc.cuh: no call flag
-// is read); split: the block of 2 kMcBlock threads also needs the exchange
-// buffer of simulate_paths_f32<1>.
+// opt_bytes: an FP32 log-Euler option takes 8 or 4 (McOption, McSignedStrike; no
+// call flag is read); others the strike in the working precision.  split: the
+// block of 2 kMcBlock threads also needs the exchange buffer of
+// simulate_paths_f32<1>.
 template <class R>
-__host__ __device__ inline McSmem mc_smem_layout(int n_steps, int n_quotes, int n_mats, int n_slots, bool split) {
+__host__ __device__ inline McSmem mc_smem_layout(int n_steps, int n_quotes, int n_mats, int n_slots, int opt_bytes, bool split) {
   // (the conditional-Bessel form leaves its step table in global memory and
   // passes n_steps = 0)
   McSmem L;
@@ -36,7 +37,7 @@ __host__ __device__ inline McSmem mc_smem_layout(int n_steps, int n_quotes, int 
   };
   L.wacc = take(sizeof(double) * kMcWarps * n_slots * 32);
   L.tab = take(sizeof(StepCoef<R>) * n_steps);
-  L.K = take(sizeof(R) * n_quotes);
+  L.K = take((size_t)opt_bytes * n_quotes);
   L.land = take(sizeof(int) * n_mats);
   L.q0 = take(sizeof(int) * n_mats);
   L.nq = take(sizeof(int) * n_mats);
@@ -62,7 +63,7 @@ __host__ __device__ inline McSmem mc_smem_layout(int n_steps, int n_quotes, int 
 __host__ __device__ constexpr int mc_resident_blocks(int prec, int scheme) {
   return prec == SABR_FP64 ? 3 : (scheme == SABR_MC_BESSEL ? 5 : 4);
 }
-template <class R, int SCHEME, bool SPLIT>
+template <class R, int SCHEME, bool SPLIT, class Option>
 __global__ void __launch_bounds__((SPLIT ? 2 * kMcBlock : kMcBlock),
                                   (SPLIT ? 1 : mc_resident_blocks(sizeof(R) == 8 ? SABR_FP64 : SABR_FP32, SCHEME)))
     mc_paths_kernel(McDev P, const double* __restrict__ set_params, const int* __restrict__ set_valid,
@@ -72,11 +73,11 @@ __global__ void __launch_bounds__((SPLIT ? 2 * kMcBlock : kMcBlock),
   if (set_valid && !set_valid[set]) return;
   constexpr bool kPairs = sizeof(R) == 4 && SCHEME == SABR_MC_LOG_EULER;
   const McSmem L =
-      mc_smem_layout<R>(SCHEME == SABR_MC_BESSEL ? 0 : P.n_steps, P.n_quotes, P.n_mats, P.n_slots, SPLIT);
+      mc_smem_layout<R>(SCHEME == SABR_MC_BESSEL ? 0 : P.n_steps, P.n_quotes, P.n_mats, P.n_slots, sizeof(Option), SPLIT);
   double* wacc = (double*)(smem + L.wacc);
   StepCoef<R>* tab = (StepCoef<R>*)(smem + L.tab);
   R* sK = (R*)(smem + L.K);
-  float* sopt = (float*)(smem + L.K);
+  Option* sopt = (Option*)(smem + L.K);
   int* land = (int*)(smem + L.land);
   int* s_q0 = (int*)(smem + L.q0);
   int* s_nq = (int*)(smem + L.nq);
@@ -97,7 +98,7 @@ __global__ void __launch_bounds__((SPLIT ? 2 * kMcBlock : kMcBlock),
   }
   for (int q = threadIdx.x; q < P.n_quotes; q += blockDim.x) {
     if constexpr (kPairs) {
-      sopt[q] = signed_strike((float)P.K[q], P.is_call[q] != 0);
+      set_option(sopt[q], (float)P.K[q], P.is_call[q] != 0);
     } else {
       sK[q] = (R)P.K[q];
       scall[q] = P.is_call[q];
@@ -290,12 +291,13 @@ sabr_status mc_prepare(int model, double fwd, const double* T, const double* K, 
   h.n_steps = (int)h.step_t.size();
   if (h.n_steps > kMaxMcSteps) return fail(SABR_EINVAL, "more than 8192 time steps");
   h.Tmax = h.mats.back();
-  // what a block of the log-Euler kernel takes (the conditional-Bessel kernel
-  // keeps its step table in global memory; the same limit holds for it)
+  // what a block of the log-Euler kernel takes at its least (the
+  // conditional-Bessel kernel keeps its step table in global memory; the same
+  // limit holds for it)
   const int M = (int)h.mats.size();
   const size_t smem = prec == SABR_FP64
-                          ? mc_smem_layout<double>(h.n_steps, h.n_quotes, M, h.n_slots, false).total
-                          : mc_smem_layout<float>(h.n_steps, h.n_quotes, M, h.n_slots, false).total;
+                          ? mc_smem_layout<double>(h.n_steps, h.n_quotes, M, h.n_slots, 8, false).total
+                          : mc_smem_layout<float>(h.n_steps, h.n_quotes, M, h.n_slots, 4, false).total;
   if (smem > 220 * 1024) return fail(SABR_EINVAL, "too many time steps and options for one launch");
   h.smem = smem;
   return SABR_OK;
@@ -363,21 +365,44 @@ static_assert(sizeof(BesselStep<float>) == 48 && sizeof(BesselStep<double>) == 9
 
 using McPathsFn = void (*)(McDev, const double*, const int*, double*, int, int);
 
+// Resident blocks of kMcBlock threads per SM that grids count on, by the
+// registers and by a block's shared memory.
+static int mc_blocks_per_sm(int prec, int scheme, size_t smem) {
+  const size_t per_block = ((smem + 127) & ~(size_t)127) + 1024;
+  return (int)std::min<size_t>(mc_resident_blocks(prec, scheme), std::max<size_t>(1, (228 * 1024) / per_block));
+}
+
 // The path kernel of a problem's precision and scheme (split: the FP32
 // log-Euler form with a pair of paths a thread), with its dynamic shared
-// memory allowance raised to what the problem needs.
+// memory allowance raised to what the problem needs.  FP32 log-Euler options
+// take 8 bytes where that leaves as many blocks an SM as 4 (2^22 paths x 504
+// steps, 120 options: 3.499 ms, with 4 bytes 3.512), else 4 (512 options x 1200
+// steps, 600 000 paths: 1.34 ms on three blocks an SM, 1.37 where the grid counts
+// four and three fit).
 static McPathsFn mc_paths_fn(const McHost& h, bool split, size_t* smem) {
-  McPathsFn fn;
-  const int M = (int)h.mats.size(), S = h.scheme == SABR_MC_BESSEL ? 0 : h.n_steps;
+  const int M = (int)h.mats.size();
   if (h.prec == SABR_FP64) {
-    fn = h.scheme == SABR_MC_BESSEL ? mc_paths_kernel<double, SABR_MC_BESSEL, false>
-                                    : mc_paths_kernel<double, SABR_MC_LOG_EULER, false>;
-    *smem = mc_smem_layout<double>(S, h.n_quotes, M, h.n_slots, false).total;
-  } else {
-    fn = h.scheme == SABR_MC_BESSEL ? mc_paths_kernel<float, SABR_MC_BESSEL, false>
-                                    : (split ? mc_paths_kernel<float, SABR_MC_LOG_EULER, true>
-                                             : mc_paths_kernel<float, SABR_MC_LOG_EULER, false>);
-    *smem = mc_smem_layout<float>(S, h.n_quotes, M, h.n_slots, split).total;
+    const bool bessel = h.scheme == SABR_MC_BESSEL;
+    const McPathsFn fn = bessel ? mc_paths_kernel<double, SABR_MC_BESSEL, false, double>
+                                : mc_paths_kernel<double, SABR_MC_LOG_EULER, false, double>;
+    *smem = mc_smem_layout<double>(bessel ? 0 : h.n_steps, h.n_quotes, M, h.n_slots, 8, false).total;
+    allow_smem((const void*)fn, *smem);
+    return fn;
+  }
+  if (h.scheme == SABR_MC_BESSEL) {
+    const McPathsFn fn = mc_paths_kernel<float, SABR_MC_BESSEL, false, float>;
+    *smem = mc_smem_layout<float>(0, h.n_quotes, M, h.n_slots, 4, false).total;
+    allow_smem((const void*)fn, *smem);
+    return fn;
+  }
+  McPathsFn fn = mc_paths_kernel<float, SABR_MC_LOG_EULER, true, McOption>;
+  *smem = mc_smem_layout<float>(h.n_steps, h.n_quotes, M, h.n_slots, 8, split).total;
+  if (!split) {
+    fn = mc_paths_kernel<float, SABR_MC_LOG_EULER, false, McOption>;
+    if (mc_blocks_per_sm(h.prec, h.scheme, *smem) < mc_blocks_per_sm(h.prec, h.scheme, h.smem)) {
+      fn = mc_paths_kernel<float, SABR_MC_LOG_EULER, false, McSignedStrike>;
+      *smem = h.smem;
+    }
   }
   allow_smem((const void*)fn, *smem);
   return fn;
@@ -392,11 +417,7 @@ static int mc_thread_paths(const McHost& h) {
 // paths share a thread and a warp, hence the order of the FP32 payoff sums,
 // so it is a rule on the precision, the scheme and the table bytes and not
 // what a build's register count happens to allow.
-static int mc_grid_blocks_per_sm(const McHost& h) {
-  const int cap = mc_resident_blocks(h.prec, h.scheme);
-  const size_t per_block = ((h.smem + 127) & ~(size_t)127) + 1024;
-  return (int)std::min<size_t>(cap, std::max<size_t>(1, (228 * 1024) / per_block));
-}
+static int mc_grid_blocks_per_sm(const McHost& h) { return mc_blocks_per_sm(h.prec, h.scheme, h.smem); }
 
 // Blocks per parameter set.  Every block of a launch does the same work
 // (n_paths / blocks-per-set paths), so with R resident blocks a launch of

@@ -467,11 +467,22 @@ __device__ __forceinline__ void run_path_pairs(const McDev& P, const StepCoef<fl
 }
 
 // One option in shared memory, FP32: payoff (sgn F + c)^+ with sgn = 1,
-// c = -K for a call and sgn = -1, c = K for a put.  Only c is stored: its sign
-// bit (set for a call, at K = 0 too) gives sgn.
-__device__ __forceinline__ float signed_strike(float K, bool call) { return call ? -K : K; }
-__device__ __forceinline__ float forward_sign(float c) {
-  return __uint_as_float(0xBF800000u ^ (__float_as_uint(c) & 0x80000000u));
+// c = -K for a call and sgn = -1, c = K for a put: both (8 bytes), or c alone,
+// whose sign bit (set for a call, at K = 0 too) gives sgn for one more instruction
+// an option and maturity.
+struct McOption {
+  float sgn, c;
+};
+struct McSignedStrike {
+  float c;
+};
+__device__ __forceinline__ void set_option(McOption& o, float K, bool call) {
+  o = call ? McOption{1.0f, -K} : McOption{-1.0f, K};
+}
+__device__ __forceinline__ void set_option(McSignedStrike& o, float K, bool call) { o.c = call ? -K : K; }
+__device__ __forceinline__ float forward_sign(const McOption& o) { return o.sgn; }
+__device__ __forceinline__ float forward_sign(const McSignedStrike& o) {
+  return __uint_as_float(0xBF800000u ^ (__float_as_uint(o.c) & 0x80000000u));
 }
 
 // The FP32 path loop: four paths per virtual thread as two pairs
@@ -485,10 +496,10 @@ __device__ __forceinline__ float forward_sign(float c) {
 // them, by the maturity's parity, adds the payoffs of all four paths -- the
 // same FP32 sums in the same order as PAIRS = 2, so the prices are equal bit
 // for bit.
-template <int PAIRS>
+template <int PAIRS, class Option>
 __device__ __forceinline__ void simulate_paths_f32(const McDev& P, const double* p, const StepCoef<float>* tab,
                                                    const int* land, const int* s_q0, const int* s_nq,
-                                                   const int* s_slot, const float* opt, int64_t path0,
+                                                   const int* s_slot, const Option* opt, int64_t path0,
                                                    int64_t pstride, double* wacc, float* fx) {
   const int lane = threadIdx.x & 31;
   const int vt = threadIdx.x & (kMcBlock - 1), half = PAIRS == 1 ? threadIdx.x / kMcBlock : 0;
@@ -536,10 +547,11 @@ __device__ __forceinline__ void simulate_paths_f32(const McDev& P, const double*
             const int j = (c0 + kk) >> 1;
             float pay = 0.0f, pay2 = 0.0f;
             if (j < nq) {
-              const float c = opt[q0 + j], sgn = forward_sign(c);
+              const Option o = opt[q0 + j];
+              const float sgn = forward_sign(o);
 #pragma unroll
               for (int k = 0; k < NF; ++k) {
-                const float x = fmaxf(fmaf(sgn, F[k], c), 0.0f);
+                const float x = fmaxf(fmaf(sgn, F[k], o.c), 0.0f);
                 const float y = live[k] ? x : 0.0f;
                 pay += y;
                 pay2 = fmaf(y, y, pay2);

@@ -1,5 +1,5 @@
-"""Calls and puts of an FP32 pricing are kept as signed strikes, and the grid
-counts the blocks that fit with them: prices of mixed option sets, strikes of
+"""Calls and puts of an FP32 pricing are kept as pairs of a sign and a strike, or as
+signed strikes where pairs would cost a block an SM: prices of mixed option sets, strikes of
 zero among them, match the FP64 oracle on the same streams (1e-5, the pricer's
 FP32 tolerance; past 1800 steps by the square root of their number, as the
 per-step errors of the SFU functions, times sqrt(h), add up) at sizes where a
